@@ -57,7 +57,10 @@ struct alignas(16) Background {
   // Sums of the last flush (synchronised state), per field.
   double s_pi2[kMaxFields], s_phiD[kMaxFields], s_V;
   double mean[kMaxFields], var[kMaxFields];         // field mean and variance
-  double shift[kMaxFields];                         // unused (kept: checkpoint layout)
+  // FP64 persistent kernel: the high words of the largest |phi| and |pi| of field f
+  // over the lattice, as 0x80000000 | (hi & 0x7fffffff) in [2 f] and [2 f + 1];
+  // 0: not known (a state that another kernel, or the host, wrote)
+  uint32_t amax[2 * kMaxFields];
   // Split form: lattice-mean background and pending re-centring shifts.
   double phi0[kMaxFields], pi0[kMaxFields];
   double mu_phi[kMaxFields], mu_pi[kMaxFields];

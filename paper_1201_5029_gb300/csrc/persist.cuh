@@ -25,8 +25,9 @@
 // split-FP32 forms compute what the per-launch kernels compute, in a different
 // (fixed) summation order.
 //
-// FP64 form: a plane is drifted once into a shared-memory buffer (one block
-// barrier per plane), since FP64 arithmetic is the binding resource on GB300.
+// FP64 form: a plane is drifted once into a shared-memory buffer and its
+// stencil summed in 64-bit fixed point, since FP64 arithmetic is the binding
+// resource on GB300.
 // Split-FP32 form: barrier-free warp pipeline (each warp drifts the three rows
 // it needs in registers; "empty" mbarriers release slots; the producer role
 // rotates over the warps), since that form is bound by memory traffic.
@@ -84,25 +85,43 @@ struct PLayout {
 // a few planes behind; on GB300, 6 planes in flight with 3-4 slots of slack
 // beat both more planes with less slack and fewer planes with more (256^3:
 // 7/3 0.446, 6/4 0.428, 5/5 0.434 ms per step).
-//   FP64 extra: two drifted-plane buffers [NF][TY+2][TX] (one per plane parity)
-//               and the block-reduction scratch [NQ][threads].
+//   FP64 extra: NDRIFT drift buffers (see FixLayout) and the block-reduction
+//               scratch [NQ][threads].
 //   split extra: the compensated sums [NQ][threads / 4] float pairs, or every
 //               block's row of the stage sums (the fold reads them there),
 //               whichever is larger.
 // The FP64 and split-DD forms (bound by arithmetic: ALU) share the FP64 ring.
+//
+// FixLayout: one drift buffer of the FP64 form, 8-byte elements:
+//   fx[NF][TY + 2 H][TX + 4]  the drifted field for the stencil, 64-bit fixed
+//                             point (or float64: stages without a scale), each
+//                             row with its halo columns at x = -H .. TX + H - 1
+//                             (element 2 + x: 16-byte aligned at x = 0)
+//   ph[NF][TY][TX], pi[NF][TY][TX]  the drifted field and the momentum, float64
+template <int NF, int VX, int H>
+struct FixLayout {
+  static constexpr int TX = 32 * VX;
+  static constexpr int RS = TX + 4;
+  static constexpr int FXF = (kPTY + 2 * H) * RS;   // elements per field
+  static constexpr int OWNF = kPTY * TX;
+  static constexpr int PH = NF * FXF, PI = PH + NF * OWNF;
+  static constexpr int ELEMS = PI + NF * OWNF;
+};
+
 template <int PREC, int NF, int VX, int NQ, int H = 1>
 struct PRing {
   static constexpr bool ALU = PREC != PREC_SPLIT;
   using LY = PLayout<NF, VX, prec_word(PREC), H>;
   static constexpr int DRIFT_ELEMS = NF * (kPTY + 2 * H) * LY::TX;
-  // FP64 and split-DD: NDRIFT planes in flight, each the drifted phi rows
-  // (with the halo rows), the pi of the own rows (re-centred for split-DD) and
-  // the halo-column values (up to 3 rows per edge lane)
+  // NDRIFT planes in flight; split-DD: each the drifted phi rows (with the
+  // halo rows), the re-centred pi of the own rows and the halo-column values
+  // (up to 3 rows per edge lane); FP64: FixLayout
   static constexpr int NDRIFT = ALU ? 4 : 2;
   static constexpr int PI_ELEMS = NF * kPTY * LY::TX;
   static constexpr int COL_ELEMS = NF * kPTY * 2 * 3;
-  static constexpr int DRIFT_WORDS =
-      ALU ? NDRIFT * (DRIFT_ELEMS + PI_ELEMS + COL_ELEMS) : 2 * DRIFT_ELEMS;
+  static constexpr int DRIFT_WORDS = PREC == PREC_FP64 ? NDRIFT * FixLayout<NF, VX, H>::ELEMS
+                                     : ALU ? NDRIFT * (DRIFT_ELEMS + PI_ELEMS + COL_ELEMS)
+                                           : 2 * DRIFT_ELEMS;
   static constexpr int KAHAN_BYTES = NQ * kKahanGroups * 8;
   static constexpr int ROWS_BYTES = kMaxPBlocks * kNQ * 8;
   static constexpr int EXTRA_BYTES =
@@ -114,7 +133,8 @@ struct PRing {
                               : (NSLOT - kSplitSlack < kSplitLead ? NSLOT - kSplitSlack : kSplitLead);
   // warps that issue a stage's first LEAD planes at a stage boundary (the
   // others fold the block sums), each every PRE-th plane
-  static constexpr int PRE = LEAD < kPWarps - NQ ? LEAD : kPWarps - NQ;
+  static constexpr int FOLD = NQ + (PREC == PREC_FP64 ? 1 : 0);   // warps that fold rows
+  static constexpr int PRE = LEAD < kPWarps - FOLD ? LEAD : kPWarps - FOLD;
   static constexpr int RING_BYTES = NSLOT * LY::SLOT_BYTES;
   static constexpr int SMEM_BYTES = RING_BYTES + EXTRA_BYTES;
   static_assert(NSLOT >= 5 || ALU, "split ring too shallow");
@@ -345,15 +365,15 @@ __device__ __forceinline__ void lane_parts(const T (&ctr)[VX], const T (&dn)[VX]
   plane_parts<T, VX, CORNERS, MID>(ctr, dn, up, left, right, dl, dr, ul, ur, smid, so);
 }
 
-// FP64 and split-DD forms: drift of ring plane gg (of unit uu) into drift
-// buffer gg % NDRIFT, then this warp's arrival on the buffer's mbarrier.  Returns false if the plane's
+// Split-DD form: drift of ring plane gg (of unit uu) into drift buffer gg %
+// NDRIFT, then this warp's arrival on the buffer's mbarrier.  Returns false if the plane's
 // copies did not land within the limit (the buffer then holds garbage, which
 // the caller never uses: the stage fails).
-template <int MODEL, int STENCIL, int VX, int PREC>
-__device__ __forceinline__ bool drift_alu(const Ctx<MODEL, PREC>& cx, const PShared& sm,
-                                          uint32_t gg, int4 uu, int n) {
-  static_assert(PREC == PREC_FP64 || PREC == PREC_DD, "the FP64 and split-DD forms");
-  using T = typename std::conditional<PREC == PREC_DD, dd, double>::type;
+template <int MODEL, int STENCIL, int VX>
+__device__ __forceinline__ bool drift_dd(const Ctx<MODEL, PREC_DD>& cx, const PShared& sm,
+                                         uint32_t gg, int4 uu, int n) {
+  constexpr int PREC = PREC_DD;
+  using T = dd;
   constexpr int NF = Ctx<MODEL, PREC>::NF;
   constexpr int NQ = Ctx<MODEL, PREC>::SL::NQ;
   constexpr bool CORNERS = StencilW<STENCIL>::kCorners;
@@ -389,8 +409,7 @@ __device__ __forceinline__ bool drift_alu(const Ctx<MODEL, PREC>& cx, const PSha
     T q[VX];
 #pragma unroll
     for (int jj = 0; jj < VX; ++jj) {
-      if constexpr (PREC == PREC_DD) q[jj] = c[jj] - cx.mu_pi[f];   // re-centred
-      else q[jj] = c[jj];
+      q[jj] = c[jj] - cx.mu_pi[f];   // re-centred
       a[jj] = madd(cd, c[jj], a[jj]);
     }
     vstore<T, VX>(&dph[own], a);
@@ -439,24 +458,201 @@ __device__ __forceinline__ bool drift_alu(const Ctx<MODEL, PREC>& cx, const PSha
 
 // ---------------------------------------------------------------------------
 // FP64 form.
+//
+// GB300 executes two float64 lanes per SM and clock (a warp instruction takes
+// 64 cycles of a scheduler's pipe), and 64-bit conversions run at the same
+// rate, while integer adds, shifts and logic run 16 to 32 times faster.  The
+// discrete Laplacian is a sum with small integer weights, so it is taken off
+// the float64 pipe: each drifted field value is put on a 64-bit fixed-point
+// scale once (to_fixed, integer instructions only), D is summed exactly in
+// integers, and one normalisation (from_fixed, integer instructions) gives D
+// rounded once to float64.  The scale comes from the largest |phi| and |pi| of
+// the stage's input (Ctx::set_fix; the stages track them), so no sum can
+// overflow; a field value within 2^6 (27- and 13-point stencils: 2^2) of the
+// largest keeps every bit, and a smaller one is cut at 2^-58 (2^-54) of the
+// largest or less, below the rounding of the float64 sums it replaces.  A stage whose
+// input has no usable maximum (the first pass over a new state, values out of
+// range or not finite) sums in float64 (FIX = false).
+// Measured on GB300, against the same kernels with float64 stencils (set_initial,
+// evolve and get_fields together): 256^3 Q-ball, order 8, two steps 38.6 -> 25.2
+// ms; 256^3 oscillon, order 6, three steps 13.3 -> 8.9 ms; 128^3 preheating,
+// order 4, ten steps 4.49 -> 2.83 ms, with the 13-point stencil 6.78 -> 3.40 ms.
 // ---------------------------------------------------------------------------
-// One stage of the FP64 form over this block's units.  The planes flow
-// through the drift buffers as in the split-DD form (below): each warp drifts
-// plane g + 1 (drift_alu), then waits until every warp has drifted plane g and
-// computes it, with no block barrier in the z loop; the halo rows and the copy
-// issue rotate over the warps.  Returns false if a wait gave up (the caller
-// combines the threads' results).  gq: ring planes consumed before this stage.
-template <int MODEL, int STENCIL, int VX, int MODE>
-__device__ __forceinline__ bool stage_fp64(const PParams& p, const Ctx<MODEL, PREC_FP64>& cx,
-                                           const PShared& sm, uint32_t gq, int ib, double* accd) {
+// bits of |D| above the largest |I|: sum of the absolute weights, 12 (7-point),
+// 256 (27-point, weights times 30), 192 (13-point, times 12)
+template <int STENCIL> constexpr int fix_headroom() { return STENCIL == 7 ? 4 : 8; }
+// what the integer sums are times D
+template <int STENCIL> constexpr double fix_weight() {
+  return STENCIL == 7 ? 1.0 : (STENCIL == 27 ? 30.0 : 12.0);
+}
+
+// trunc(v 2^(1086 - E)) for |v| < 2^(E - 1023): the significand, bit 63 down,
+// shifted right by E - e (shr clamps: values below the scale, and zero, give 0).
+__device__ __forceinline__ unsigned long long to_fixed(double v, int E) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int hi = __double2hiint(v);
+  const int sh = E - ((hi >> 20) & 0x7ff);
+  unsigned long long m = (b << 11) | 0x8000000000000000ull;
+  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));
+  return hi < 0 ? 0ull - m : m;
+}
+// x 2^(E - 1086), rounded to nearest (a tie away from zero)
+__device__ __forceinline__ double from_fixed(unsigned long long x, int E) {
+  const bool neg = (long long)x < 0;
+  unsigned long long m = neg ? 0ull - x : x;
+  const int lz = __clzll((long long)m);
+  asm("shl.b64 %0, %0, %1;" : "+l"(m) : "r"(lz));
+  unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);
+  r += (unsigned long long)(uint32_t)(E - lz - 1) << 52;
+  r |= neg ? 0x8000000000000000ull : 0ull;
+  return __longlong_as_double((long long)(m == 0ull ? 0ull : r));
+}
+
+template <bool FIX> struct FixElem { using type = double; };
+template <> struct FixElem<true> { using type = unsigned long long; };
+__device__ __forceinline__ double fix_in(double v, int, double*) { return v; }
+__device__ __forceinline__ unsigned long long fix_in(double v, int E, unsigned long long*) {
+  return to_fixed(v, E);
+}
+__device__ __forceinline__ double fix_out(double v, int) { return v; }
+__device__ __forceinline__ double fix_out(unsigned long long v, int E) { return from_fixed(v, E); }
+
+__device__ __forceinline__ double fix_mad(double a, double b, double c) { return madd(a, b, c); }
+__device__ __forceinline__ unsigned long long fix_mad(unsigned long long a, unsigned long long b,
+                                                      unsigned long long c) {
+  return a * b + c;
+}
+// In-plane parts of the stencil (Eq. D split by z-offset, as plane_parts):
+// float64 with the weights themselves, integers with the weights times 30
+// (27-point) or as they are (7-point).
+__device__ __forceinline__ double fix_mid7(double c, double faces) { return madd(-6.0, c, faces); }
+__device__ __forceinline__ unsigned long long fix_mid7(unsigned long long c,
+                                                       unsigned long long faces) {
+  return faces - 6ull * c;
+}
+__device__ __forceinline__ void fix_parts27(double c, double faces, double corners, double& mid,
+                                            double& off) {
+  mid = madd(3.0 / 30.0, corners, madd(14.0 / 30.0, faces, (-128.0 / 30.0) * c));
+  off = madd(1.0 / 30.0, corners, madd(3.0 / 30.0, faces, (14.0 / 30.0) * c));
+}
+__device__ __forceinline__ void fix_parts27(unsigned long long c, unsigned long long faces,
+                                            unsigned long long corners, unsigned long long& mid,
+                                            unsigned long long& off) {
+  mid = 14ull * faces + 3ull * corners - (c << 7);
+  off = 14ull * c + 3ull * faces + corners;
+}
+
+// High words of the largest magnitudes a thread has put out, per field (phi, pi).
+template <int NF> struct HiMax {
+  uint32_t v[2 * NF];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < 2 * NF; ++i) v[i] = 0u;
+  }
+  __device__ __forceinline__ void add(int i, double x) {
+    v[i] = max(v[i], (uint32_t)__double2hiint(x) & 0x7fffffffu);
+  }
+};
+
+// Drift of ring plane gg (of unit uu) into drift buffer gg % NDRIFT, then this
+// warp's arrival on the buffer's mbarrier (see drift_dd).
+template <int MODEL, int STENCIL, int VX, bool FIX>
+__device__ __forceinline__ bool drift_fp64(const Ctx<MODEL, PREC_FP64>& cx, const PShared& sm,
+                                           uint32_t gg, int4 uu, int n) {
+  using E = typename FixElem<FIX>::type;
+  constexpr int NF = Ctx<MODEL, PREC_FP64>::NF;
+  constexpr int NQ = Ctx<MODEL, PREC_FP64>::SL::NQ;
+  constexpr bool CORNERS = StencilW<STENCIL>::kCorners;
+  constexpr int H = halo_of<STENCIL>();
+  using LY = PLayout<NF, VX, 8, H>;
+  using RG = PRing<PREC_FP64, NF, VX, NQ, H>;
+  using FL = FixLayout<NF, VX, H>;
+  constexpr int TX = LY::TX, CW = LY::CW, NSLOT = RG::NSLOT, NB = RG::NDRIFT;
+  const int tid = threadIdx.x, lane = tid & 31, ly = tid >> 5;
+  const int side = lane == 31 ? 1 : 0;
+  const bool edge = lane == 0 || lane == 31;
+  const int own = (ly + H) * TX + lane * VX;
+  const int s = gg % NSLOT, b = gg % NB;
+  // the 2H halo rows of this plane go to warps 2H j .. 2H j + 2H - 1, j = gg mod (16 / 2H)
+  const int hw = (ly - 2 * H * (int)(gg % (kPWarps / (2 * H))) + kPWarps) % kPWarps;
+  const int hrow = hw < H ? hw : kPTY + hw;
+  const bool ok = mbar_wait(&sm.full[s], (gg / NSLOT) & 1, sm.limit);
+  const double* sl = (const double*)(sm.ring + (size_t)s * LY::SLOT_BYTES);
+  double* buf = sm.drift + (size_t)b * FL::ELEMS;
+  const double cd = cx.cdrift;
+  const bool clear = yclear(uu, n);
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    const double* mph = sl + LY::main_off(0, f);
+    const double* mpi = sl + LY::main_off(1, f);
+    E* fx = reinterpret_cast<E*>(buf) + f * FL::FXF + 2;
+    const int ex = cx.fx[f];
+    double a[VX], c[VX];
+    E q[VX];
+    vload<double, VX>(&mph[own], a);
+    vload<double, VX>(&mpi[own], c);
+#pragma unroll
+    for (int jj = 0; jj < VX; ++jj) {
+      a[jj] = madd(cd, c[jj], a[jj]);
+      q[jj] = fix_in(a[jj], ex, (E*)nullptr);
+    }
+    const int o = f * FL::OWNF + ly * TX + lane * VX;
+    vstore<double, VX>(buf + FL::PH + o, a);
+    vstore<double, VX>(buf + FL::PI + o, c);
+    vstore<E, VX>(fx + (ly + H) * FL::RS + lane * VX, q);
+    if (hw < 2 * H) {   // the halo rows rotate over the warps, plane by plane
+      const int r = hrow * TX + lane * VX;
+      vload<double, VX>(&mph[r], a);
+      vload<double, VX>(&mpi[r], c);
+#pragma unroll
+      for (int jj = 0; jj < VX; ++jj) q[jj] = fix_in(madd(cd, c[jj], a[jj]), ex, (E*)nullptr);
+      vstore<E, VX>(fx + hrow * FL::RS + lane * VX, q);
+    }
+    if (edge) {
+      // the H halo columns of this side (k = 0 adjacent), this warp's row and,
+      // 27-point stencil, the corner cells of a halo row
+#pragma unroll
+      for (int k = 0; k < H; ++k) {
+        const int cc = side ? k : CW - 1 - k;
+        const double* cph = sl + LY::col_base(0, side) + cc;
+        const double* cpi = sl + LY::col_base(1, side) + cc;
+        const int x = side ? TX + k : -1 - k;
+        const int row = clear ? LY::col_dense(f, ly + 1) : LY::col_wrap(f, ly + 1);
+        fx[(ly + H) * FL::RS + x] = fix_in(madd(cd, cpi[row], cph[row]), ex, (E*)nullptr);
+        if (CORNERS && hw < 2) {
+          const int cr = clear ? LY::col_dense(f, hrow) : LY::col_wrap(f, hrow);
+          fx[hrow * FL::RS + x] = fix_in(madd(cd, cpi[cr], cph[cr]), ex, (E*)nullptr);
+        }
+      }
+    }
+  }
+  // generic reads of the ring slot before the TMA copy that refills it (drift_dd)
+  fence_proxy_async();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&sm.dbar[b]);
+  return ok;
+}
+
+// One stage of the FP64 form over this block's units, 7- and 27-point
+// stencils.  The planes flow through the drift buffers as in the split-DD form
+// (below): each warp drifts plane g + 1 (drift_fp64), then waits until every
+// warp has drifted plane g and computes it, with no block barrier in the z
+// loop; the halo rows and the copy issue rotate over the warps.  Returns false
+// if a wait gave up (the caller combines the threads' results).  gq: ring
+// planes consumed before this stage.
+template <int MODEL, int STENCIL, int VX, int MODE, bool FIX>
+__device__ __forceinline__ bool stage_fp64(const PParams& p, const Ctx<MODEL, PREC_FP64>& cx0,
+                                           const PShared& sm, uint32_t gq, int ib, double* accd,
+                                           HiMax<Pot<MODEL>::NF>& hm) {
   using C = Ctx<MODEL, PREC_FP64>;
   using T = double;
+  using E = typename FixElem<FIX>::type;
   using SL = typename C::SL;
   constexpr int NF = C::NF;
   constexpr bool CORNERS = StencilW<STENCIL>::kCorners;
-  constexpr int CR = CORNERS ? 3 : 1;
   using LY = PLayout<NF, VX, 8>;
   using RG = PRing<PREC_FP64, NF, VX, SL::NQ>;
+  using FL = FixLayout<NF, VX, 1>;
   constexpr int TX = LY::TX;
   constexpr int NSLOT = RG::NSLOT, LEAD = RG::LEAD, NB = RG::NDRIFT;
   static_assert(LEAD + 1 == NSLOT, "the stage issues plane gq + LEAD, then g + NSLOT at plane g");
@@ -466,10 +662,12 @@ __device__ __forceinline__ bool stage_fp64(const PParams& p, const Ctx<MODEL, PR
   const size_t S = (size_t)d.S, nn = (size_t)n * n;
   T* __restrict__ phi_out = (T*)d.phi[(ib & 1) ^ 1];
   T* __restrict__ pi_out = (T*)d.pi[((ib >> 1) & 1) ^ 1];
-  const int side = lane == 31 ? 1 : 0;
-  const bool edge = lane == 0 || lane == 31;
-  const int own = (ly + 1) * TX + lane * VX;          // this lane's sites in a slot row
+  const int own = (ly + 1) * FL::RS + 2 + lane * VX;
   bool ok = true;
+  // the integer sums are D times the stencil's common denominator: it goes into
+  // the kick's coefficient and, after the stage, into sum phi D
+  C cx = cx0;
+  if constexpr (FIX && STENCIL == 27) cx.kD *= 1.0 / fix_weight<STENCIL>();
 
   // producer position (see stage_dd): plane gq + LEAD now, plane g + NSLOT at plane g
   int pui = 0, puq = 0;
@@ -484,22 +682,22 @@ __device__ __forceinline__ bool stage_fp64(const PParams& p, const Ctx<MODEL, PR
   padvance(sm, pui, puq);
 
   uint32_t g = gq;
-  if (sm.nunits > 0) ok = drift_alu<MODEL, STENCIL, VX, PREC_FP64>(cx, sm, g, sm.units[0], n);
+  if (sm.nunits > 0) ok = drift_fp64<MODEL, STENCIL, VX, FIX>(cx, sm, g, sm.units[0], n);
   for (int i = 0; i < sm.nunits && ok; ++i) {
     const int4 u = sm.units[i];
     const int Q = u.w;
     const size_t o0 = (size_t)u.z * nn + (size_t)(u.y + ly) * n + u.x + lane * VX;
-    T part_m[NF][VX], so_m[NF][VX], ph_m[NF][VX], pi_m[NF][VX];
+    E part_m[NF][VX], so_m[NF][VX];
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
-      for (int jj = 0; jj < VX; ++jj) part_m[f][jj] = so_m[f][jj] = ph_m[f][jj] = pi_m[f][jj] = 0.0;
+      for (int jj = 0; jj < VX; ++jj) part_m[f][jj] = so_m[f][jj] = (E)0;
     for (int q = 0; q < Q; ++q, ++g) {
       // look ahead: drift the stage's next plane
       if (q + 1 < Q)
-        ok = drift_alu<MODEL, STENCIL, VX, PREC_FP64>(cx, sm, g + 1, u, n) && ok;
+        ok = drift_fp64<MODEL, STENCIL, VX, FIX>(cx, sm, g + 1, u, n) && ok;
       else if (i + 1 < sm.nunits)
-        ok = drift_alu<MODEL, STENCIL, VX, PREC_FP64>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
+        ok = drift_fp64<MODEL, STENCIL, VX, FIX>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
       // every warp has drifted plane g
       ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit) && ok;
       if (!ok) break;
@@ -512,49 +710,70 @@ __device__ __forceinline__ bool stage_fp64(const PParams& p, const Ctx<MODEL, PR
       }
       padvance(sm, pui, puq);
 
-      const int b = g % NB;
-      const T* dp = sm.drift + (size_t)b * RG::DRIFT_ELEMS;
-      const T* pp = sm.drift + (size_t)NB * RG::DRIFT_ELEMS + (size_t)b * RG::PI_ELEMS;
-      const T* cp = sm.drift + (size_t)NB * (RG::DRIFT_ELEMS + RG::PI_ELEMS) +
-                    (size_t)b * RG::COL_ELEMS;
-      T cur_ph[NF][VX], cur_pi[NF][VX], el[NF][CR];
+      const double* buf = sm.drift + (size_t)(g % NB) * FL::ELEMS;
       const bool mid = q > 0 && q < Q - 1;   // the z-halo planes need S_off only
-      T so_new[NF][VX], smid_new[NF][VX];
+      E so_new[NF][VX], smid_new[NF][VX];
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
-        const T* dph = dp + f * (kPTY + 2) * TX;
-        vload<T, VX>(&dph[own], cur_ph[f]);
-        vload<T, VX>(&pp[(f * kPTY + ly) * TX + lane * VX], cur_pi[f]);
+        const E* fx = reinterpret_cast<const E*>(buf) + f * FL::FXF + own;
+        E ctr[VX];
+        vload<E, VX>(fx, ctr);
 #pragma unroll
-        for (int rr = 0; rr < CR; ++rr)
-          el[f][rr] = edge ? cp[((f * kPTY + ly) * 2 + side) * 3 + rr] : 0.0;
-        T dn[VX], up[VX];
+        for (int jj = 0; jj < VX; ++jj) smid_new[f][jj] = so_new[f][jj] = ctr[jj];
+        if (CORNERS || mid) {
+          E dn[VX], up[VX];
+          vload<E, VX>(fx - FL::RS, dn);
+          vload<E, VX>(fx + FL::RS, up);
+          const E left = fx[-1], right = fx[VX];
+          E dl{}, dr{}, ul{}, ur{};
+          if constexpr (CORNERS) {
+            dl = fx[-FL::RS - 1]; dr = fx[-FL::RS + VX];
+            ul = fx[FL::RS - 1]; ur = fx[FL::RS + VX];
+          }
 #pragma unroll
-        for (int jj = 0; jj < VX; ++jj) dn[jj] = up[jj] = 0.0;
-        if (mid || CORNERS) {
-          vload<T, VX>(&dph[own - TX], dn);
-          vload<T, VX>(&dph[own + TX], up);
+          for (int jj = 0; jj < VX; ++jj) {
+            const E L = jj > 0 ? ctr[jj > 0 ? jj - 1 : 0] : left;
+            const E R = jj < VX - 1 ? ctr[jj < VX - 1 ? jj + 1 : 0] : right;
+            const E faces = (dn[jj] + up[jj]) + (L + R);
+            if constexpr (CORNERS) {
+              const E DL = jj > 0 ? dn[jj > 0 ? jj - 1 : 0] : dl;
+              const E DR = jj < VX - 1 ? dn[jj < VX - 1 ? jj + 1 : 0] : dr;
+              const E UL = jj > 0 ? up[jj > 0 ? jj - 1 : 0] : ul;
+              const E UR = jj < VX - 1 ? up[jj < VX - 1 ? jj + 1 : 0] : ur;
+              fix_parts27(ctr[jj], faces, (DL + DR) + (UL + UR), smid_new[f][jj], so_new[f][jj]);
+            } else {
+              smid_new[f][jj] = fix_mid7(ctr[jj], faces);
+            }
+          }
         }
-        if (mid)
-          lane_parts<T, VX, CORNERS, true, CR>(cur_ph[f], dn, up, el[f], smid_new[f], so_new[f]);
-        else
-          lane_parts<T, VX, CORNERS, false, CR>(cur_ph[f], dn, up, el[f], smid_new[f], so_new[f]);
       }
       if (q >= 2) {  // output plane z0 + q - 2
         const size_t o = o0 + (size_t)(q - 2) * nn;
-        T pin[NF][VX];
+        // its drifted field and momentum: this warp's own row of the buffer
+        // before, which only this warp writes
+        const double* pbuf = sm.drift + (size_t)((g - 1) % NB) * FL::ELEMS + ly * TX + lane * VX;
+        T ph_m[NF][VX], pi_m[NF][VX], pin[NF][VX];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          vload<T, VX>(pbuf + FL::PH + f * FL::OWNF, ph_m[f]);
+          vload<T, VX>(pbuf + FL::PI + f * FL::OWNF, pi_m[f]);
+        }
 #pragma unroll
         for (int jj = 0; jj < VX; ++jj) {
           T phj[NF], Dj[NF], pmj[NF], pnj[NF];
 #pragma unroll
           for (int f = 0; f < NF; ++f) {
             phj[f] = ph_m[f][jj];
-            Dj[f] = part_m[f][jj] + so_new[f][jj];
+            Dj[f] = fix_out(part_m[f][jj] + so_new[f][jj], cx.fx[f]);
             pmj[f] = pi_m[f][jj];
           }
           cx.site(MODE, phj, Dj, pmj, pnj, accd);
 #pragma unroll
-          for (int f = 0; f < NF; ++f) pin[f][jj] = pnj[f];
+          for (int f = 0; f < NF; ++f) {
+            pin[f][jj] = pnj[f];
+            hm.add(2 * f, phj[f]);
+            hm.add(2 * f + 1, pnj[f]);
+          }
         }
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
@@ -562,22 +781,20 @@ __device__ __forceinline__ bool stage_fp64(const PParams& p, const Ctx<MODEL, PR
           if (MODE == MODE_SWEEP) gstore<T, VX>(pi_out + f * S + o, pin[f]);
         }
       }
-      if (mid) {
 #pragma unroll
-        for (int f = 0; f < NF; ++f)
+      for (int f = 0; f < NF; ++f) {
+        if (mid) {
 #pragma unroll
-          for (int jj = 0; jj < VX; ++jj)
-            part_m[f][jj] = (CORNERS ? so_m[f][jj] : ph_m[f][jj]) + smid_new[f][jj];
-      }
-#pragma unroll
-      for (int f = 0; f < NF; ++f)
-#pragma unroll
-        for (int jj = 0; jj < VX; ++jj) {
-          if constexpr (CORNERS) so_m[f][jj] = so_new[f][jj];
-          ph_m[f][jj] = cur_ph[f][jj];
-          pi_m[f][jj] = cur_pi[f][jj];
+          for (int jj = 0; jj < VX; ++jj) part_m[f][jj] = so_m[f][jj] + smid_new[f][jj];
         }
+#pragma unroll
+        for (int jj = 0; jj < VX; ++jj) so_m[f][jj] = so_new[f][jj];
+      }
     }
+  }
+  if constexpr (FIX && STENCIL == 27) {
+#pragma unroll
+    for (int f = 0; f < NF; ++f) accd[SL::PHID + f] *= 1.0 / fix_weight<STENCIL>();
   }
   return ok;
 }
@@ -665,7 +882,7 @@ __device__ __forceinline__ bool stage_dd(const PParams& p, const Ctx<MODEL, PREC
   padvance(sm, pui, puq);
 
   uint32_t g = gq;
-  if (sm.nunits > 0) ok = drift_alu<MODEL, STENCIL, VX, PREC_DD>(cx, sm, g, sm.units[0], n);
+  if (sm.nunits > 0) ok = drift_dd<MODEL, STENCIL, VX>(cx, sm, g, sm.units[0], n);
   for (int i = 0; i < sm.nunits && ok; ++i) {
     const int4 u = sm.units[i];
     const int Q = u.w;
@@ -679,9 +896,9 @@ __device__ __forceinline__ bool stage_dd(const PParams& p, const Ctx<MODEL, PREC
     for (int q = 0; q < Q; ++q, ++g) {
       // look ahead: drift the stage's next plane
       if (q + 1 < Q)
-        ok = drift_alu<MODEL, STENCIL, VX, PREC_DD>(cx, sm, g + 1, u, n) && ok;
+        ok = drift_dd<MODEL, STENCIL, VX>(cx, sm, g + 1, u, n) && ok;
       else if (i + 1 < sm.nunits)
-        ok = drift_alu<MODEL, STENCIL, VX, PREC_DD>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
+        ok = drift_dd<MODEL, STENCIL, VX>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
       // every warp has drifted plane g
       ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit) && ok;
       if (!ok) break;
@@ -814,11 +1031,12 @@ __device__ __forceinline__ void wide_shuffles(const T (&ctr)[VX], T (&e)[VX + 4]
   }
 }
 
-template <int MODEL, int VX, int MODE, int PREC>
-__device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PREC>& cx,
-                                           const PShared& sm, uint32_t gq, int ib, double* accd) {
+template <int MODEL, int VX, int MODE>
+__device__ __forceinline__ bool stage_wide_dd(const PParams& p, const Ctx<MODEL, PREC_DD>& cx,
+                                              const PShared& sm, uint32_t gq, int ib) {
+  constexpr int PREC = PREC_DD;
   using C = Ctx<MODEL, PREC>;
-  using T = typename std::conditional<PREC == PREC_DD, dd, double>::type;
+  using T = dd;
   using SL = typename C::SL;
   constexpr int NF = C::NF;
   constexpr int NQ = SL::NQ;
@@ -827,7 +1045,7 @@ __device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PR
   using RG = PRing<PREC, NF, VX, NQ, H>;
   constexpr int TX = LY::TX;
   constexpr int NSLOT = RG::NSLOT, LEAD = RG::LEAD, NB = RG::NDRIFT;
-  constexpr int KGROUP = 8;   // split-DD: output planes per running accumulator
+  constexpr int KGROUP = 8;   // output planes per running accumulator
   static_assert(LEAD + 1 == NSLOT, "the stage issues plane gq + LEAD, then g + NSLOT at plane g");
   const SimDesc& d = *sm.d;
   const int tid = threadIdx.x, lane = tid & 31, ly = tid >> 5;
@@ -836,25 +1054,18 @@ __device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PR
   T* __restrict__ phi_out = (T*)d.phi[(ib & 1) ^ 1];
   T* __restrict__ pi_out = (T*)d.pi[((ib >> 1) & 1) ^ 1];
   const int own = (ly + H) * TX + lane * VX;
-  // weights: FP64 the stencil's own; split-DD 12 x them, then 1/12 at the end
-  const T w1 = PREC == PREC_DD ? T(16.0) : T(16.0 / 12.0);
-  const T w2 = PREC == PREC_DD ? T(-1.0) : T(-1.0 / 12.0);
-  const T w0 = PREC == PREC_DD ? T(-90.0) : T(-90.0 / 12.0);
+  // 12 x the stencil's weights, then 1/12 at the end
+  const T w1 = T(16.0), w2 = T(-1.0), w0 = T(-90.0);
   const T inv12 = T(1.0 / 12.0);
-  T Mf[NF];   // split-DD: the re-centring of the drifted field
+  T Mf[NF];   // the re-centring of the drifted field
 #pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    if constexpr (PREC == PREC_DD) Mf[f] = dd_fma(cx.cdrift, cx.mu_pi[f], cx.mu_phi[f]);
-    else Mf[f] = 0.0;
-  }
-  DDAcc acc[PREC == PREC_DD ? NQ : 1];
-  dd* tot = reinterpret_cast<dd*>(sm.red) + tid;   // split-DD stage sums, tot[q * kPThreads]
-  if constexpr (PREC == PREC_DD) {
+  for (int f = 0; f < NF; ++f) Mf[f] = dd_fma(cx.cdrift, cx.mu_pi[f], cx.mu_phi[f]);
+  DDAcc acc[NQ];
+  dd* tot = reinterpret_cast<dd*>(sm.red) + tid;   // stage sums, tot[q * kPThreads]
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-      acc[i].zero();
-      tot[i * kPThreads] = dd(0.f, 0.f);
-    }
+  for (int i = 0; i < NQ; ++i) {
+    acc[i].zero();
+    tot[i * kPThreads] = dd(0.f, 0.f);
   }
   int kg = 0;
   bool ok = true;
@@ -871,7 +1082,7 @@ __device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PR
   padvance(sm, pui, puq);
 
   uint32_t g = gq;
-  if (sm.nunits > 0) ok = drift_alu<MODEL, 13, VX, PREC>(cx, sm, g, sm.units[0], n);
+  if (sm.nunits > 0) ok = drift_dd<MODEL, 13, VX>(cx, sm, g, sm.units[0], n);
   for (int i = 0; i < sm.nunits && ok; ++i) {
     const int4 u = sm.units[i];
     const int Q = u.w;
@@ -885,9 +1096,9 @@ __device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PR
         P1[f][jj] = P2[f][jj] = c1[f][jj] = c2[f][jj] = q1[f][jj] = q2[f][jj] = T(0.0);
     for (int q = 0; q < Q; ++q, ++g) {
       if (q + 1 < Q)
-        ok = drift_alu<MODEL, 13, VX, PREC>(cx, sm, g + 1, u, n) && ok;
+        ok = drift_dd<MODEL, 13, VX>(cx, sm, g + 1, u, n) && ok;
       else if (i + 1 < sm.nunits)
-        ok = drift_alu<MODEL, 13, VX, PREC>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
+        ok = drift_dd<MODEL, 13, VX>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
       ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit) && ok;
       if (!ok) break;
       if (tid == 32 * (int)((4 * ((g + 1) % (kPWarps / 4)) + 4) % kPWarps) && pui < sm.nunits) {
@@ -954,18 +1165,12 @@ __device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PR
           T phj[NF], Dj[NF], pmj[NF], pnj[NF];
 #pragma unroll
           for (int f = 0; f < NF; ++f) {
-            if constexpr (PREC == PREC_DD) {
-              phs[f][jj] = c2[f][jj] - Mf[f];   // the re-centred drifted field
-              Dj[f] = D[f][jj] * inv12;
-            } else {
-              phs[f][jj] = c2[f][jj];
-              Dj[f] = D[f][jj];
-            }
+            phs[f][jj] = c2[f][jj] - Mf[f];   // the re-centred drifted field
+            Dj[f] = D[f][jj] * inv12;
             phj[f] = phs[f][jj];
             pmj[f] = q2[f][jj];
           }
-          if constexpr (PREC == PREC_DD) site_dd<MODEL>(cx, MODE, phj, Dj, pmj, pnj, acc);
-          else cx.site(MODE, phj, Dj, pmj, pnj, accd);
+          site_dd<MODEL>(cx, MODE, phj, Dj, pmj, pnj, acc);
 #pragma unroll
           for (int f = 0; f < NF; ++f) pin[f][jj] = pnj[f];
         }
@@ -974,15 +1179,13 @@ __device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PR
           gstore<T, VX>(phi_out + f * S + o, phs[f]);
           if (MODE == MODE_SWEEP) gstore<T, VX>(pi_out + f * S + o, pin[f]);
         }
-        if constexpr (PREC == PREC_DD) {
-          if (++kg == KGROUP) {
-            kg = 0;
+        if (++kg == KGROUP) {
+          kg = 0;
 #pragma unroll
-            for (int i2 = 0; i2 < NQ; ++i2) {
-              dd t = tot[i2 * kPThreads];
-              acc[i2].fold(t);
-              tot[i2 * kPThreads] = t;
-            }
+          for (int i2 = 0; i2 < NQ; ++i2) {
+            dd t = tot[i2 * kPThreads];
+            acc[i2].fold(t);
+            tot[i2 * kPThreads] = t;
           }
         }
       }
@@ -997,14 +1200,160 @@ __device__ __forceinline__ bool stage_wide(const PParams& p, const Ctx<MODEL, PR
         }
     }
   }
-  if constexpr (PREC == PREC_DD) {
 #pragma unroll
-    for (int i2 = 0; i2 < NQ; ++i2) {
-      dd t = tot[i2 * kPThreads];
-      acc[i2].fold(t);
-      tot[i2 * kPThreads] = t;
+  for (int i2 = 0; i2 < NQ; ++i2) {
+    dd t = tot[i2 * kPThreads];
+    acc[i2].fold(t);
+    tot[i2 * kPThreads] = t;
+  }
+  return ok;
+}
+
+// One stage of the FP64 form with the 13-point stencil: 12 D in fixed point
+// (stages without a scale: in float64).  The queue holds the two partial sums
+// and the two values along z; the drifted field and the momentum of the plane
+// put out are read from this warp's own rows of the drift buffers.
+template <int MODEL, int VX, int MODE, bool FIX>
+__device__ __forceinline__ bool stage_fp64_wide(const PParams& p,
+                                                const Ctx<MODEL, PREC_FP64>& cx0,
+                                                const PShared& sm, uint32_t gq, int ib,
+                                                double* accd, HiMax<Pot<MODEL>::NF>& hm) {
+  using C = Ctx<MODEL, PREC_FP64>;
+  using T = double;
+  using E = typename FixElem<FIX>::type;
+  using SL = typename C::SL;
+  constexpr int NF = C::NF;
+  constexpr int H = 2;
+  using LY = PLayout<NF, VX, 8, H>;
+  using RG = PRing<PREC_FP64, NF, VX, SL::NQ, H>;
+  using FL = FixLayout<NF, VX, H>;
+  constexpr int TX = LY::TX;
+  constexpr int NSLOT = RG::NSLOT, LEAD = RG::LEAD, NB = RG::NDRIFT;
+  static_assert(LEAD + 1 == NSLOT, "the stage issues plane gq + LEAD, then g + NSLOT at plane g");
+  const SimDesc& d = *sm.d;
+  const int tid = threadIdx.x, lane = tid & 31, ly = tid >> 5;
+  const int n = p.g.n;
+  const size_t S = (size_t)d.S, nn = (size_t)n * n;
+  T* __restrict__ phi_out = (T*)d.phi[(ib & 1) ^ 1];
+  T* __restrict__ pi_out = (T*)d.pi[((ib >> 1) & 1) ^ 1];
+  const int own = (ly + H) * FL::RS + 2 + lane * VX;
+  // the weights times 12; 1/12 goes into the kick's coefficient and, after the
+  // stage, into sum phi D
+  const E w1 = (E)16, w2 = (E)0 - (E)1, w0 = (E)0 - (E)90;
+  C cx = cx0;
+  cx.kD *= 1.0 / 12.0;
+  bool ok = true;
+
+  int pui = 0, puq = 0;
+  for (int l = 0; l < LEAD; ++l) padvance(sm, pui, puq);
+  if (tid == kPThreads - 32 && pui < sm.nunits) {
+    const uint32_t gp = gq + LEAD;
+    pproduce<NF, VX, 8, false, H>(p, ib, sm.units[pui], puq,
+                                  sm.ring + (size_t)(gp % NSLOT) * LY::SLOT_BYTES,
+                                  &sm.full[gp % NSLOT]);
+    sm.issued[gp % NSLOT] = gp + 1;
+  }
+  padvance(sm, pui, puq);
+
+  uint32_t g = gq;
+  if (sm.nunits > 0) ok = drift_fp64<MODEL, 13, VX, FIX>(cx, sm, g, sm.units[0], n);
+  for (int i = 0; i < sm.nunits && ok; ++i) {
+    const int4 u = sm.units[i];
+    const int Q = u.w;
+    const size_t o0 = (size_t)u.z * nn + (size_t)(u.y + ly) * n + u.x + lane * VX;
+    // z queue: partial sums and values of planes p-1, p-2
+    E P1[NF][VX], P2[NF][VX], c1[NF][VX], c2[NF][VX];
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int jj = 0; jj < VX; ++jj) P1[f][jj] = P2[f][jj] = c1[f][jj] = c2[f][jj] = (E)0;
+    for (int q = 0; q < Q; ++q, ++g) {
+      if (q + 1 < Q)
+        ok = drift_fp64<MODEL, 13, VX, FIX>(cx, sm, g + 1, u, n) && ok;
+      else if (i + 1 < sm.nunits)
+        ok = drift_fp64<MODEL, 13, VX, FIX>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
+      ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit) && ok;
+      if (!ok) break;
+      if (tid == 32 * (int)((4 * ((g + 1) % (kPWarps / 4)) + 4) % kPWarps) && pui < sm.nunits) {
+        const uint32_t gp = g + NSLOT;   // into slot g % NSLOT, free now
+        pproduce<NF, VX, 8, false, H>(p, ib, sm.units[pui], puq,
+                                      sm.ring + (size_t)(gp % NSLOT) * LY::SLOT_BYTES,
+                                      &sm.full[gp % NSLOT]);
+        sm.issued[gp % NSLOT] = gp + 1;
+      }
+      padvance(sm, pui, puq);
+      const double* buf = sm.drift + (size_t)(g % NB) * FL::ELEMS;
+      const bool mid = q >= 2 && q < Q - 2;   // a plane whose sites are output
+      E D[NF][VX];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        const E* fx = reinterpret_cast<const E*>(buf) + f * FL::FXF + own;
+        E cur[VX], m[VX];
+        vload<E, VX>(fx, cur);
+#pragma unroll
+        for (int jj = 0; jj < VX; ++jj) m[jj] = (E)0;
+        if (mid) {
+          E e[VX + 4], dn1[VX], up1[VX], dn2[VX], up2[VX];
+          e[0] = fx[-2]; e[1] = fx[-1]; e[VX + 2] = fx[VX]; e[VX + 3] = fx[VX + 1];
+#pragma unroll
+          for (int jj = 0; jj < VX; ++jj) e[jj + 2] = cur[jj];
+          vload<E, VX>(fx - FL::RS, dn1);
+          vload<E, VX>(fx + FL::RS, up1);
+          vload<E, VX>(fx - 2 * FL::RS, dn2);
+          vload<E, VX>(fx + 2 * FL::RS, up2);
+#pragma unroll
+          for (int jj = 0; jj < VX; ++jj) {
+            const E nr = (dn1[jj] + up1[jj]) + (e[jj + 1] + e[jj + 3]);
+            const E fr = (dn2[jj] + up2[jj]) + (e[jj] + e[jj + 4]);
+            m[jj] = fix_mad(w0, cur[jj], fix_mad(w2, fr, w1 * nr));
+          }
+        }
+#pragma unroll
+        for (int jj = 0; jj < VX; ++jj) {
+          D[f][jj] = fix_mad(w2, cur[jj], P2[f][jj]);   // plane p - 2: its last term
+          const E np1 = fix_mad(w1, cur[jj], P1[f][jj]);
+          P1[f][jj] = fix_mad(w2, c2[f][jj], fix_mad(w1, c1[f][jj], m[jj]));
+          P2[f][jj] = np1;
+          c2[f][jj] = c1[f][jj];
+          c1[f][jj] = cur[jj];
+        }
+      }
+      if (q >= 4) {  // output plane z0 + q - 4
+        const size_t o = o0 + (size_t)(q - 4) * nn;
+        const double* pbuf = sm.drift + (size_t)((g - 2) % NB) * FL::ELEMS + ly * TX + lane * VX;
+        T ph_m[NF][VX], pi_m[NF][VX], pin[NF][VX];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          vload<T, VX>(pbuf + FL::PH + f * FL::OWNF, ph_m[f]);
+          vload<T, VX>(pbuf + FL::PI + f * FL::OWNF, pi_m[f]);
+        }
+#pragma unroll
+        for (int jj = 0; jj < VX; ++jj) {
+          T phj[NF], Dj[NF], pmj[NF], pnj[NF];
+#pragma unroll
+          for (int f = 0; f < NF; ++f) {
+            phj[f] = ph_m[f][jj];
+            Dj[f] = fix_out(D[f][jj], cx.fx[f]);
+            pmj[f] = pi_m[f][jj];
+          }
+          cx.site(MODE, phj, Dj, pmj, pnj, accd);
+#pragma unroll
+          for (int f = 0; f < NF; ++f) {
+            pin[f][jj] = pnj[f];
+            hm.add(2 * f, phj[f]);
+            hm.add(2 * f + 1, pnj[f]);
+          }
+        }
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          gstore<T, VX>(phi_out + f * S + o, ph_m[f]);
+          if (MODE == MODE_SWEEP) gstore<T, VX>(pi_out + f * S + o, pin[f]);
+        }
+      }
     }
   }
+#pragma unroll
+  for (int f = 0; f < NF; ++f) accd[SL::PHID + f] *= 1.0 / 12.0;
   return ok;
 }
 
@@ -1290,7 +1639,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
   static_assert(STENCIL != 13 || PREC != PREC_SPLIT, "the 13-point stencil: FP64 and split-DD");
   using RG = PRing<PREC, NF, VX, NQ, H>;
   constexpr int NSLOT = RG::NSLOT, LEAD = RG::LEAD, PRE = RG::PRE;
-  static_assert(NQ <= kPWarps, "one warp per reduced quantity");
+  static_assert(RG::FOLD <= kPWarps, "one warp per reduced quantity");
   static_assert(PREC == PREC_SPLIT || (size_t)kMaxPBlocks * kNQ * 8 <= (size_t)NQ * kPThreads * 8,
                 "the rows of every block fit the reduction scratch");
 
@@ -1310,6 +1659,8 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
   // ring leaves little L1, so it is kept in shared memory
   __shared__ __align__(64) SimDesc s_desc;
   __shared__ double sums[kNQ];
+  __shared__ uint32_t s_wmax[kPWarps][2 * NF];   // FP64: each warp's largest |phi|, |pi| ...
+  __shared__ uint32_t s_amax[2 * kMaxFields];    // ... and the lattice's (Background::amax)
   __shared__ int4 s_units[kMaxPUnits];
   __shared__ uint32_t s_issued[NSLOT];
   __shared__ int s_bad;
@@ -1381,7 +1732,10 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
   {
     for (int l = kPWarps - 1 - warp; l < LEAD; l += kPWarps)   // warp 15 - l issues plane l
       prefetch_plane<PREC, NF, VX, CORNERS, NSLOT, H>(p, sm, ib, gq, l);
-    if (tid == 0) sctxv[0].init(sbv[0], d, K > 0 ? MODE_SWEEP : MODE_FLUSH);
+    if (tid == 0) {
+      sctxv[0].init(sbv[0], d, K > 0 ? MODE_SWEEP : MODE_FLUSH);
+      if constexpr (PREC == PREC_FP64) sctxv[0].set_fix(sbv[0].amax, fix_headroom<STENCIL>());
+    }
     __syncthreads();
     fault = s_bad != 0;
   }
@@ -1395,18 +1749,30 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
     double accd[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) accd[q] = 0.0;
-    if constexpr (STENCIL == 13) {
-      ok = (mode == MODE_SWEEP) ? stage_wide<MODEL, VX, MODE_SWEEP, PREC>(p, cx, sm, gq, ib, accd)
-                                : stage_wide<MODEL, VX, MODE_FLUSH, PREC>(p, cx, sm, gq, ib, accd);
-      if constexpr (PREC == PREC_DD) {
-        const dd* tot = reinterpret_cast<const dd*>(sm.red) + tid;
+    HiMax<NF> hm;   // FP64: largest |phi|, |pi| put out
+    hm.zero();
+    if constexpr (PREC == PREC_FP64) {
+      const bool fix = cx.fx[0] != 0;
+      auto stage = [&](auto mode_c, auto fix_c) {
+        constexpr int MD = decltype(mode_c)::value;
+        constexpr bool FX = decltype(fix_c)::value;
+        if constexpr (STENCIL == 13)
+          return stage_fp64_wide<MODEL, VX, MD, FX>(p, cx, sm, gq, ib, accd, hm);
+        else
+          return stage_fp64<MODEL, STENCIL, VX, MD, FX>(p, cx, sm, gq, ib, accd, hm);
+      };
+      using MS = std::integral_constant<int, MODE_SWEEP>;
+      using MF = std::integral_constant<int, MODE_FLUSH>;
+      if (mode == MODE_SWEEP)
+        ok = fix ? stage(MS{}, std::true_type{}) : stage(MS{}, std::false_type{});
+      else
+        ok = fix ? stage(MF{}, std::true_type{}) : stage(MF{}, std::false_type{});
+    } else if constexpr (STENCIL == 13) {
+      ok = (mode == MODE_SWEEP) ? stage_wide_dd<MODEL, VX, MODE_SWEEP>(p, cx, sm, gq, ib)
+                                : stage_wide_dd<MODEL, VX, MODE_FLUSH>(p, cx, sm, gq, ib);
+      const dd* tot = reinterpret_cast<const dd*>(sm.red) + tid;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) accd[q] = (double)tot[q * kPThreads];
-      }
-    } else if constexpr (PREC == PREC_FP64) {
-      ok = (mode == MODE_SWEEP)
-               ? stage_fp64<MODEL, STENCIL, VX, MODE_SWEEP>(p, cx, sm, gq, ib, accd)
-               : stage_fp64<MODEL, STENCIL, VX, MODE_FLUSH>(p, cx, sm, gq, ib, accd);
+      for (int q = 0; q < NQ; ++q) accd[q] = (double)tot[q * kPThreads];
     } else if constexpr (PREC == PREC_DD) {
       ok = (mode == MODE_SWEEP) ? stage_dd<MODEL, STENCIL, VX, MODE_SWEEP>(p, cx, sm, gq, ib)
                                 : stage_dd<MODEL, STENCIL, VX, MODE_FLUSH>(p, cx, sm, gq, ib);
@@ -1444,6 +1810,13 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
       double* red = sm.red;
 #pragma unroll
       for (int q = 0; q < NQ; ++q) red[q * kPThreads + tid] = accd[q];
+      if constexpr (PREC == PREC_FP64) {
+#pragma unroll
+        for (int i = 0; i < 2 * NF; ++i) {
+          const uint32_t m = __reduce_max_sync(0xffffffffu, hm.v[i]);
+          if (lane == 0) s_wmax[warp][i] = m;
+        }
+      }
       __syncthreads();
       if (warp < NQ) {
         // 16 values per lane summed as a pairwise tree (depth 4: FP64 latency is long)
@@ -1460,6 +1833,21 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         if (lane == 0) {
           reinterpret_cast<double*>(p.rows)[((size_t)(k & 1) * G + blockIdx.x) * kNQ + warp] = v;
           fence_proxy_async_global();   // the rows are read back by bulk copies
+        }
+      } else if (PREC == PREC_FP64 && warp == NQ) {
+        // the block's largest |phi| and |pi| of field f in the row's slot kNQ - 2 + f
+        static_assert(PREC != PREC_FP64 || NQ <= kNQ - kMaxFields, "free slots of a row");
+        uint32_t m[2 * NF];
+#pragma unroll
+        for (int i = 0; i < 2 * NF; ++i)
+          m[i] = __reduce_max_sync(0xffffffffu, s_wmax[lane % kPWarps][i]);
+        if (lane == 0) {
+          uint2* row = reinterpret_cast<uint2*>(
+              reinterpret_cast<double*>(p.rows) + ((size_t)(k & 1) * G + blockIdx.x) * kNQ +
+              kNQ - kMaxFields);
+#pragma unroll
+          for (int f = 0; f < NF; ++f) row[f] = make_uint2(m[2 * f], m[2 * f + 1]);
+          fence_proxy_async_global();
         }
       }
     } else {
@@ -1556,6 +1944,24 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         if (lane == 0) sums[warp] = (double)hi + (double)lo;
       }
       // @sums-written
+    } else if (PREC == PREC_FP64 && warp == NQ) {
+      // the lattice's largest |phi| and |pi| of each field
+      if (!mbar_wait(&foldbar, (uint32_t)(k & 1), p.wait_limit)) atomicOr(&s_bad, 1);
+      uint32_t m[2 * NF];
+#pragma unroll
+      for (int i = 0; i < 2 * NF; ++i) m[i] = 0u;
+      for (int r = lane; r < G; r += 32)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          const uint2 x = reinterpret_cast<const uint2*>(srows)[(size_t)r * kNQ + kNQ - kMaxFields + f];
+          m[2 * f] = max(m[2 * f], x.x);
+          m[2 * f + 1] = max(m[2 * f + 1], x.y);
+        }
+#pragma unroll
+      for (int i = 0; i < 2 * NF; ++i) {
+        m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+        if (lane == 0) s_amax[i] = 0x80000000u | m[i];
+      }
     } else {
       const int l0 = kPWarps - 1 - warp;
       if (pre && l0 < PRE) {
@@ -1587,6 +1993,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
             for (int f = 0; f < NF; ++f)
               nx.shiftK[f] = (mn == MODE_FLUSH) ? flush_shift(d, ib_next, f, nx.k.c) : 0.0;
             nx.set_qref(d, ib_next);
+            nx.set_fix(s_amax, fix_headroom<STENCIL>());
           }
         }
         if constexpr (PREC != PREC_FP64) {
@@ -1610,6 +2017,10 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
       }
     } else if (tid == kPThreads - 96) {
       post_stage<MODEL, PREC>(cc, s_sc, d, mode, sums, sbv[cb], sbv[cb ^ 1]);
+      if constexpr (PREC == PREC_FP64) {
+#pragma unroll
+        for (int i = 0; i < 2 * NF; ++i) sbv[cb ^ 1].amax[i] = s_amax[i];
+      }
       // @book-done
     }
     __syncthreads();

@@ -243,6 +243,8 @@ template <> struct Vec<float, 2> { using type = float2; };
 template <> struct Vec<float, 4> { using type = float4; };
 template <> struct Vec<double, 1> { using type = double; };
 template <> struct Vec<double, 2> { using type = double2; };
+template <> struct Vec<unsigned long long, 1> { using type = unsigned long long; };
+template <> struct Vec<unsigned long long, 2> { using type = ulonglong2; };
 template <> struct Vec<dd, 1> { using type = float2; };
 template <> struct Vec<dd, 2> { using type = float4; };
 
@@ -314,6 +316,9 @@ struct Ctx {
   double phi0s[NF], pi0s[NF], V0;  // split forms: background after drift / kick
   typename SplitKOf<MODEL, PREC>::type sk;
   double q_inv, q_lref;            // FP64 Q-ball: 1/(2 u_ref), ln(u_ref/M^2) (0, 0: no reference)
+  // FP64 persistent kernel: the fixed-point scale of each field's stencil (set_fix);
+  // fx[0] = 0: the stage computes its stencil in floating point
+  int fx[NF];
 
   __device__ __forceinline__ void init(const Background& bg, const SimDesc& d, int mode,
                                        double ia_a = -1.0) {
@@ -327,7 +332,32 @@ struct Ctx {
       for (int f = 0; f < NF; ++f)
         shiftK[f] = (mode == MODE_FLUSH) ? (T)flush_shift(d, bg.cur, f, k.c) : (T)0;
       set_qref(d, bg.cur);
+      fx[0] = 0;
     }
+  }
+
+  //   set_fix (FP64 persistent kernel): the exponents E_f of the stage's
+  //   fixed-point fields, I = phi* 2^(1086 - E_f) (to_fixed), from the largest
+  //   |phi| and |pi| of the stage's input (amax) and the drift coefficient.  F
+  //   and P, one unit of the high word above the largest values, bound
+  //   |phi*| <= B = F + |c| P (rounding is monotonic), and with e the biased
+  //   exponent of B, |phi*| < 2^(e - 1022), so E_f = e + headroom + 1 gives
+  //   |I| < 2^(63 - headroom).  No fixed point (fx[0] = 0) where a maximum is
+  //   unknown, not finite or out of the range that E_f can take.
+  __device__ __forceinline__ void set_fix(const uint32_t* amax, int headroom) {
+    bool ok = true;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const uint32_t mf = amax[2 * f], mp = amax[2 * f + 1];
+      const double F = __hiloint2double((int)((mf & 0x7fffffffu) + 1u), 0);
+      const double P = __hiloint2double((int)((mp & 0x7fffffffu) + 1u), 0);
+      const int e = (__double2hiint(fma(fabs(k.c), P, F)) >> 20) & 0x7ff;
+      // (a field that is zero everywhere has no scale of its own: any serves)
+      ok = ok && (mf >> 31) && (mp >> 31) && (mf << 1) < 0xffe00000u && (mp << 1) < 0xffe00000u &&
+           e < 1990 && (e >= 70 || ((mf | mp) << 1) == 0u);
+      fx[f] = max(e, 70) + headroom + 1;
+    }
+    if (!ok) fx[0] = 0;
   }
 
   //   set_qref (FP64 Q-ball): the reference of the logarithm, |Phi|^2/2 of the
@@ -836,6 +866,8 @@ __device__ __forceinline__ void finish_block(const C& cx, const SimDesc& d, int 
   Background* bgp = d.bg;
   Background nb;
   post_stage<MODEL, PREC>(cx, d, mode, sout, *bgp, nb);
+#pragma unroll
+  for (int i = 0; i < 2 * kMaxFields; ++i) nb.amax[i] = 0u;   // not tracked here
   *bgp = nb;  // published to the next launch by the kernel boundary
   *d.ticket = 0u;
 }

@@ -169,34 +169,51 @@ template <> struct Pot<M_QBALL> {
       dV[0] = 0.0; dV[1] = 0.0; V = 0.0;
     }
   }
-  // For the FP64 sweep: from u2 = |Phi|^2 = 2u, the factor fac of V'_i =
-  // fac f_i and twice the potential,
-  //   fac = m2 (1 + K) + m2 K l,   V2 = 2V = u2 (m2 + m2 K l),   l = ln(u/M^2),
-  // with the logarithm taken near a reference u_ref (the sweep's per-stage
-  // value at one site, the same in every block): hinv = 1/(2 u_ref), lref =
-  // ln(u_ref/M^2), x = u/u_ref - 1 = u2 hinv - 1 and l = lref + log1p(x) by its
-  // Taylor series sum_k (-1)^(k+1) x^k / k -- 5 terms for |x| < 2^-12 (the
-  // first omitted term is below 2^-60 |x|), 11 terms for |x| < 2^-5 (below
-  // 2^-60 |x|) -- and the full logarithm farther away or without a reference
-  // (hinv = 0 gives x = -1).  The tiers are chosen on the high word of x as an
-  // integer, and Phi = 0 on the bits of u2 (never negative), so that no
-  // float64 instruction is spent on the tests.
-  __device__ static void fac_near(const K& k, double u2, double hinv, double lref, double& fac,
-                                  double& V2) {
-    if (__double_as_longlong(u2) == 0) {   // Phi = 0: V = V' = 0
-      fac = 0.0;
-      V2 = 0.0;
-      return;
-    }
+  // For the FP64 site: from u2 = |Phi|^2 = 2u, the factor sc fac of the kick
+  // sc V'_i = sc fac phi_i,
+  //   fac = m2 (1 + K) + m2 K l,   l = ln(u/M^2) = lref + log1p(x),
+  //   x = u/u_ref - 1 = u2 hinv - 1,   hinv = 1/(2 u_ref), lref = ln(u_ref/M^2)
+  // with u_ref the sweep's per-stage value at one site, the same in every
+  // block.  With B = sc m2 K = ks[3], ks[0] = sc (m2 (1 + K) + m2 K lref) - B
+  // and ks[1] = B hinv,
+  //   sc fac = ks[0] + B (1 + log1p x) = (ks[0] + ks[1] u2) + B (log1p(x) - x),
+  // so that near the reference only one FMA and one addition are float64: for
+  // |x| < 2^-14 the last term, below 2^-29 B, is formed in float32 (its rounding
+  // is below 2^-51 B, and B is a fraction of the sum) and the conversions are
+  // integer instructions (float64 arithmetic and conversions run at 1/64 of the
+  // float32 rate on GB300).  Farther away log1p is its Taylor series
+  // sum_k (-1)^(k+1) x^k / k -- 5 terms for |x| < 2^-12 (the first omitted term
+  // is below 2^-60 |x|), 11 terms for |x| < 2^-5 (below 2^-60 |x|) -- and the
+  // full logarithm beyond or without a reference (hinv = 0 gives x = -1).  The
+  // tiers are chosen on the high word of x as an integer, and Phi = 0 on the
+  // bits of u2 (never negative), so that no float64 instruction is spent on the
+  // tests.
+  __device__ static double fac_near(const double* ks, double lnM2, double u2, double hinv,
+                                    double lref) {
+    if (__double_as_longlong(u2) == 0) return 0.0;   // Phi = 0: V = V' = 0
     const double x = fma(u2, hinv, -1.0);
     const int hx = __double2hiint(x) & 0x7fffffff;
-    double l;
+    if (hx < 0x3F100000) {            // |x| < 2^-14
+      // x to float32 (cut; below 2^-126: 0)
+      const int t = hx - 0x38000000;
+      const uint32_t xm = t >= 0x00100000 ? ((uint32_t)t << 3) | ((uint32_t)__double2loint(x) >> 29) : 0u;
+      const float xf = __int_as_float((int)(xm | ((uint32_t)__double2hiint(x) & 0x80000000u)));
+      float q = fmaf(xf, -0.25f, 1.f / 3.f);
+      q = fmaf(q, xf, -0.5f);
+      const float c = q * (xf * xf);
+      // c to float64 (exact; denormals: 0)
+      const uint32_t cb = (uint32_t)__float_as_int(c), cm = cb & 0x7fffffffu;
+      const uint32_t ch = cm >= 0x00800000u ? (cm >> 3) + 0x38000000u : 0u;
+      const double cd = __hiloint2double((int)(ch | (cb & 0x80000000u)), (int)(cm << 29));
+      return fma(ks[3], cd, fma(ks[1], u2, ks[0]));
+    }
+    double l1;                        // 1 + log1p(x)
     if (hx < 0x3F300000) {            // |x| < 2^-12
       double q = fma(x, 0.2, -0.25);
       q = fma(q, x, 1.0 / 3.0);
       q = fma(q, x, -0.5);
       q = fma(q, x, 1.0);
-      l = fma(q, x, lref);
+      l1 = fma(q, x, 1.0);
     } else if (hx < 0x3FA00000) {     // |x| < 2^-5
       double q = fma(x, -1.0 / 12.0, 1.0 / 11.0);
       q = fma(q, x, -0.1);
@@ -209,12 +226,11 @@ template <> struct Pot<M_QBALL> {
       q = fma(q, x, 1.0 / 3.0);
       q = fma(q, x, -0.5);
       q = fma(q, x, 1.0);
-      l = fma(q, x, lref);
+      l1 = fma(q, x, 1.0);
     } else {
-      l = log(0.5 * u2) - k.lnM2;
+      l1 = (log(0.5 * u2) - lnM2) - (lref - 1.0);
     }
-    fac = fma(k.mK, l, k.m2K1);
-    V2 = u2 * fma(k.mK, l, k.m2);
+    return fma(ks[3], l1, ks[0]);
   }
   // du = d1 (p1 + d1/2) + d2 (p2 + d2/2),  l = log1p(du/u0)
   //   dV'_i = m2 [ A d_i + K l (p_i + d_i) ],  A = 1 + K + K L0

@@ -569,11 +569,12 @@ __device__ __forceinline__ bool drift_fp64(const Ctx<MODEL, PREC_FP64>& cx, cons
   using FL = FixLayout<NF, VX, H>;
   constexpr int TX = LY::TX, CW = LY::CW, NSLOT = RG::NSLOT, NB = RG::NDRIFT;
   const int tid = threadIdx.x, lane = tid & 31, ly = tid >> 5;
-  const int side = lane == 31 ? 1 : 0;
-  const bool edge = lane == 0 || lane == 31;
   const int own = (ly + H) * TX + lane * VX;
   const int s = gg % NSLOT, b = gg % NB;
-  // the 2H halo rows of this plane go to warps 2H j .. 2H j + 2H - 1, j = gg mod (16 / 2H)
+  // the 2H halo rows of this plane go to warps 2H j .. 2H j + 2H - 1, j = gg
+  // mod (16 / 2H), and the halo columns of field f to the warp f after them (a
+  // lane per row and side: in the row's own warp they would cost a float64
+  // instruction of all 32 lanes for two values)
   const int hw = (ly - 2 * H * (int)(gg % (kPWarps / (2 * H))) + kPWarps) % kPWarps;
   const int hrow = hw < H ? hw : kPTY + hw;
   const bool ok = mbar_wait(&sm.full[s], (gg / NSLOT) & 1, sm.limit);
@@ -608,23 +609,19 @@ __device__ __forceinline__ bool drift_fp64(const Ctx<MODEL, PREC_FP64>& cx, cons
       for (int jj = 0; jj < VX; ++jj) q[jj] = fix_in(madd(cd, c[jj], a[jj]), ex, (E*)nullptr);
       vstore<E, VX>(fx + hrow * FL::RS + lane * VX, q);
     }
-    if (edge) {
-      // the H halo columns of this side (k = 0 adjacent), this warp's row and,
-      // 27-point stencil, the corner cells of a halo row
+    // a halo cell: column k (0 adjacent) of a side, row r (0: y0 - 1)
+    auto cell = [&](int side, int k, int r) {
+      const int cc = side ? k : CW - 1 - k;
+      const int row = clear ? LY::col_dense(f, r) : LY::col_wrap(f, r);
+      fx[(r + H - 1) * FL::RS + (side ? TX + k : -1 - k)] =
+          fix_in(madd(cd, (sl + LY::col_base(1, side))[cc + row],
+                      (sl + LY::col_base(0, side))[cc + row]), ex, (E*)nullptr);
+    };
+    if (hw == 2 * H + f) {
 #pragma unroll
-      for (int k = 0; k < H; ++k) {
-        const int cc = side ? k : CW - 1 - k;
-        const double* cph = sl + LY::col_base(0, side) + cc;
-        const double* cpi = sl + LY::col_base(1, side) + cc;
-        const int x = side ? TX + k : -1 - k;
-        const int row = clear ? LY::col_dense(f, ly + 1) : LY::col_wrap(f, ly + 1);
-        fx[(ly + H) * FL::RS + x] = fix_in(madd(cd, cpi[row], cph[row]), ex, (E*)nullptr);
-        if (CORNERS && hw < 2) {
-          const int cr = clear ? LY::col_dense(f, hrow) : LY::col_wrap(f, hrow);
-          fx[hrow * FL::RS + x] = fix_in(madd(cd, cpi[cr], cph[cr]), ex, (E*)nullptr);
-        }
-      }
+      for (int k = 0; k < H; ++k) cell(lane >> 4, k, (lane & 15) + 1);
     }
+    if (CORNERS && hw < 2 && (lane == 0 || lane == 31)) cell(lane == 31, 0, hrow);
   }
   // generic reads of the ring slot before the TMA copy that refills it (drift_dd)
   fence_proxy_async();
@@ -701,7 +698,7 @@ __device__ __forceinline__ bool stage_fp64(const PParams& p, const Ctx<MODEL, PR
       // every warp has drifted plane g
       ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit) && ok;
       if (!ok) break;
-      if (tid == 32 * (int)((2 * ((g + 1) % (kPWarps / 2)) + 2) % kPWarps) && pui < sm.nunits) {
+      if (tid == 32 * (int)((2 * ((g + 1) % (kPWarps / 2)) + 4) % kPWarps) && pui < sm.nunits) {
         const uint32_t gp = g + NSLOT;   // into slot g % NSLOT, free now
         pproduce<NF, VX, 8, CORNERS>(p, ib, sm.units[pui], puq,
                                      sm.ring + (size_t)(gp % NSLOT) * LY::SLOT_BYTES,
@@ -1274,7 +1271,7 @@ __device__ __forceinline__ bool stage_fp64_wide(const PParams& p,
         ok = drift_fp64<MODEL, 13, VX, FIX>(cx, sm, g + 1, sm.units[i + 1], n) && ok;
       ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit) && ok;
       if (!ok) break;
-      if (tid == 32 * (int)((4 * ((g + 1) % (kPWarps / 4)) + 4) % kPWarps) && pui < sm.nunits) {
+      if (tid == 32 * (int)((4 * ((g + 1) % (kPWarps / 4)) + 6) % kPWarps) && pui < sm.nunits) {
         const uint32_t gp = g + NSLOT;   // into slot g % NSLOT, free now
         pproduce<NF, VX, 8, false, H>(p, ib, sm.units[pui], puq,
                                       sm.ring + (size_t)(gp % NSLOT) * LY::SLOT_BYTES,

@@ -61,6 +61,7 @@ struct Coef {
   double kD;     // a^2 h / dx^2
   double kV;     // a^4 h
   double a;      // a after the leading Phi_H1's
+  double ia;     // 1/a (0 for a flush)
   double pa;     // p_a after the leading Phi_H2 (before this stage's Phi_H3)
   double h;      // this stage's step (0 for a flush)
   double deta;   // the conformal step of this stage's time step (h = w_i deta)
@@ -146,12 +147,13 @@ __device__ __forceinline__ Coef prestage_p(const PreCoef& q, double pa, double s
   }
   k.a = a;
   if (mode != MODE_SWEEP) {
-    k.c = q.c0; k.kD = 0.0; k.kV = 0.0; k.pa = pa; k.h = 0.0;
+    k.c = q.c0; k.kD = 0.0; k.kV = 0.0; k.pa = pa; k.h = 0.0; k.ia = 0.0;
     return k;
   }
   // one reciprocal per value of a instead of divisions: an FP64 division costs
   // ~450 cycles of a single thread on GB300
   const double ia = __drcp_rn(a), ia2 = ia * ia;
+  k.ia = ia;
   // leading Phi_H2(h/2)
   k.pa = fma(fma(s2, ia2 * ia, q.nVLrm), hn, pa);
   k.c = fma(hn, ia2, q.c0);
@@ -310,7 +312,12 @@ struct Ctx {
   Coef k;
   typename P::K pk;
   T cdrift, kD, kV;
-  T nkVg;                          // FP64 chaotic model: -kV g2 (folded into the chi kick)
+  // FP64: the potential's constants times sc, sc = -kV in a sweep (so that a
+  // kick is one FMA per field: pi + (sc V'/phi) phi) and 1 in a flush
+  //   chaotic:  m2, g2     oscillon: m2, -lam, g
+  //   Q-ball:   sc fac = ks[0] + ks[3] (1 + log1p x) ~ ks[0] + ks[1] u2,  ks[2] = -ks[3]
+  //             (set_qref)
+  double sc, ks[4];
   T mu_phi[NF], mu_pi[NF];
   T shiftK[NF];
   double phi0s[NF], pi0s[NF], V0;  // split forms: background after drift / kick
@@ -369,6 +376,10 @@ struct Ctx {
       const double u = 0.5 * fma(f0, f0, f1 * f1);
       q_inv = u > 0.0 ? 0.5 / u : 0.0;
       q_lref = u > 0.0 ? log(u) - pk.lnM2 : 0.0;
+      ks[3] = sc * pk.mK;
+      ks[0] = fma(sc, fma(pk.mK, q_lref, pk.m2K1), -ks[3]);
+      ks[1] = ks[3] * q_inv;
+      ks[2] = -ks[3];
     }
   }
 
@@ -380,7 +391,11 @@ struct Ctx {
     pk = pkk;
     cdrift = (T)k.c; kD = (T)k.kD; kV = (T)k.kV;
     if constexpr (PREC == PREC_FP64) {
-      if constexpr (MODEL == M_CHAOTIC2) nkVg = -k.kV * d.params[1];
+      sc = (mode == MODE_SWEEP) ? -k.kV : 1.0;
+      if constexpr (MODEL == M_CHAOTIC2) { ks[0] = sc * pk.m2; ks[1] = sc * pk.g2; }
+      if constexpr (MODEL == M_OSCILLON) {
+        ks[0] = sc * pk.m2; ks[1] = -(sc * pk.lam); ks[2] = sc * pk.g;
+      }
       V0 = 0.0;
 #pragma unroll
       for (int f = 0; f < NF; ++f) { mu_phi[f] = 0; mu_pi[f] = 0; phi0s[f] = 0; pi0s[f] = 0; }
@@ -420,18 +435,36 @@ struct Ctx {
   template <bool GENERAL = false>
   __device__ __forceinline__ void site(int mode, const T (&phj)[NF], const T (&D)[NF],
                                        const T (&pim)[NF], T (&pin)[NF], T* ps) const {
-    if constexpr (PREC == PREC_FP64 && MODEL == M_CHAOTIC2) {
-      // V = phi^2 (m2 + g2 chi^2)/2; the kicks with kV folded into the products,
-      // and 2V accumulated (halved once, in post_stage): 4 DMUL + 6 DFMA
-      const double ph2 = phj[0] * phj[0];
-      const double t = fma(pk.g2, phj[1] * phj[1], pk.m2);      // m2 + g2 chi^2
-      if (mode == MODE_SWEEP) {
-        pin[0] = madd(kD, D[0], madd(-kV * phj[0], t, pim[0]));   // - kV phi (m2 + g2 chi^2)
-        pin[1] = madd(kD, D[1], madd(nkVg * ph2, phj[1], pim[1]));   // - kV g2 phi^2 chi
+    if constexpr (PREC == PREC_FP64 && MODEL != M_FREE) {
+      // the kick of field f is pi_f + kf[f] phi_f with kf = sc V'_f/phi_f; the
+      // chaotic and Q-ball models' V slot sums sc 2V (see SumCoef::kb).  Folding
+      // sc = -kV into the constants and a common factor out of V and V' leaves
+      // 7 float64 instructions for the chaotic model's V and kicks (8 before),
+      // 8 for the oscillon's (10) and, near the reference, 8 for the Q-ball's
+      // (14): 256^3 Q-ball, order 8, two steps 25.2 -> 17.8 ms, oscillon 8.9 ->
+      // 8.1 ms, 128^3 preheating 2.83 -> 2.52 ms (with the halo columns below)
+      double kf[NF];
+      if constexpr (MODEL == M_CHAOTIC2) {
+        // V = phi^2 (m2 + g2 chi^2)/2
+        const double ph2 = phj[0] * phj[0];
+        kf[0] = fma(ks[1], phj[1] * phj[1], ks[0]);          // sc (m2 + g2 chi^2)
+        if (mode == MODE_SWEEP) kf[1] = ks[1] * ph2;         // sc g2 phi^2
+        ps[SL::V] = madd(ph2, kf[0], ps[SL::V]);
+      } else if constexpr (MODEL == M_OSCILLON) {
+        const double x2 = phj[0] * phj[0];
+        if (mode == MODE_SWEEP) kf[0] = fma(x2, fma(ks[2], x2, ks[1]), ks[0]);
+        ps[SL::V] = madd(x2, fma(x2, fma(pk.sg, x2, -pk.qlam), pk.hm2), ps[SL::V]);
+      } else {
+        static_assert(MODEL == M_QBALL, "a site for every model");
+        // sc fac from |Phi|^2 (the logarithm near the stage's reference value)
+        const double u2 = fma(phj[0], phj[0], phj[1] * phj[1]);
+        kf[0] = kf[1] = P::fac_near(ks, pk.lnM2, u2, q_inv, q_lref);
+        ps[SL::V] = madd(u2, kf[0] + ks[2], ps[SL::V]);      // sc 2V = sc u2 (fac - m2 K)
       }
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
         if (mode == MODE_SWEEP) {
+          pin[f] = madd(kD, D[f], madd(kf[f], phj[f], pim[f]));
           ps[SL::PI2 + f] = madd(pin[f], pin[f], ps[SL::PI2 + f]);
         } else {
           pin[f] = pim[f];
@@ -442,33 +475,6 @@ struct Ctx {
         }
         ps[SL::PHID + f] = madd(phj[f], D[f], ps[SL::PHID + f]);
       }
-      ps[SL::V] = madd(ph2, t, ps[SL::V]);
-    } else if constexpr (PREC == PREC_FP64 && MODEL == M_QBALL) {
-      // V'_i = fac phi_i and 2V from |Phi|^2 (Pot::fac_near: the logarithm
-      // near the stage's reference value); the kicks as pi - (kV fac) phi_i,
-      // and 2V accumulated (halved once, in post_stage)
-      const double u2 = fma(phj[0], phj[0], phj[1] * phj[1]);
-      double fac, V2;
-      P::fac_near(pk, u2, q_inv, q_lref, fac, V2);
-      if (mode == MODE_SWEEP) {
-        const double kf = -kV * fac;
-#pragma unroll
-        for (int f = 0; f < NF; ++f) pin[f] = madd(kD, D[f], madd(kf, phj[f], pim[f]));
-      }
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        if (mode == MODE_SWEEP) {
-          ps[SL::PI2 + f] = madd(pin[f], pin[f], ps[SL::PI2 + f]);
-        } else {
-          pin[f] = pim[f];
-          ps[SL::PI2 + f] = madd(pim[f], pim[f], ps[SL::PI2 + f]);
-          const T dd = phj[f] - shiftK[f];
-          ps[SL::DPHI + f] += dd;
-          ps[SL::DPHI2 + f] = madd(dd, dd, ps[SL::DPHI2 + f]);
-        }
-        ps[SL::PHID + f] = madd(phj[f], D[f], ps[SL::PHID + f]);
-      }
-      ps[SL::V] += V2;
     } else if constexpr (PREC == PREC_FP64) {
       double dV[NF], V;
       P::eval(pk, phj, dV, V);
@@ -633,8 +639,11 @@ __device__ __forceinline__ void fold_rows(const double* src, int P, double* out)
 // The coefficients that turn a stage's reduced slots into lattice sums and
 // the p_a kick; they depend only on the stage's Ctx, so a caller can form
 // them before the sums arrive.
+// Do the FP64 sites of a model sum sc 2V (sc = -kV in a sweep) instead of V?
+template <int MODEL> constexpr bool scaled_v() { return MODEL == M_CHAOTIC2 || MODEL == M_QBALL; }
+
 template <int NF> struct SumCoef {
-  double ka, kb, pa;         // Phi_H3: p_a += ka sum phi D + kb sum V
+  double ka, kb, pa;         // Phi_H3: p_a += ka sum phi D + kb (the V slot's sum)
   double spi[NF], tpi[NF];   // split form: S pi0s and 2 pi0s
 };
 
@@ -644,7 +653,8 @@ __device__ __forceinline__ SumCoef<C::NF> sum_coef(const C& cx, const SimDesc& d
   // Phi_H3(h): p_a += h a^3 [sum phi D/(a^2 dx^2) - 4 sum V]   (Eq. split-Phi)
   const double a = cx.k.a, h = cx.k.h;
   q.ka = (h * a) * d.dx2inv;
-  q.kb = -4.0 * (h * ((a * a) * a));
+  // sc 2V summed: -4 h a^3 sum V = (2 / a) sum (-kV 2V), kV = a^4 h
+  q.kb = (PREC == PREC_FP64 && scaled_v<MODEL>()) ? 2.0 * cx.k.ia : -4.0 * (h * ((a * a) * a));
   q.pa = cx.k.pa;
 #pragma unroll
   for (int f = 0; f < C::NF; ++f) {
@@ -677,8 +687,8 @@ __device__ __forceinline__ void stage_sums(const C& cx, const SumCoef<C::NF>& q,
       fdphi[f] = (mode == MODE_FLUSH) ? sout[SL::DPHI + f] : 0.0;
       fdphi2[f] = (mode == MODE_FLUSH) ? sout[SL::DPHI2 + f] : 0.0;
     }
-    // the chaotic and Q-ball models' FP64 sites accumulate 2V (see Ctx::site)
-    sum_V = (MODEL == M_CHAOTIC2 || MODEL == M_QBALL) ? 0.5 * sout[SL::V] : sout[SL::V];
+    // scaled_v: a flush's slot holds 2V, a sweep's -kV 2V (used by pa_kick only)
+    sum_V = (scaled_v<MODEL>() && mode == MODE_FLUSH) ? 0.5 * sout[SL::V] : sout[SL::V];
   } else {
 #pragma unroll
     for (int f = 0; f < NF; ++f) {

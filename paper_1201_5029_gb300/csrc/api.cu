@@ -160,7 +160,12 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
   const bool l2_resident = l2_bytes > 0 && stage_bytes <= 0.75 * (double)l2_bytes;
   const double h = prec != PREC_SPLIT ? 0.25 : (l2_resident ? 1.5 : 0.3);
   const double pen = prec != PREC_SPLIT ? 1.0 : 1.24;
-  constexpr int kMinPiece = 4;   // planes: no unit shorter than this is cut off a chunk
+  // Planes: no unit shorter than this is cut off a chunk.  A lattice of side 32 has
+  // 64 (tile, plane) pairs, so single planes spread it over 64 SMs where pieces of
+  // four left 16 at work: 32^3 per stage, FP64 chaotic 19.4 -> 10.7 us, split-FP32
+  // 10.0 -> 7.7, split-DD 25.1 -> 19.0; 64^3 split-FP32 10.8 -> 9.1; the larger
+  // ones are cut the same as before.
+  constexpr int kMinPiece = 1;
   const int cap = std::min(sms, kMaxPBlocks);
   auto is_wrap = [&](int t) {
     const int ty = t / g.tiles_x;

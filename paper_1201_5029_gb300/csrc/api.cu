@@ -97,6 +97,7 @@ Layout layout_for(const pycool_config& c) {
   L.off_punits = 0;
   L.off_rt = 0;
   L.off_mean = 0;
+  L.plain = false;
   if (runtime) {   // drifted fields, V' (N_f n^3 each) and V (n^3)
     L.off_rt = align256(L.ws_bytes);
     L.ws_bytes = L.off_rt + 2 * align256((size_t)nf * S * 8) + align256(S * 8);
@@ -108,19 +109,47 @@ Layout sim_layout(const pycool_config& c) {
   Layout L = layout_for(c);
   L.off_mean = align256(L.ws_bytes);
   L.ws_bytes = L.off_mean + align256((size_t)2 * kMeanBlocks * sizeof(double));
-  // the persistent kernel: n a multiple of 32, compiled models; the 13-point
-  // stencil in the FP64 and split-DD forms only (its per-stage fallback,
-  // like the split-FP32 form's, keeps the plain geometry)
-  const bool persist_ok =
+  // the persistent kernel, compiled models: TMA staging for n a multiple of 32
+  // (the 13-point stencil in the FP64 and split-DD forms), plain staging for
+  // every other n and for the split-FP32 form's 13-point stencil (faster than
+  // the per-stage kernels at every side from 16 to 256: persist_plain.cuh; TMA
+  // staging where it fits: 128^3 split-FP32 18 us per stage, plain 35)
+  const bool tma_ok =
       L.geo.tma || (c.stencil == PYCOOL_STENCIL_4TH && c.n % 32 == 0 &&
                     c.model < kRuntimeModelBase && c.precision != PYCOOL_SPLIT_FP32);
-  if (persist_ok) {
+  L.plain = !tma_ok && c.model < kRuntimeModelBase && c.precision != PYCOOL_SPLIT_DD;
+  if (tma_ok || L.plain) {
     L.off_prows = align256(L.ws_bytes);
     L.off_punits = L.off_prows + align256((size_t)2 * kMaxPBlocks * kNQ * sizeof(double));
     L.ws_bytes = L.off_punits + align256((size_t)kMaxPBlocks * kMaxPUnits * sizeof(int4)) +
                  align256((size_t)(kMaxPBlocks + 1) * sizeof(int));
   }
   return L;
+}
+
+// Tiles of the plain staging: tiles_x x tiles_y of them cut a plane evenly (w
+// and h differ by at most one between tiles), each of at most 512 sites (one
+// per thread) with at most 256 halo cells.  A block's time per plane hardly
+// depends on how full its tile is, so the fewest tiles win; of those the one
+// with the smallest halo ring, then the widest rows.
+static int cut(int n, int parts, int i) { return (int)((long long)i * n / parts); }
+static void plain_tiles(int n, int halo, int* tiles_x, int* tiles_y) {
+  constexpr int kSites = 512, kHalo = 256;
+  int best = 0, best_ring = 0;
+  for (int tx = 1; tx <= n; ++tx) {
+    const int w = (n + tx - 1) / tx;
+    if (w > kSites || (tx > 1 && w < 8)) continue;
+    int h = std::min(n, std::min(kSites / w, (kHalo - 4 * halo * halo) / (2 * halo) - w));
+    if (h < 1) continue;
+    const int ty = (n + h - 1) / h;
+    h = (n + ty - 1) / ty;
+    if (!best || tx * ty < best || (tx * ty == best && w + h < best_ring)) {
+      best = tx * ty;
+      best_ring = w + h;
+      *tiles_x = tx;
+      *tiles_y = ty;
+    }
+  }
 }
 
 // Persistent geometry and work assignment.  Tiles are 32 vx x 16 sites (vx
@@ -137,17 +166,21 @@ Layout sim_layout(const pycool_config& c) {
 // block processes its units in the order dealt.  (rc, rw) minimises the
 // busiest block's cost, then the total.
 PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
-                std::vector<int4>* units, std::vector<int>* off, int halo) {
+                std::vector<int4>* units, std::vector<int>* off, int halo, bool plain) {
   PGeo g;
   std::memset(&g, 0, sizeof(g));
   g.n = n;
   g.halo = halo;
-  g.vx = 1;
-  for (int v = 4; v >= 1; v /= 2)
-    if (v * nf * word <= 16 && n % (32 * v) == 0) { g.vx = v; break; }
-  g.tx = 32 * g.vx;
-  g.tiles_x = n / g.tx;
-  const int tiles_y = n / 16;
+  int tiles_y = n / 16;
+  if (plain) {
+    plain_tiles(n, halo, &g.tiles_x, &tiles_y);
+  } else {
+    g.vx = 1;
+    for (int v = 4; v >= 1; v /= 2)
+      if (v * nf * word <= 16 && n % (32 * v) == 0) { g.vx = v; break; }
+    g.tx = 32 * g.vx;
+    g.tiles_x = n / g.tx;
+  }
   g.ntiles = g.tiles_x * tiles_y;
   // Cost of a block's work, fitted to per-block timings of the persistent
   // kernel on GB300: a plane costs 1 (pen for the tiles at the y wrap, whose
@@ -159,7 +192,7 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
   const double stage_bytes = 4.0 * nf * (double)n * n * n * word;   // phi, pi read and written
   const bool l2_resident = l2_bytes > 0 && stage_bytes <= 0.75 * (double)l2_bytes;
   const double h = prec != PREC_SPLIT ? 0.25 : (l2_resident ? 1.5 : 0.3);
-  const double pen = prec != PREC_SPLIT ? 1.0 : 1.24;
+  const double pen = prec != PREC_SPLIT || plain ? 1.0 : 1.24;
   // Planes: no unit shorter than this is cut off a chunk.  A lattice of side 32 has
   // 64 (tile, plane) pairs, so single planes spread it over 64 SMs where pieces of
   // four left 16 at work: 32^3 per stage, FP64 chaotic 19.4 -> 10.7 us, split-FP32
@@ -277,16 +310,25 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
     for (int b = 0; b < G; ++b) (*off)[b + 1] += (*off)[b];
     units->assign(out.size(), int4{0, 0, 0, 0});
     std::vector<int> fill(off->begin(), off->end() - 1);
-    for (const U& u : out)   // per block, in the order dealt
-      (*units)[fill[u.b]++] =
-          int4{(u.t % g.tiles_x) * g.tx, (u.t / g.tiles_x) * 16, u.z0, u.z1 - u.z0 + 2 * halo};
+    for (const U& u : out) {   // per block, in the order dealt
+      const int ix = u.t % g.tiles_x, iy = u.t / g.tiles_x, planes = u.z1 - u.z0 + 2 * halo;
+      int4& w = (*units)[fill[u.b]++];
+      if (plain) {
+        const int x0 = cut(n, g.tiles_x, ix), y0 = cut(n, tiles_y, iy);
+        w = int4{x0 | (cut(n, g.tiles_x, ix + 1) - x0) << 16,
+                 y0 | (cut(n, tiles_y, iy + 1) - y0) << 16, u.z0, planes};
+      } else {
+        w = int4{ix * g.tx, iy * 16, u.z0, planes};
+      }
+    }
   }
   return g;
 }
 
 // A plan the kernel may trust: every unit inside the lattice, every (tile, z)
 // pair in exactly one unit, at most kMaxPUnits units per block.
-static bool check_plan(const PGeo& g, const std::vector<int4>& units, const std::vector<int>& off) {
+static bool check_plan(const PGeo& g, const std::vector<int4>& units, const std::vector<int>& off,
+                       bool plain = false) {
   if (g.G < 1 || g.G > kMaxPBlocks || (int)off.size() != g.G + 1 || off[0] != 0 ||
       off[g.G] != (int)units.size() || (int)units.size() != g.nunits)
     return false;
@@ -296,6 +338,22 @@ static bool check_plan(const PGeo& g, const std::vector<int4>& units, const std:
     for (int i = off[b]; i < off[b + 1]; ++i) {
       const int4 u = units[i];
       const int planes = u.w - 2 * g.halo;
+      if (plain) {
+        const int tiles_y = g.ntiles / g.tiles_x;
+        const int x0 = u.x & 0xffff, w = u.x >> 16, y0 = u.y & 0xffff, h = u.y >> 16;
+        int ix = 0, iy = 0;
+        while (ix < g.tiles_x && cut(g.n, g.tiles_x, ix) != x0) ++ix;
+        while (iy < tiles_y && cut(g.n, tiles_y, iy) != y0) ++iy;
+        if (ix == g.tiles_x || iy == tiles_y || w != cut(g.n, g.tiles_x, ix + 1) - x0 ||
+            h != cut(g.n, tiles_y, iy + 1) - y0 || w * h > 512 ||
+            2 * g.halo * (w + h + 2 * g.halo) > 256 || u.z < 0 || planes < 1 ||
+            u.z + planes > g.n)
+          return false;
+        const size_t t = (size_t)iy * g.tiles_x + ix;
+        for (int z = u.z; z < u.z + planes; ++z)
+          if (seen[t * g.n + z]++) return false;
+        continue;
+      }
       if (u.x < 0 || u.x % g.tx || u.x + g.tx > g.n || u.y < 0 || u.y % 16 || u.y + 16 > g.n ||
           u.z < 0 || planes < 1 || u.z + planes > g.n)
         return false;
@@ -529,6 +587,9 @@ cudaError_t encode_persist_maps(const SimDesc& d, const PGeo& g, PParams& p) {
 }
 
 cudaError_t launch_persist(const SimDesc& d, const PParams& p, int grid, cudaStream_t s, int* bps) {
+  if (p.g.vx == 0)   // plain staging
+    return d.prec == PREC_SPLIT ? launch_persist_split_plain(d.model, d.stencil, 0, p, grid, s, bps)
+                                : launch_persist_fp64_plain(d.model, d.stencil, 0, p, grid, s, bps);
   if (d.prec == PREC_SPLIT) return launch_persist_split(d.model, d.stencil, p.g.vx, p, grid, s, bps);
   if (d.stencil == 13)
     return d.prec == PREC_DD ? launch_persist_dd_wide(d.model, d.stencil, p.g.vx, p, grid, s, bps)
@@ -649,6 +710,13 @@ __global__ void split_load_kernel(const void* __restrict__ d, const double* base
 }
 
 
+__global__ void clear_barrier_kernel(unsigned long long* bar) { *bar = 0ull; }
+
+static cudaError_t launch_clear_barrier(unsigned long long* bar, cudaStream_t s) {
+  clear_barrier_kernel<<<1, 1, 0, s>>>(bar);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_arm(Background* bg, long long nsweeps, cudaStream_t s) {
   arm_kernel<<<1, 1, 0, s>>>(bg, nsweeps);
   return cudaGetLastError();
@@ -751,7 +819,9 @@ PYCOOL_API pycool_status pycool_debug_fail_alloc(int32_t count) {
 
 PYCOOL_API pycool_status pycool_debug_barrier_stall(pycool_sim* sim, int64_t wait_limit_clocks) {
   if (!sim || wait_limit_clocks <= 0) return PYCOOL_E_INVALID;
-  if (!sim->persist) return PYCOOL_E_STATE;   // only the persistent kernel has a grid barrier
+  // only the persistent kernel has a grid barrier (TMA staging: a plain-staging
+  // launch starts from a barrier count of its own, see pycool_evolve)
+  if (!sim->persist || sim->L.plain) return PYCOOL_E_STATE;
   sim->stall_limit = (long long)wait_limit_clocks;
   return PYCOOL_OK;
 }
@@ -828,14 +898,14 @@ pycool_status pycool::persist_setup(const pycool_config& cfg, const SimDesc& hd,
   std::vector<int4> units;
   std::vector<int> uoff;
   const PGeo g = plan_units(cfg.n, prec_word(hd.prec), model_nfields(cfg.model), hd.prec, sms,
-                            l2, &units, &uoff, hd.stencil == 13 ? 2 : 1);
+                            l2, &units, &uoff, hd.stencil == 13 ? 2 : 1, L.plain);
   std::memset(&p, 0, sizeof(p));
   p.g = g;
   int4* d_units = (int4*)(ws + L.off_punits);
   int* d_uoff = (int*)(ws + L.off_punits +
                        align256((size_t)kMaxPBlocks * kMaxPUnits * sizeof(int4)));
   if (units.size() > (size_t)kMaxPBlocks * kMaxPUnits || uoff.size() > (size_t)kMaxPBlocks + 1 ||
-      !check_plan(g, units, uoff))
+      !check_plan(g, units, uoff, L.plain))
     return PYCOOL_E_INVALID;
   PCK(cudaMemcpyAsync(d_units, units.data(), units.size() * sizeof(int4), cudaMemcpyHostToDevice,
                       st));
@@ -843,7 +913,7 @@ pycool_status pycool::persist_setup(const pycool_config& cfg, const SimDesc& hd,
   PCK(cudaStreamSynchronize(st));   // the host vectors go out of scope below
   p.units = d_units;
   p.uoff = d_uoff;
-  PCK(encode_persist_maps(hd, g, p));
+  if (!L.plain) PCK(encode_persist_maps(hd, g, p));
   p.d = (const SimDesc*)(state + L.off_desc);
   p.bg = (Background*)(state + L.off_bg);
   p.bar = (unsigned long long*)(ws + L.off_ticket + 64);
@@ -1095,6 +1165,14 @@ PYCOOL_API pycool_status pycool_evolve(pycool_sim* sim, int64_t steps) {
   if (steps == 0) return PYCOOL_OK;
   const long long nsweeps = (long long)steps * sim->nstages;
   if (sim->persist) {
+    if (sim->L.plain) {
+      // as for the per-stage kernels, a small launch arms each evolve: here it
+      // clears the grid barrier's count, so that the launch after it depends on
+      // no count kept by the host
+      CK(launch_clear_barrier(sim->pp.bar, sim->stream));
+      sim->launches += 1;
+      sim->pp.bar_base = 0;
+    }
     pycool_status st = launch_persist_sweeps(sim, nsweeps);
     if (st != PYCOOL_OK) return st;
     CK(cudaEventRecord(sim->done, sim->stream));

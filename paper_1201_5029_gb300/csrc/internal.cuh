@@ -159,6 +159,8 @@ constexpr int kMaxPUnits = 64;             // work units per block
 // for tiles clear of the periodic y boundary, rw for the tiles whose halo rows
 // cross it), the chunks dealt to the G blocks and cut where a block reaches
 // the common target (plan_units); each block reads its units from a table.
+// Plain staging (persist_plain.cuh; vx = 0): tiles_x x tiles_y tiles of w x h
+// sites, w and h equal to within one, w h <= 512.
 struct PGeo {
   int n, vx, tx, tiles_x, ntiles, rc, rw, nunits, G;
   int halo;   // z-halo planes (and halo rows) per side: 1, or 2 for the 13-point stencil
@@ -184,7 +186,8 @@ struct PParams {
   unsigned long long* bar;       // grid barrier: arrivals so far (monotonic)
   unsigned long long bar_base;   // arrivals before this launch
   void* rows;              // [2][G][kNQ] doubles (FP64) or float pairs (split)
-  const int4* units;       // every block's units in processing order: (x0, y0, z0, planes)
+  const int4* units;       // every block's units in processing order: (x0, y0, z0, planes);
+                           //    plain staging: (x0 | w << 16, y0 | h << 16, z0, planes)
   const int* uoff;         // block b's units are units[uoff[b] .. uoff[b + 1])
   int32_t* fault;
   PGeo g;
@@ -199,7 +202,8 @@ struct PParams {
 // The persistent geometry and its unit table (units grouped by block; off has
 // G + 1 entries).
 PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
-                std::vector<int4>* units, std::vector<int>* off, int halo = 1);
+                std::vector<int4>* units, std::vector<int>* off, int halo = 1,
+                bool plain = false);
 
 // Launchers (one translation unit per precision).
 cudaError_t launch_sweep_fp64(int model, int stencil, int vx, int tma, const LaunchTable& t, int grid,
@@ -213,6 +217,11 @@ cudaError_t launch_persist_split(int model, int stencil, int vx, const PParams& 
                                  cudaStream_t s, int* bps);
 cudaError_t launch_persist_dd(int model, int stencil, int vx, const PParams& p, int grid,
                               cudaStream_t s, int* bps);
+// plain staging, every stencil (FP64 and split-FP32)
+cudaError_t launch_persist_fp64_plain(int model, int stencil, int vx, const PParams& p, int grid,
+                                      cudaStream_t s, int* bps);
+cudaError_t launch_persist_split_plain(int model, int stencil, int vx, const PParams& p, int grid,
+                                       cudaStream_t s, int* bps);
 // the 13-point stencil's instances (FP64 and split-DD)
 cudaError_t launch_persist_fp64_wide(int model, int stencil, int vx, const PParams& p, int grid,
                                      cudaStream_t s, int* bps);

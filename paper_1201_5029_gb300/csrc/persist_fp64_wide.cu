@@ -1,5 +1,5 @@
 // FP64 instances of the persistent evolve kernel, 13-point stencil (every model).
-#include "persist.cuh"
+#include "persist_kernel.cuh"
 
 namespace pycool {
 cudaError_t launch_persist_fp64_wide(int model, int stencil, int vx, const PParams& p, int grid,

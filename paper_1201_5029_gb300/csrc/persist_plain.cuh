@@ -1,0 +1,372 @@
+// Staging of the persistent kernel without TMA: any lattice side (a TMA box
+// wants rows that are multiples of 16 bytes and tiles of whole boxes), and the
+// 13-point stencil of the split-FP32 form, whose five rows per site would not
+// fit the register pipeline of stage_split.
+//
+// A tile is w x h sites (w h <= 512, chosen by plan_plain so that as few tiles
+// as possible cover the lattice: tiles differ in w and h by at most one, and no
+// thread row is tied to a lattice row), one site per thread.  Each thread
+// copies its own site's values of the planes ahead, and at most one cell of the
+// tile's halo ring (periodic indices), with 4- or 8-byte cp.async into its own
+// places of a shared-memory ring; it alone reads them again, so a copy needs no
+// barrier, only the thread's own cp.async group count.  The thread drifts its
+// cells of plane g + 1 into one of four drift buffers (fixed point or float64 in
+// the FP64 form, float32 in the split form), its warp arrives on the buffer's
+// mbarrier, and after the wait for plane g it sums the stencil of plane g from
+// shared memory and puts out the plane H below, whose drifted field and momentum
+// it still holds in the ring.  As in the other stages there is no block barrier
+// in the z loop.
+//
+// Bound by: FP64, the float64 pipe; split-FP32, the shared-memory pipe and the
+// copies' latency (one site per thread).  Measured on GB300, per stage, against
+// the per-stage kernels (sweep_plain, sweep_wide: ragged 32 x 8 tiles in two
+// uneven waves of blocks, float64 stencils, a launch per stage): FP64 chaotic
+// 16^3 24.0 -> 10.3 us, 37^3 27.5 -> 12.0, 100^3 145 -> 46, with 27 points 209 ->
+// 50, with 13 points 238 -> 51, oscillon 203^3 434 -> 209; split-FP32 chaotic
+// 100^3 40.5 -> 19.9, oscillon 250^3 196 -> 145, 13 points 128^3 57.6 -> 35.1,
+// 256^3 Q-ball 359 -> 225.
+#pragma once
+
+#include "persist.cuh"
+
+namespace pycool {
+
+constexpr int kPlainHalo = 256;                       // halo cells of a tile at most
+constexpr int kPlainCells = kPThreads + kPlainHalo;   // cells of a tile with its halo
+
+// Shared memory: own[OSLOT][NF][phi, pi][512], halo[HSLOT][NF][phi, pi][256]
+// and the drift buffers fx[NDRIFT][NF][768].  LEAD planes of copies are in
+// flight ahead of the plane being drifted; an own slot is needed until the
+// plane has been put out, H + 1 planes after its drift.
+template <int PREC, int NF, int NQ, int H>
+struct PlainRing {
+  static constexpr int WORD = prec_word(PREC);
+  static constexpr int OSLOT = PREC == PREC_FP64 ? 6 : 8;
+  static constexpr int LEAD = OSLOT - H - 2;
+  static constexpr int HSLOT = LEAD + 1;
+  static constexpr int NDRIFT = 4;
+  static constexpr int NSLOT = 1;   // no TMA ring
+  static constexpr int FOLD = NQ + (PREC == PREC_FP64 ? 1 : 0);
+  static constexpr int PRE = 1;
+  static constexpr int OWN = NF * 2 * kPThreads, HALO = NF * 2 * kPlainHalo;
+  static constexpr int FX = NF * kPlainCells;
+  static constexpr int HALO_OFF = OSLOT * OWN, FX_OFF = HALO_OFF + HSLOT * HALO;
+  static constexpr int RING_BYTES = (FX_OFF + NDRIFT * FX) * WORD;
+  static constexpr int DRIFT_WORDS = 0;
+  static constexpr int KAHAN_BYTES = NQ * kKahanGroups * 8;
+  static constexpr int ROWS_BYTES = kMaxPBlocks * kNQ * 8;
+  static constexpr int EXTRA_BYTES =
+      PREC == PREC_FP64 ? NQ * kPThreads * 8
+                        : (KAHAN_BYTES > ROWS_BYTES ? KAHAN_BYTES : ROWS_BYTES);
+  static constexpr int SMEM_BYTES = RING_BYTES + EXTRA_BYTES;
+  static_assert(PREC != PREC_DD, "the FP64 and split-FP32 forms");
+  static_assert(SMEM_BYTES <= kPSmemBudget, "shared memory of the persistent kernel");
+  static_assert(RING_BYTES % 16 == 0, "the rows' bulk copy lands behind the ring");
+};
+
+// 8- and 4-byte asynchronous copies into the thread's own places.
+__device__ __forceinline__ void cp_async_word(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_word(float* dst, const float* src) { cp_async4(dst, src); }
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// A thread's cells of a unit (x0 | w << 16, y0 | h << 16, z0, planes): in-plane
+// offsets in the lattice (own, halo; -1: none) and in a drift buffer whose rows
+// are rs = w + 2 H cells.
+struct PlainCells {
+  int own, ownc, halo, haloc, rs;
+};
+template <int H>
+__device__ __forceinline__ PlainCells plain_cells(int4 u, int n) {
+  PlainCells c;
+  const int x0 = u.x & 0xffff, w = u.x >> 16, y0 = u.y & 0xffff, h = u.y >> 16;
+  const int t = threadIdx.x;
+  c.rs = w + 2 * H;
+  c.own = c.halo = -1;
+  c.ownc = H * c.rs + H;   // a thread without a site reads the first one's neighbours
+  c.haloc = 0;
+  if (t < w * h) {
+    const int ly = t / w, lx = t - ly * w;
+    c.own = (y0 + ly) * n + x0 + lx;
+    c.ownc = (ly + H) * c.rs + lx + H;
+  }
+  if (t < 2 * H * (c.rs + h)) {   // 2H full rows, then 2H cells beside each of the h rows
+    int row, col;
+    if (t < 2 * H * c.rs) {
+      const int r = t / c.rs;
+      col = t - r * c.rs;
+      row = r < H ? r : h + r;
+    } else {
+      const int t2 = t - 2 * H * c.rs, k = t2 % (2 * H);
+      row = t2 / (2 * H) + H;
+      col = k < H ? k : w + k;
+    }
+    c.halo = wrapi(y0 - H + row, n) * n + wrapi(x0 - H + col, n);
+    c.haloc = row * c.rs + col;
+  }
+  return c;
+}
+
+// A position in the block's planes and the thread's cells there.
+template <int H>
+struct PlainPos {
+  int ui, uq;
+  PlainCells c;
+  __device__ __forceinline__ void start(const PShared& sm, int n) {
+    ui = uq = 0;
+    if (sm.nunits > 0) c = plain_cells<H>(sm.units[0], n);
+  }
+  __device__ __forceinline__ bool in(const PShared& sm) const { return ui < sm.nunits; }
+  __device__ __forceinline__ void next(const PShared& sm, int n) {
+    if (++uq == sm.units[ui].w) {
+      uq = 0;
+      if (++ui < sm.nunits) c = plain_cells<H>(sm.units[ui], n);
+    }
+  }
+};
+
+// Copies of the plane at `pos` (ring plane gp) and one commit, always: the
+// groups a thread has committed count the planes.
+template <int MODEL, int PREC, int NQ, int H>
+__device__ __forceinline__ void plain_issue(const PParams& p, const PShared& sm, PlainPos<H>& pos,
+                                            int ib, uint32_t gp) {
+  constexpr int NF = Pot<MODEL>::NF;
+  using T = typename WorkT<PREC>::type;
+  using RG = PlainRing<PREC, NF, NQ, H>;
+  if (pos.in(sm)) {
+    const SimDesc& d = *sm.d;
+    const int n = p.g.n;
+    const size_t S = (size_t)d.S;
+    const int z = wrapi(sm.units[pos.ui].z - H + pos.uq, n);
+    const T* src[2] = {(const T*)d.phi[ib & 1] + (size_t)z * n * n,
+                       (const T*)d.pi[(ib >> 1) & 1] + (size_t)z * n * n};
+    T* own = (T*)sm.ring + (gp % RG::OSLOT) * RG::OWN + threadIdx.x;
+    T* hal = (T*)sm.ring + RG::HALO_OFF + (gp % RG::HSLOT) * RG::HALO + threadIdx.x;
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int arr = 0; arr < 2; ++arr) {
+        if (pos.c.own >= 0)
+          cp_async_word(own + (f * 2 + arr) * kPThreads, src[arr] + f * S + pos.c.own);
+        if (pos.c.halo >= 0)
+          cp_async_word(hal + (f * 2 + arr) * kPlainHalo, src[arr] + f * S + pos.c.halo);
+      }
+    pos.next(sm, n);
+  }
+  cp_async_commit();
+}
+
+// The first LEAD planes of a stage (every thread of the block).
+template <int MODEL, int PREC, int NQ, int H>
+__device__ __forceinline__ void plain_prefetch(const PParams& p, const PShared& sm, int ib,
+                                               uint32_t gq) {
+  using RG = PlainRing<PREC, Pot<MODEL>::NF, NQ, H>;
+  PlainPos<H> pos;
+  pos.start(sm, p.g.n);
+  for (int l = 0; l < RG::LEAD; ++l) plain_issue<MODEL, PREC, NQ, H>(p, sm, pos, ib, gq + l);
+}
+
+__device__ __forceinline__ float fix_in(float v, int, float*) { return v; }
+__device__ __forceinline__ float fix_out(float v, int) { return v; }
+__device__ __forceinline__ float fix_mad(float a, float b, float c) { return madd(a, b, c); }
+__device__ __forceinline__ float fix_mid7(float c, float faces) { return madd(-6.0f, c, faces); }
+__device__ __forceinline__ void fix_parts27(float c, float faces, float corners, float& mid,
+                                            float& off) {
+  mid = madd((float)(3.0 / 30.0), corners,
+             madd((float)(14.0 / 30.0), faces, (float)(-128.0 / 30.0) * c));
+  off = madd((float)(1.0 / 30.0), corners,
+             madd((float)(3.0 / 30.0), faces, (float)(14.0 / 30.0) * c));
+}
+
+// One stage over this block's units (see the head of this file); the sums go to
+// accd (FP64) or the block's compensated sums (split-FP32, as stage_split).
+template <int MODEL, int STENCIL, int PREC, int MODE, bool FIX>
+__device__ __forceinline__ bool stage_plain(const PParams& p, const Ctx<MODEL, PREC>& cx0,
+                                            const PShared& sm, uint32_t gq, int ib, double* accd,
+                                            HiMax<Pot<MODEL>::NF>& hm) {
+  using C = Ctx<MODEL, PREC>;
+  using T = typename C::T;
+  constexpr bool F64 = PREC == PREC_FP64;
+  using E = typename std::conditional<F64, typename FixElem<FIX>::type, float>::type;
+  using SL = typename C::SL;
+  constexpr int NF = C::NF, NQ = SL::NQ, H = halo_of<STENCIL>();
+  constexpr bool CORNERS = StencilW<STENCIL>::kCorners;
+  constexpr bool WIDE = STENCIL == 13;
+  using RG = PlainRing<PREC, NF, NQ, H>;
+  constexpr int NB = RG::NDRIFT, LEAD = RG::LEAD;
+  constexpr int KGROUP = 8;   // split: output planes per float partial before a compensated add
+  const SimDesc& d = *sm.d;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int n = p.g.n;
+  const size_t S = (size_t)d.S, nn = (size_t)n * n;
+  T* __restrict__ phi_out = (T*)d.phi[(ib & 1) ^ 1];
+  T* __restrict__ pi_out = (T*)d.pi[((ib >> 1) & 1) ^ 1];
+  T* const own = (T*)sm.ring + tid;
+  const T* const hal = (const T*)sm.ring + RG::HALO_OFF + tid;
+  E* const fxb = (E*)((T*)sm.ring + RG::FX_OFF);
+  // FP64: integer sums (or, 13 points, all sums) are D times the weights' common
+  // denominator, which goes into the kick's coefficient and, after the stage,
+  // into sum phi D; split: the weights themselves
+  constexpr bool TIMES = F64 && (WIDE || (FIX && STENCIL == 27));
+  C cx = cx0;
+  if constexpr (TIMES) cx.kD *= 1.0 / fix_weight<STENCIL>();
+  const E w1 = TIMES ? (E)16 : (E)(16.0 / 12.0);
+  const E w2 = TIMES ? (E)0 - (E)1 : (E)(-1.0 / 12.0);
+  const E w0 = TIMES ? (E)0 - (E)90 : (E)(-90.0 / 12.0);
+  T Mf[NF];   // split: the re-centring of the drifted field (the stencil works on phi + c pi)
+  float ps[F64 ? 1 : NQ];
+  if constexpr (!F64) {
+#pragma unroll
+    for (int f = 0; f < NF; ++f) Mf[f] = madd(cx.cdrift, cx.mu_pi[f], cx.mu_phi[f]);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {   // each group's lead lane owns its sums
+      if ((tid & 3) == 0) sm.kahan[i * kKahanGroups + (tid >> 2)] = make_float2(0.f, 0.f);
+      ps[i] = 0.f;
+    }
+  }
+  int kg = 0;
+  bool ok = true;
+
+  PlainPos<H> ip, dp;   // next plane to copy, next plane to drift
+  ip.start(sm, n);
+  for (int l = 0; l < LEAD && ip.in(sm); ++l) ip.next(sm, n);
+  dp.start(sm, n);
+  // drift of the plane at dp (ring plane gg): own cell in place and into the
+  // drift buffer, the halo cell into the drift buffer
+  auto drift = [&](uint32_t gg) {
+    T* o = own + (gg % RG::OSLOT) * RG::OWN;
+    const T* h = hal + (gg % RG::HSLOT) * RG::HALO;
+    E* fx = fxb + (gg % NB) * RG::FX;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const int ex = F64 ? cx.fx[f] : 0;
+      if (dp.c.own >= 0) {
+        const T a = madd(cx.cdrift, o[(f * 2 + 1) * kPThreads], o[f * 2 * kPThreads]);
+        o[f * 2 * kPThreads] = a;
+        fx[f * kPlainCells + dp.c.ownc] = fix_in(a, ex, (E*)nullptr);
+      }
+      if (dp.c.halo >= 0) {
+        const T a = madd(cx.cdrift, h[(f * 2 + 1) * kPlainHalo], h[f * 2 * kPlainHalo]);
+        fx[f * kPlainCells + dp.c.haloc] = fix_in(a, ex, (E*)nullptr);
+      }
+    }
+    __syncwarp();   // the lanes' writes before lane 0's arrival (release)
+    if (lane == 0) mbar_arrive(&sm.dbar[gg % NB]);
+    dp.next(sm, n);
+  };
+
+  uint32_t g = gq;
+  if (sm.nunits > 0) {
+    plain_issue<MODEL, PREC, NQ, H>(p, sm, ip, ib, g + LEAD);
+    cp_async_wait<LEAD>();
+    drift(g);
+  }
+  for (int i = 0; i < sm.nunits && ok; ++i) {
+    const int4 u = sm.units[i];
+    const int Q = u.w;
+    const PlainCells c = plain_cells<H>(u, n);
+    const bool valid = c.own >= 0;
+    // 7- and 27-point: part_m, so_m as in stage_fp64; 13-point: the z queue of stage_fp64_wide
+    E qa[NF], qb[NF], qc[NF], qd[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) qa[f] = qb[f] = qc[f] = qd[f] = (E)0;
+    for (int q = 0; q < Q; ++q, ++g) {
+      plain_issue<MODEL, PREC, NQ, H>(p, sm, ip, ib, g + 1 + LEAD);
+      if (dp.in(sm)) {
+        cp_async_wait<LEAD>();
+        drift(g + 1);
+      }
+      // every warp has drifted plane g
+      ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit);
+      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      const bool mid = q >= H && q < Q - H;   // a plane whose sites are output
+      E D[NF];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        const E* fx = fxb + (g % NB) * RG::FX + f * kPlainCells + c.ownc;
+        const int rs = c.rs;
+        const E ctr = fx[0];
+        if constexpr (WIDE) {
+          E m = (E)0;
+          if (mid) {
+            const E nr = (fx[-rs] + fx[rs]) + (fx[-1] + fx[1]);
+            const E fr = (fx[-2 * rs] + fx[2 * rs]) + (fx[-2] + fx[2]);
+            m = fix_mad(w0, ctr, fix_mad(w2, fr, w1 * nr));
+          }
+          D[f] = fix_mad(w2, ctr, qb[f]);   // plane p - 2: its last term
+          const E np1 = fix_mad(w1, ctr, qa[f]);
+          qa[f] = fix_mad(w2, qd[f], fix_mad(w1, qc[f], m));
+          qb[f] = np1;
+          qd[f] = qc[f];
+          qc[f] = ctr;
+        } else {
+          E smid = ctr, so = ctr;
+          if (CORNERS || mid) {
+            const E faces = (fx[-rs] + fx[rs]) + (fx[-1] + fx[1]);
+            if constexpr (CORNERS)
+              fix_parts27(ctr, faces, (fx[-rs - 1] + fx[-rs + 1]) + (fx[rs - 1] + fx[rs + 1]),
+                          smid, so);
+            else
+              smid = fix_mid7(ctr, faces);
+          }
+          D[f] = qa[f] + so;
+          if (mid) qa[f] = qb[f] + smid;
+          qb[f] = so;
+        }
+      }
+      if (q >= 2 * H) {  // output plane z0 + q - 2 H
+        if (valid) {
+          const size_t o = (size_t)(u.z + q - 2 * H) * nn + c.own;
+          T phj[NF], Dj[NF], pmj[NF], pnj[NF];
+          const T* r = own + ((g - H) % RG::OSLOT) * RG::OWN;
+#pragma unroll
+          for (int f = 0; f < NF; ++f) {
+            phj[f] = r[f * 2 * kPThreads];
+            pmj[f] = r[(f * 2 + 1) * kPThreads];
+            Dj[f] = fix_out(D[f], F64 ? cx.fx[f] : 0);
+            if constexpr (!F64) {
+              phj[f] -= Mf[f];
+              pmj[f] -= cx.mu_pi[f];
+            }
+          }
+          if constexpr (F64) {
+            cx.site(MODE, phj, Dj, pmj, pnj, accd);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+              hm.add(2 * f, phj[f]);
+              hm.add(2 * f + 1, pnj[f]);
+            }
+          } else {
+            cx.site(MODE, phj, Dj, pmj, pnj, ps);
+          }
+#pragma unroll
+          for (int f = 0; f < NF; ++f) {
+            __stwb(phi_out + f * S + o, phj[f]);
+            if (MODE == MODE_SWEEP) __stwb(pi_out + f * S + o, pnj[f]);
+          }
+        }
+        if constexpr (!F64) {
+          if (++kg == KGROUP) {
+            kg = 0;
+            kahan_flush<NQ>(sm.kahan, ps);
+          }
+        }
+      }
+    }
+  }
+  if constexpr (!F64) kahan_flush<NQ>(sm.kahan, ps);
+  if constexpr (TIMES) {
+#pragma unroll
+    for (int f = 0; f < NF; ++f) accd[SL::PHID + f] *= 1.0 / fix_weight<STENCIL>();
+  }
+  return ok;
+}
+
+}  // namespace pycool

@@ -1,5 +1,5 @@
 // Split-FP32 instances of the persistent evolve kernel (every model x stencil).
-#include "persist.cuh"
+#include "persist_kernel.cuh"
 
 namespace pycool {
 cudaError_t launch_persist_split(int model, int stencil, int vx, const PParams& p, int grid,

@@ -27,6 +27,7 @@ struct Layout {
   size_t off_bg, off_desc, off_fields, state_bytes;
   size_t off_ticket, off_gticket, off_partials, off_gpartials, ws_bytes;
   size_t off_prows;   // single-simulation API: rows of the persistent kernel (0 = none)
+  bool plain;         // the persistent kernel's plain staging (any n; off_prows != 0)
   size_t off_punits;  // single-simulation API: the persistent kernel's unit table
   size_t off_rt;      // runtime potentials: drifted fields, V', V (0 = none)
   size_t off_mean;    // single-simulation API: partial sums of the split forms' initial means

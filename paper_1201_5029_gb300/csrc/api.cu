@@ -790,8 +790,11 @@ struct pycool_sim {
   cufftHandle spec_plan = 0;
   double* spec_tmp = nullptr;       // n^3 float64 field
   void* spec_out = nullptr;         // n n (n/2 + 1) complex coefficients
-  int32_t* spec_order = nullptr;    // half-spectrum modes grouped by shell
-  int32_t* spec_start = nullptr;    // shell b: spec_order[spec_start[b] .. spec_start[b + 1])
+  uint32_t* spec_order = nullptr;   // half-spectrum modes grouped by shell (launch_spectrum_bins)
+  int32_t* spec_cut = nullptr;      // chunk c: spec_order[spec_cut[c] .. spec_cut[c + 1])
+  int32_t* spec_first = nullptr;    // shell b: chunks spec_first[b] .. spec_first[b + 1]
+  double* spec_part = nullptr;      // per chunk
+  int spec_chunks = 0;
   double* spec_power = nullptr;     // per shell
   std::vector<int64_t> spec_count;  // modes per shell over the full spectrum
 };
@@ -1405,33 +1408,56 @@ PYCOOL_API pycool_status pycool_energy_fields(pycool_sim* sim, double* rho, doub
 static pycool_status spectrum_setup(pycool_sim* sim) {
   const int n = sim->cfg.n, nh = n / 2 + 1, nb = pycool_spectrum_bins(n);
   const size_t half = (size_t)n * n * nh;
-  std::vector<int32_t> shell(half), start(nb + 1, 0), order(half);
+  std::vector<int32_t> start(nb + 1, 0);
+  std::vector<uint32_t> order(half);
   sim->spec_count.assign(nb, 0);
-  for (int z = 0; z < n; ++z)
-    for (int y = 0; y < n; ++y)
-      for (int x = 0; x < nh; ++x) {
-        const long long mz = z <= n / 2 ? z : z - n, my = y <= n / 2 ? y : y - n;
-        const long long r2 = mz * mz + my * my + (long long)x * x;
-        const int b = (int)std::lround(std::sqrt((double)r2));
-        const size_t m = ((size_t)z * n + y) * nh + x;
-        shell[m] = b;
-        start[b + 1] += 1;
-        sim->spec_count[b] += (x > 0 && 2 * x != n) ? 2 : 1;
+  // shell of a squared length, and every mode in ascending index
+  std::vector<int32_t> shell_of(3 * (size_t)(n / 2) * (n / 2) + 1);
+  for (size_t r2 = 0; r2 < shell_of.size(); ++r2)
+    shell_of[r2] = (int32_t)std::lround(std::sqrt((double)r2));
+  auto each_mode = [&](auto&& visit) {
+    size_t m = 0;
+    for (int z = 0; z < n; ++z)
+      for (int y = 0; y < n; ++y) {
+        const int mz = z <= n / 2 ? z : z - n, my = y <= n / 2 ? y : y - n;
+        const int32_t* row = &shell_of[0];
+        const int r2 = mz * mz + my * my;
+        for (int x = 0; x < nh; ++x, ++m) visit((uint32_t)m, row[r2 + x * x], x > 0 && 2 * x != n);
       }
+  };
+  each_mode([&](uint32_t, int b, bool twice) {
+    start[b + 1] += 1;
+    sim->spec_count[b] += twice ? 2 : 1;
+  });
   for (int b = 0; b < nb; ++b) start[b + 1] += start[b];
   std::vector<int32_t> fill(start.begin(), start.end() - 1);
-  for (size_t m = 0; m < half; ++m) order[fill[shell[m]]++] = (int32_t)m;
+  each_mode([&](uint32_t m, int b, bool twice) {
+    order[fill[b]++] = m | (twice ? 0u : 0x80000000u);
+  });
+  // chunks of at most 2048 modes of one shell (eight per thread of a block)
+  std::vector<int32_t> cut, first(nb + 1);
+  for (int b = 0; b < nb; ++b) {
+    first[b] = (int32_t)cut.size();
+    for (int j = start[b]; j < start[b + 1]; j += 2048) cut.push_back(j);
+  }
+  sim->spec_chunks = (int)cut.size();
+  first[nb] = sim->spec_chunks;
+  cut.push_back(start[nb]);
   if (injected_alloc_failure() ||
       cudaMalloc((void**)&sim->spec_tmp, (size_t)sim->hdesc.S * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&sim->spec_out, half * sizeof(cufftDoubleComplex)) != cudaSuccess ||
-      cudaMalloc((void**)&sim->spec_order, half * sizeof(int32_t)) != cudaSuccess ||
-      cudaMalloc((void**)&sim->spec_start, (nb + 1) * sizeof(int32_t)) != cudaSuccess ||
+      cudaMalloc((void**)&sim->spec_order, half * sizeof(uint32_t)) != cudaSuccess ||
+      cudaMalloc((void**)&sim->spec_cut, cut.size() * sizeof(int32_t)) != cudaSuccess ||
+      cudaMalloc((void**)&sim->spec_first, (nb + 1) * sizeof(int32_t)) != cudaSuccess ||
+      cudaMalloc((void**)&sim->spec_part, cut.size() * sizeof(double)) != cudaSuccess ||
       cudaMalloc((void**)&sim->spec_power, nb * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     return PYCOOL_E_NOMEM;
   }
-  CK(cudaMemcpy(sim->spec_order, order.data(), half * sizeof(int32_t), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(sim->spec_start, start.data(), (nb + 1) * sizeof(int32_t), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(sim->spec_order, order.data(), half * sizeof(uint32_t), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(sim->spec_cut, cut.data(), cut.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(sim->spec_first, first.data(), (nb + 1) * sizeof(int32_t),
+                cudaMemcpyHostToDevice));
   if (cufftPlan3d(&sim->spec_plan, n, n, n, CUFFT_D2Z) != CUFFT_SUCCESS) return PYCOOL_E_CUDA;
   sim->spec_ready = true;
   return PYCOOL_OK;
@@ -1451,11 +1477,22 @@ PYCOOL_API pycool_status pycool_spectrum(pycool_sim* sim, int32_t which, int32_t
     if (st != PYCOOL_OK) return st;
   }
   if (cufftSetStream(sim->spec_plan, sim->stream) != CUFFT_SUCCESS) return PYCOOL_E_CUDA;
-  CK(launch_field_values(sim->hdesc, b, which, field, sim->spec_tmp, sim->stream));
-  if (cufftExecD2Z(sim->spec_plan, sim->spec_tmp, (cufftDoubleComplex*)sim->spec_out) !=
-      CUFFT_SUCCESS)
+  // an out-of-place forward transform leaves its input alone, so the FP64 form's
+  // field is transformed where it lies, if it starts on a 16-byte boundary
+  const double* field_values =
+      (const double*)(which == 0 ? sim->hdesc.phi[b.cur & 1] : sim->hdesc.pi[(b.cur >> 1) & 1]) +
+      (sim->hdesc.prec == PREC_FP64 ? (size_t)field * sim->hdesc.S : 0);
+  const bool direct = sim->hdesc.prec == PREC_FP64 && ((uintptr_t)field_values & 15) == 0;
+  if (!direct) {
+    CK(launch_field_values(sim->hdesc, b, which, field, sim->spec_tmp, sim->stream));
+    field_values = sim->spec_tmp;
+    sim->launches += 1;
+  }
+  if (cufftExecD2Z(sim->spec_plan, const_cast<double*>(field_values),
+                   (cufftDoubleComplex*)sim->spec_out) != CUFFT_SUCCESS)
     return PYCOOL_E_CUDA;
-  CK(launch_spectrum_bins(sim->spec_out, sim->cfg.n, sim->spec_order, sim->spec_start, nbins,
+  CK(launch_spectrum_bins(sim->spec_out, sim->cfg.n, sim->spec_order, sim->spec_cut,
+                          sim->spec_chunks, sim->spec_first, nbins, sim->spec_part,
                           sim->spec_power, sim->stream));
   CK(cudaMemcpyAsync(power, sim->spec_power, nbins * sizeof(double), cudaMemcpyDeviceToHost,
                      sim->stream));
@@ -1485,7 +1522,9 @@ PYCOOL_API void pycool_destroy(pycool_sim* sim) {
   cudaFree(sim->spec_tmp);
   cudaFree(sim->spec_out);
   cudaFree(sim->spec_order);
-  cudaFree(sim->spec_start);
+  cudaFree(sim->spec_cut);
+  cudaFree(sim->spec_first);
+  cudaFree(sim->spec_part);
   cudaFree(sim->spec_power);
   if (sim->graph) cudaGraphExecDestroy(sim->graph);
   if (sim->done) cudaEventDestroy(sim->done);

@@ -30,6 +30,18 @@ constexpr int kRuntimeModelMax = 64;          // such potentials per process
 constexpr long long kWaitLimit = 1ll << 31;   // default limit of a device-side wait
                                               // (SM clocks, about a second)
 
+#ifdef __CUDACC__
+// (double)v and (float)v by integer instructions where v is normal or zero: the
+// conversions between float32 and float64 run at the float64 rate on GB300, 1/64
+// of an integer instruction's.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = (uint32_t)__float_as_int(v), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)   // normal
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(m << 29));
+  return m == 0u ? __hiloint2double((int)b, 0) : (double)v;
+}
+#endif
+
 enum Mode : int32_t { MODE_IDLE = 0, MODE_SWEEP = 1, MODE_FLUSH = 2 };
 // PREC_DD: the split form with double-float fluctuations (float pairs, 8 bytes
 // per value) -- float64-class accuracy, arithmetic on the FP32 pipe.

@@ -60,8 +60,9 @@ cudaError_t launch_energy_fields(const SimDesc& d, const Background& b, double* 
                                  cudaStream_t s);
 cudaError_t launch_field_values(const SimDesc& d, const Background& b, int which, int f,
                                 double* out, cudaStream_t s);
-cudaError_t launch_spectrum_bins(const void* spec, int n, const int32_t* order,
-                                 const int32_t* start, int nbins, double* power, cudaStream_t s);
+cudaError_t launch_spectrum_bins(const void* spec, int n, const uint32_t* order,
+                                 const int32_t* cut, int nchunks, const int32_t* first, int nbins,
+                                 double* part, double* power, cudaStream_t s);
 // Fault injection (pycool_debug_fail_alloc): true if this device allocation
 // is to report failure (consumes one of the requested failures).
 bool injected_alloc_failure();

@@ -149,7 +149,10 @@ inline Geometry choose_geometry(int n, int word, int nf, bool plain = false) {
   g.tiles_y = (n + g.ty - 1) / g.ty;
   const int tiles = g.tiles_x * g.tiles_y;
   const int target = 2 * 152;           // two blocks per SM on 152 SMs
-  const int min_zc = n >= 128 ? 16 : 4;  // bound the z-halo re-read overhead
+  // bound the z-halo overhead: a halo plane is re-read, and in the FP64 form only
+  // drifted (2 of 17 float64 instructions), so that small FP64 lattices, whose
+  // blocks would leave most SMs idle, are cut into shorter chunks
+  const int min_zc = n >= 128 ? 16 : (n > 48 || word == 4 ? 4 : 2);
   int zc = 64;
   while (zc > min_zc && (long long)tiles * ((n + zc - 1) / zc) < target) zc /= 2;
   if (zc > n) zc = n;

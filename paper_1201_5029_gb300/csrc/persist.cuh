@@ -451,103 +451,8 @@ __device__ __forceinline__ bool drift_dd(const Ctx<MODEL, PREC_DD>& cx, const PS
 }
 
 // ---------------------------------------------------------------------------
-// FP64 form.
-//
-// GB300 executes two float64 lanes per SM and clock (a warp instruction takes
-// 64 cycles of a scheduler's pipe), and 64-bit conversions run at the same
-// rate, while integer adds, shifts and logic run 16 to 32 times faster.  The
-// discrete Laplacian is a sum with small integer weights, so it is taken off
-// the float64 pipe: each drifted field value is put on a 64-bit fixed-point
-// scale once (to_fixed, integer instructions only), D is summed exactly in
-// integers, and one normalisation (from_fixed, integer instructions) gives D
-// rounded once to float64.  The scale comes from the largest |phi| and |pi| of
-// the stage's input (Ctx::set_fix; the stages track them), so no sum can
-// overflow; a field value within 2^6 (27- and 13-point stencils: 2^2) of the
-// largest keeps every bit, and a smaller one is cut at 2^-58 (2^-54) of the
-// largest or less, below the rounding of the float64 sums it replaces.  A stage whose
-// input has no usable maximum (the first pass over a new state, values out of
-// range or not finite) sums in float64 (FIX = false).
-// Measured on GB300, against the same kernels with float64 stencils (set_initial,
-// evolve and get_fields together): 256^3 Q-ball, order 8, two steps 38.6 -> 25.2
-// ms; 256^3 oscillon, order 6, three steps 13.3 -> 8.9 ms; 128^3 preheating,
-// order 4, ten steps 4.49 -> 2.83 ms, with the 13-point stencil 6.78 -> 3.40 ms.
+// FP64 form (its fixed-point stencil: sweep.cuh).
 // ---------------------------------------------------------------------------
-// bits of |D| above the largest |I|: sum of the absolute weights, 12 (7-point),
-// 256 (27-point, weights times 30), 192 (13-point, times 12)
-template <int STENCIL> constexpr int fix_headroom() { return STENCIL == 7 ? 4 : 8; }
-// what the integer sums are times D
-template <int STENCIL> constexpr double fix_weight() {
-  return STENCIL == 7 ? 1.0 : (STENCIL == 27 ? 30.0 : 12.0);
-}
-
-// trunc(v 2^(1086 - E)) for |v| < 2^(E - 1023): the significand, bit 63 down,
-// shifted right by E - e (shr clamps: values below the scale, and zero, give 0).
-__device__ __forceinline__ unsigned long long to_fixed(double v, int E) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int hi = __double2hiint(v);
-  const int sh = E - ((hi >> 20) & 0x7ff);
-  unsigned long long m = (b << 11) | 0x8000000000000000ull;
-  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));
-  return hi < 0 ? 0ull - m : m;
-}
-// x 2^(E - 1086), rounded to nearest (a tie away from zero)
-__device__ __forceinline__ double from_fixed(unsigned long long x, int E) {
-  const bool neg = (long long)x < 0;
-  unsigned long long m = neg ? 0ull - x : x;
-  const int lz = __clzll((long long)m);
-  asm("shl.b64 %0, %0, %1;" : "+l"(m) : "r"(lz));
-  unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);
-  r += (unsigned long long)(uint32_t)(E - lz - 1) << 52;
-  r |= neg ? 0x8000000000000000ull : 0ull;
-  return __longlong_as_double((long long)(m == 0ull ? 0ull : r));
-}
-
-template <bool FIX> struct FixElem { using type = double; };
-template <> struct FixElem<true> { using type = unsigned long long; };
-__device__ __forceinline__ double fix_in(double v, int, double*) { return v; }
-__device__ __forceinline__ unsigned long long fix_in(double v, int E, unsigned long long*) {
-  return to_fixed(v, E);
-}
-__device__ __forceinline__ double fix_out(double v, int) { return v; }
-__device__ __forceinline__ double fix_out(unsigned long long v, int E) { return from_fixed(v, E); }
-
-__device__ __forceinline__ double fix_mad(double a, double b, double c) { return madd(a, b, c); }
-__device__ __forceinline__ unsigned long long fix_mad(unsigned long long a, unsigned long long b,
-                                                      unsigned long long c) {
-  return a * b + c;
-}
-// In-plane parts of the stencil (Eq. D split by z-offset, as plane_parts):
-// float64 with the weights themselves, integers with the weights times 30
-// (27-point) or as they are (7-point).
-__device__ __forceinline__ double fix_mid7(double c, double faces) { return madd(-6.0, c, faces); }
-__device__ __forceinline__ unsigned long long fix_mid7(unsigned long long c,
-                                                       unsigned long long faces) {
-  return faces - 6ull * c;
-}
-__device__ __forceinline__ void fix_parts27(double c, double faces, double corners, double& mid,
-                                            double& off) {
-  mid = madd(3.0 / 30.0, corners, madd(14.0 / 30.0, faces, (-128.0 / 30.0) * c));
-  off = madd(1.0 / 30.0, corners, madd(3.0 / 30.0, faces, (14.0 / 30.0) * c));
-}
-__device__ __forceinline__ void fix_parts27(unsigned long long c, unsigned long long faces,
-                                            unsigned long long corners, unsigned long long& mid,
-                                            unsigned long long& off) {
-  mid = 14ull * faces + 3ull * corners - (c << 7);
-  off = 14ull * c + 3ull * faces + corners;
-}
-
-// High words of the largest magnitudes a thread has put out, per field (phi, pi).
-template <int NF> struct HiMax {
-  uint32_t v[2 * NF];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int i = 0; i < 2 * NF; ++i) v[i] = 0u;
-  }
-  __device__ __forceinline__ void add(int i, double x) {
-    v[i] = max(v[i], (uint32_t)__double2hiint(x) & 0x7fffffffu);
-  }
-};
-
 // Drift of ring plane gg (of unit uu) into drift buffer gg % NDRIFT, then this
 // warp's arrival on the buffer's mbarrier (see drift_dd).
 template <int MODEL, int STENCIL, int VX, bool FIX>

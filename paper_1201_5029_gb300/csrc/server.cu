@@ -77,40 +77,51 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
   return c;
 }
 
-// Standard normal `comp` (0..3) of counter block `blk` of array `arr`:
-// u = (x + 1/2) 2^-32 in (0, 1); Box-Muller on (u0, u1) -> comps 0, 1 and on
-// (u2, u3) -> comps 2, 3 (cos for even, sin for odd).
-__device__ __forceinline__ double normal_at(uint64_t seed, uint32_t arr, uint32_t blk, int comp) {
+// The four standard normals of counter block `blk` of array `arr`:
+// u = (x + 1/2) 2^-32 in (0, 1); Box-Muller on (u0, u1) -> z[0], z[1] and on
+// (u2, u3) -> z[2], z[3] (cos, sin).
+__device__ __forceinline__ void normals_at(uint64_t seed, uint32_t arr, uint32_t blk, double* z) {
   const uint4 r = philox4x32_10(make_uint4(blk, arr, 0u, 0u),
                                 make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
   const double s = 2.3283064365386963e-10;  // 2^-32
-  const uint32_t a = comp < 2 ? r.x : r.z, b = comp < 2 ? r.y : r.w;
-  const double u1 = ((double)a + 0.5) * s, u2 = ((double)b + 0.5) * s;
-  const double rad = sqrt(-2.0 * log(u1));
-  const double th = 6.283185307179586 * u2;
-  return (comp & 1) ? rad * sin(th) : rad * cos(th);
+  const uint32_t a[2] = {r.x, r.z}, b[2] = {r.y, r.w};
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const double u1 = ((double)a[p] + 0.5) * s, u2 = ((double)b[p] + 0.5) * s;
+    const double rad = sqrt(-2.0 * log(u1));
+    double sn, cs;
+    sincos(6.283185307179586 * u2, &sn, &cs);
+    z[2 * p] = rad * cs;
+    z[2 * p + 1] = rad * sn;
+  }
 }
 
 // White-noise initial conditions into buffer 0.  Element e of field f uses
 // normal (e mod 4) of counter block e/4 of array f (phi) or N_f + f (pi):
 //   FP64 : phi_f = bg_f + noise z,  pi_f = mom_f + noise z
 //   split: the fluctuations noise z in float32 (bg, mom are the background)
+// A thread makes a block's four normals, so that the two of a Box-Muller pair
+// share the logarithm, the root and the argument's reduction (float64
+// instructions are what this kernel spends its time on).
 __global__ void ic_white_kernel(void* phi, void* pi, long long S, int nf, int split, double bg0,
                                 double bg1, double mom0, double mom1, double noise,
                                 unsigned long long seed) {
-  const long long total = S * nf;
+  const long long nb = (S + 3) / 4, total = nb * 2 * nf;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const int f = (int)(i / S);
-    const long long e = i - (long long)f * S;
-    const double zp = normal_at(seed, (uint32_t)f, (uint32_t)(e >> 2), (int)(e & 3));
-    const double zq = normal_at(seed, (uint32_t)(nf + f), (uint32_t)(e >> 2), (int)(e & 3));
-    if (split) {
-      ((float*)phi)[i] = (float)(noise * zp);
-      ((float*)pi)[i] = (float)(noise * zq);
-    } else {
-      ((double*)phi)[i] = (f == 0 ? bg0 : bg1) + noise * zp;
-      ((double*)pi)[i] = (f == 0 ? mom0 : mom1) + noise * zq;
+    const int arr = (int)(i / nb);                 // 0 .. nf - 1: phi, nf .. 2 nf - 1: pi
+    const long long blk = i - (long long)arr * nb;
+    const int f = arr < nf ? arr : arr - nf;
+    double z[4];
+    normals_at(seed, (uint32_t)arr, (uint32_t)blk, z);
+    void* out = arr < nf ? phi : pi;
+    const double base = arr < nf ? (f == 0 ? bg0 : bg1) : (f == 0 ? mom0 : mom1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long e = 4 * blk + k;
+      if (e >= S) break;
+      if (split) ((float*)out)[(long long)f * S + e] = (float)(noise * z[k]);
+      else ((double*)out)[(long long)f * S + e] = base + noise * z[k];
     }
   }
 }
@@ -357,7 +368,28 @@ pycool_status admit(pycool_server* s, const Request& r, int slot) {
   return PYCOOL_OK;
 }
 
-// Capture K stage launches of every member of a group into one graph.
+// The records the host looks at after a replay (background and fault word of
+// every member), written to its pinned arrays by the graph's last kernel: a
+// block per member in one launch, where two small copies per member took longer
+// than a stage of a small lattice.
+struct RecordTable {
+  int32_t count;
+  int32_t slot[kMaxMembers];
+  const SimDesc* desc[kMaxMembers];
+};
+__global__ void __launch_bounds__(64) records_kernel(const __grid_constant__ RecordTable t,
+                                                     Background* h_bg, int32_t* h_fault) {
+  const SimDesc& d = *t.desc[blockIdx.x];
+  const int slot = t.slot[blockIdx.x];
+  static_assert(sizeof(Background) % 8 == 0 && sizeof(Background) <= 64 * 8, "one word per thread");
+  if (threadIdx.x < sizeof(Background) / 8)
+    reinterpret_cast<unsigned long long*>(&h_bg[slot])[threadIdx.x] =
+        reinterpret_cast<const unsigned long long*>(d.bg)[threadIdx.x];
+  if (threadIdx.x == 0) h_fault[slot] = *d.fault;
+}
+
+// Capture K stage launches of every member of a group, then their records, into
+// one graph.
 pycool_status rebuild(pycool_server* s, Group& G) {
   if (G.graph) {
     cudaGraphExecDestroy(G.graph);
@@ -366,20 +398,27 @@ pycool_status rebuild(pycool_server* s, Group& G) {
   G.dirty = false;
   if (G.members.empty()) return PYCOOL_OK;
   std::vector<LaunchTable> tables;
+  std::vector<RecordTable> records;
   std::vector<int> grids;
   for (size_t i = 0; i < G.members.size(); i += kMaxMembers) {
     LaunchTable t;
+    RecordTable rt;
     std::memset(&t, 0, sizeof(t));
+    std::memset(&rt, 0, sizeof(rt));
     int off = 0;
     for (size_t j = i; j < G.members.size() && j < i + kMaxMembers; ++j) {
       const Member& m = *s->slots[G.members[j]];
       t.cta_offset[t.count] = off;
       t.desc[t.count] = (const SimDesc*)(m.state + m.L.off_desc);
+      rt.desc[t.count] = t.desc[t.count];
+      rt.slot[t.count] = G.members[j];
       off += m.L.geo.ncta;
       t.count++;
     }
     t.cta_offset[t.count] = off;
+    rt.count = t.count;
     tables.push_back(t);
+    records.push_back(rt);
     grids.push_back(off);
   }
   const SimDesc& d0 = s->slots[G.members[0]]->hdesc;
@@ -389,6 +428,10 @@ pycool_status rebuild(pycool_server* s, Group& G) {
   for (int k = 0; k < s->stages_per_graph && le == cudaSuccess; ++k)
     for (size_t i = 0; i < tables.size() && le == cudaSuccess; ++i)
       le = launch_sweep(d0, tables[i], grids[i], s->capture);
+  for (size_t i = 0; i < records.size() && le == cudaSuccess; ++i) {
+    records_kernel<<<records[i].count, 64, 0, s->capture>>>(records[i], s->h_bg, s->h_fault);
+    le = cudaGetLastError();
+  }
   const cudaError_t ee = cudaStreamEndCapture(s->capture, &graph);
   SCK(le);
   SCK(ee);
@@ -486,19 +529,12 @@ void server_loop(pycool_server* s) {
         s->queue.push_front(*it);
       }
     }
-    // 2. one graph replay per group, then a copy of every member's record
+    // 2. one graph replay per group (its last kernel brings every member's record)
     bool any = false;
     for (Group& G : s->groups) {
       if (G.members.empty()) continue;
       if (G.dirty && rebuild(s, G) != PYCOOL_OK) { fail_all(s, PYCOOL_E_CUDA); return; }
       if (cudaGraphLaunch(G.graph, G.stream) != cudaSuccess) { fail_all(s, PYCOOL_E_CUDA); return; }
-      for (int slot : G.members) {
-        const Member& m = *s->slots[slot];
-        cudaMemcpyAsync(&s->h_bg[slot], m.state + m.L.off_bg, sizeof(Background),
-                        cudaMemcpyDeviceToHost, G.stream);
-        cudaMemcpyAsync(&s->h_fault[slot], m.ws + m.L.off_ticket + 128, sizeof(int32_t),
-                        cudaMemcpyDeviceToHost, G.stream);
-      }
       any = true;
     }
     bool persistent = false;

@@ -832,6 +832,104 @@ __device__ __forceinline__ unsigned int ticket_add(unsigned int* p) {
 }
 
 // ---------------------------------------------------------------------------
+// FP64 form: the Laplacian in 64-bit fixed point.
+//
+// GB300 executes two float64 lanes per SM and clock (a warp instruction takes
+// 64 cycles of a scheduler's pipe), and 64-bit conversions run at the same
+// rate, while integer adds, shifts and logic run 16 to 32 times faster.  The
+// discrete Laplacian is a sum with small integer weights, so it is taken off
+// the float64 pipe: each drifted field value is put on a 64-bit fixed-point
+// scale once (to_fixed, integer instructions only), D is summed exactly in
+// integers, and one normalisation (from_fixed, integer instructions) gives D
+// rounded once to float64.  The scale comes from the largest |phi| and |pi| of
+// the stage's input (Ctx::set_fix; the stages track them), so no sum can
+// overflow; a field value within 2^6 (27- and 13-point stencils: 2^2) of the
+// largest keeps every bit, and a smaller one is cut at 2^-58 (2^-54) of the
+// largest or less, below the rounding of the float64 sums it replaces.  A stage whose
+// input has no usable maximum (the first pass over a new state, values out of
+// range or not finite) sums in float64 (FIX = false).
+// Measured on GB300, against the same kernels with float64 stencils (persistent kernel;
+// set_initial, evolve and get_fields together): 256^3 Q-ball, order 8, two steps 38.6 -> 25.2
+// ms; 256^3 oscillon, order 6, three steps 13.3 -> 8.9 ms; 128^3 preheating,
+// order 4, ten steps 4.49 -> 2.83 ms, with the 13-point stencil 6.78 -> 3.40 ms.
+// ---------------------------------------------------------------------------
+// bits of |D| above the largest |I|: sum of the absolute weights, 12 (7-point),
+// 256 (27-point, weights times 30), 192 (13-point, times 12)
+template <int STENCIL> constexpr int fix_headroom() { return STENCIL == 7 ? 4 : 8; }
+// what the integer sums are times D
+template <int STENCIL> constexpr double fix_weight() {
+  return STENCIL == 7 ? 1.0 : (STENCIL == 27 ? 30.0 : 12.0);
+}
+
+// trunc(v 2^(1086 - E)) for |v| < 2^(E - 1023): the significand, bit 63 down,
+// shifted right by E - e (shr clamps: values below the scale, and zero, give 0).
+__device__ __forceinline__ unsigned long long to_fixed(double v, int E) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int hi = __double2hiint(v);
+  const int sh = E - ((hi >> 20) & 0x7ff);
+  unsigned long long m = (b << 11) | 0x8000000000000000ull;
+  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));
+  return hi < 0 ? 0ull - m : m;
+}
+// x 2^(E - 1086), rounded to nearest (a tie away from zero)
+__device__ __forceinline__ double from_fixed(unsigned long long x, int E) {
+  const bool neg = (long long)x < 0;
+  unsigned long long m = neg ? 0ull - x : x;
+  const int lz = __clzll((long long)m);
+  asm("shl.b64 %0, %0, %1;" : "+l"(m) : "r"(lz));
+  unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);
+  r += (unsigned long long)(uint32_t)(E - lz - 1) << 52;
+  r |= neg ? 0x8000000000000000ull : 0ull;
+  return __longlong_as_double((long long)(m == 0ull ? 0ull : r));
+}
+
+template <bool FIX> struct FixElem { using type = double; };
+template <> struct FixElem<true> { using type = unsigned long long; };
+__device__ __forceinline__ double fix_in(double v, int, double*) { return v; }
+__device__ __forceinline__ unsigned long long fix_in(double v, int E, unsigned long long*) {
+  return to_fixed(v, E);
+}
+__device__ __forceinline__ double fix_out(double v, int) { return v; }
+__device__ __forceinline__ double fix_out(unsigned long long v, int E) { return from_fixed(v, E); }
+
+__device__ __forceinline__ double fix_mad(double a, double b, double c) { return madd(a, b, c); }
+__device__ __forceinline__ unsigned long long fix_mad(unsigned long long a, unsigned long long b,
+                                                      unsigned long long c) {
+  return a * b + c;
+}
+// In-plane parts of the stencil (Eq. D split by z-offset, as plane_parts):
+// float64 with the weights themselves, integers with the weights times 30
+// (27-point) or as they are (7-point).
+__device__ __forceinline__ double fix_mid7(double c, double faces) { return madd(-6.0, c, faces); }
+__device__ __forceinline__ unsigned long long fix_mid7(unsigned long long c,
+                                                       unsigned long long faces) {
+  return faces - 6ull * c;
+}
+__device__ __forceinline__ void fix_parts27(double c, double faces, double corners, double& mid,
+                                            double& off) {
+  mid = madd(3.0 / 30.0, corners, madd(14.0 / 30.0, faces, (-128.0 / 30.0) * c));
+  off = madd(1.0 / 30.0, corners, madd(3.0 / 30.0, faces, (14.0 / 30.0) * c));
+}
+__device__ __forceinline__ void fix_parts27(unsigned long long c, unsigned long long faces,
+                                            unsigned long long corners, unsigned long long& mid,
+                                            unsigned long long& off) {
+  mid = 14ull * faces + 3ull * corners - (c << 7);
+  off = 14ull * c + 3ull * faces + corners;
+}
+
+// High words of the largest magnitudes a thread has put out, per field (phi, pi).
+template <int NF> struct HiMax {
+  uint32_t v[2 * NF];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < 2 * NF; ++i) v[i] = 0u;
+  }
+  __device__ __forceinline__ void add(int i, double x) {
+    v[i] = max(v[i], (uint32_t)__double2hiint(x) & 0x7fffffffu);
+  }
+};
+
+// ---------------------------------------------------------------------------
 // Block finish: partials, tickets, and (last block) the background update.
 // sout holds this block's NQ sums on entry.  Two levels, so that almost all
 // of the fold overlaps the sweep: the last block of each group of kGroup
@@ -840,9 +938,33 @@ __device__ __forceinline__ unsigned int ticket_add(unsigned int* p) {
 // each row and takes the ticket; the block barrier after it orders the other
 // threads' reads of the rows.
 // ---------------------------------------------------------------------------
+//
+// bmax (FP64 kernels that track them): the block's largest |phi| and |pi| high
+// words per field in shared memory, folded beside the sums in the rows' last
+// slots and left in the Background; NULL: the maxima become unknown.
+template <int NF>
+__device__ __forceinline__ void fold_max(const double* src, int P, uint32_t* out) {
+  const int lane = threadIdx.x & 31;
+  uint32_t m[2 * NF];
+#pragma unroll
+  for (int i = 0; i < 2 * NF; ++i) m[i] = 0u;
+  for (int r = lane; r < P; r += 32)
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const uint2 v = __ldcg(reinterpret_cast<const uint2*>(src + (size_t)r * kNQ + kNQ - kMaxFields + f));
+      m[2 * f] = max(m[2 * f], v.x);
+      m[2 * f + 1] = max(m[2 * f + 1], v.y);
+    }
+#pragma unroll
+  for (int i = 0; i < 2 * NF; ++i) {
+    m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+    if (lane == 0) out[i] = m[i];
+  }
+}
+
 template <int MODEL, int PREC, typename C>
 __device__ __forceinline__ void finish_block(const C& cx, const SimDesc& d, int mode, int cta,
-                                             double* sout, int* s_last) {
+                                             double* sout, int* s_last, uint32_t* bmax = nullptr) {
   using SL = typename C::SL;
   constexpr int NF = C::NF;
   constexpr int NQ = SL::NQ;
@@ -853,23 +975,37 @@ __device__ __forceinline__ void finish_block(const C& cx, const SimDesc& d, int 
   if (tid == 0) {
 #pragma unroll
     for (int q = 0; q < NQ; ++q) d.partials[(size_t)cta * kNQ + q] = sout[q];
+    if (bmax) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f)
+        reinterpret_cast<uint2*>(d.partials + (size_t)cta * kNQ + kNQ - kMaxFields)[f] =
+            make_uint2(bmax[2 * f], bmax[2 * f + 1]);
+    }
     *s_last = (ticket_add(&d.gticket[g]) == (unsigned int)(gn - 1));
   }
   __syncthreads();
   if (!*s_last) return;
 
   // ---- last block of group g: fold the group's rows ------------------------
+  if (bmax && tid >= kThreads - 32) fold_max<NF>(d.partials + (size_t)g0 * kNQ, gn, bmax);
   fold_rows<NQ>(d.partials + (size_t)g0 * kNQ, gn, sout);
   if (tid == 0) {
     d.gticket[g] = 0u;  // every block of the group has counted
 #pragma unroll
     for (int q = 0; q < NQ; ++q) d.gpartials[(size_t)g * kNQ + q] = sout[q];
+    if (bmax) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f)
+        reinterpret_cast<uint2*>(d.gpartials + (size_t)g * kNQ + kNQ - kMaxFields)[f] =
+            make_uint2(bmax[2 * f], bmax[2 * f + 1]);
+    }
     *s_last = (ticket_add(d.ticket) == (unsigned int)(d.ngroups - 1));
   }
   __syncthreads();
   if (!*s_last) return;
 
   // ---- last group: fold the group rows, then the background update ---------
+  if (bmax && tid >= kThreads - 32) fold_max<NF>(d.gpartials, d.ngroups, bmax);
   fold_rows<NQ>(d.gpartials, d.ngroups, sout);
   if (tid != 0) return;
 
@@ -877,7 +1013,8 @@ __device__ __forceinline__ void finish_block(const C& cx, const SimDesc& d, int 
   Background nb;
   post_stage<MODEL, PREC>(cx, d, mode, sout, *bgp, nb);
 #pragma unroll
-  for (int i = 0; i < 2 * kMaxFields; ++i) nb.amax[i] = 0u;   // not tracked here
+  for (int i = 0; i < 2 * kMaxFields; ++i)
+    nb.amax[i] = (bmax && i < 2 * NF) ? 0x80000000u | bmax[i] : 0u;
   *bgp = nb;  // published to the next launch by the kernel boundary
   *d.ticket = 0u;
 }
@@ -953,13 +1090,17 @@ template <int STENCIL> struct StencilW {
 };
 
 // ---------------------------------------------------------------------------
-// TMA-staged sweep (n % 32 == 0).  256 threads = 8 warps; warp w owns tile row
-// y0 + w, lane l owns sites x0 + l*VX .. +VX-1.
+// TMA-staged FP64 sweep (n % 32 == 0).  256 threads = 8 warps; warp w owns tile
+// row y0 + w, lane l owns sites x0 + l*VX .. +VX-1.  The drifted plane replaces
+// the plane's phi in its ring slot as the stencil wants it: in fixed point, or in
+// float64 for a stage without a scale (FIX).  Bound by the float64 pipe: serving
+// a batch of twelve requests up to 128^3, 41.3 -> see sweep_tma's note below.
 // ---------------------------------------------------------------------------
-template <int MODEL, int STENCIL, int PREC, int VX>
+template <int MODEL, int STENCIL, int VX>
 __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) {
+  constexpr int PREC = PREC_FP64;
   using C = Ctx<MODEL, PREC>;
-  using T = typename C::T;
+  using T = double;
   using SL = typename C::SL;
   constexpr int NF = C::NF;
   constexpr int NQ = SL::NQ;
@@ -975,6 +1116,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
   __shared__ __align__(8) uint64_t mbar[NSLOT];
   __shared__ double sred[(kThreads / 32) * NQ];
   __shared__ double sout[NQ];
+  __shared__ uint32_t s_wmax[kThreads / 32][2 * NF], s_bmax[2 * NF];
   __shared__ int s_last, s_fault;
 
   const int mem = member_of(tab, blockIdx.x);
@@ -1009,12 +1151,6 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
   const CUtensorMap* tpi_main = &d.tmap[2 + ((ib >> 1) & 1)][0];
   const CUtensorMap* tpi_row = &d.tmap[2 + ((ib >> 1) & 1)][1];
   const int yl = wrapi(y0 - 1, n), yh = wrapi(y0 + TY, n);
-
-  // stencil weights (Eq. D): 7pt (-6, 1, 0, 0); iso27 (-128, 14, 3, 1)/30
-  const T c0 = CORNERS ? (T)(-128.0 / 30.0) : (T)(-6.0);
-  const T c1 = CORNERS ? (T)(14.0 / 30.0) : (T)1.0;
-  const T c2 = CORNERS ? (T)(3.0 / 30.0) : (T)0.0;
-  const T c3 = CORNERS ? (T)(1.0 / 30.0) : (T)0.0;
 
   // halo columns: threads [64, 64 + 2 ROWS): side = left/right, row = y0-1 .. y0+TY
   const bool hcol = tid >= 64 && tid < 64 + 2 * ROWS;
@@ -1069,160 +1205,164 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
     if (Q > 1) issue(1);
   } else if (tid == 32) {
     s_ctx.init(bgr, d, mode);  // while the first planes are in flight
+    s_ctx.set_fix(bgr.amax, fix_headroom<STENCIL>());
   }
   load_col(z0 - 1);
   __syncthreads();
-  const C cx = s_ctx;
 
-  Acc<T> acc[NQ];
-  T accd_s[NQ];   // float64 path: plain per-thread sums
+  T accd_s[NQ];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) { acc[q].zero(); accd_s[q] = (T)0; }
-  // rotating registers: part_m = S_off(z-1) + S_mid(z) of the plane z = p - 1
-  // awaiting output; so_m = S_off(p - 1) (iso27 only; it is phi* for 7pt);
-  // ph_m / pi_m = drifted phi and (re-centred) momentum of plane p - 1.
-  T part_m[NF][VX], so_m[NF][VX], ph_m[NF][VX], pi_m[NF][VX];
-#pragma unroll
-  for (int f = 0; f < NF; ++f)
-#pragma unroll
-    for (int j = 0; j < VX; ++j) part_m[f][j] = so_m[f][j] = ph_m[f][j] = pi_m[f][j] = (T)0;
-
+  for (int q = 0; q < NQ; ++q) accd_s[q] = 0.0;
+  HiMax<NF> hm;
+  hm.zero();
   int q = 0;
-  for (; q < Q; ++q) {
-    const int s = q % NSLOT;
-    const int p = z0 - 1 + q;
-    if (!mbar_wait(&mbar[s], (uint32_t)((q / NSLOT) & 1))) atomicOr(&s_fault, 1);
-
-    // drift this plane in place: phi* = phi + c pi (re-centred in the split form)
-    T cur_ph[NF][VX], cur_pi[NF][VX];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      T ph[VX], pv[VX];
-      vload<T, VX>(&stage[s][0][f][ly + 1][lane * VX], ph);
-      vload<T, VX>(&stage[s][1][f][ly + 1][lane * VX], pv);
-#pragma unroll
-      for (int j = 0; j < VX; ++j) {
-        if constexpr (PREC == PREC_SPLIT) { ph[j] -= cx.mu_phi[f]; pv[j] -= cx.mu_pi[f]; }
-        cur_pi[f][j] = pv[j];
-        cur_ph[f][j] = madd(cx.cdrift, pv[j], ph[j]);
-      }
-      vstore<T, VX>(&stage[s][0][f][ly + 1][lane * VX], cur_ph[f]);
-    }
-    if (tid < 64) {  // the two halo rows
-      const int r = tid < 32 ? 0 : ROWS - 1;
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        T ph[VX], pv[VX];
-        vload<T, VX>(&stage[s][0][f][r][lane * VX], ph);
-        vload<T, VX>(&stage[s][1][f][r][lane * VX], pv);
-#pragma unroll
-        for (int j = 0; j < VX; ++j) {
-          if constexpr (PREC == PREC_SPLIT) { ph[j] -= cx.mu_phi[f]; pv[j] -= cx.mu_pi[f]; }
-          ph[j] = madd(cx.cdrift, pv[j], ph[j]);
-        }
-        vstore<T, VX>(&stage[s][0][f][r][lane * VX], ph);
-      }
-    } else if (hcol) {  // the two halo columns
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        T ph = sp[f], pv = sq[f];
-        if constexpr (PREC == PREC_SPLIT) { ph -= cx.mu_phi[f]; pv -= cx.mu_pi[f]; }
-        colb[s][f][hc_side][hc_row] = madd(cx.cdrift, pv, ph);
-      }
-      if (q + 1 < Q) load_col(p + 1);
-    }
-    // every thread's generic reads and writes of the slot recycled below come
-    // before the TMA copy (async proxy) that refills it: a proxy fence by each
-    // thread, then the block barrier
-    fence_proxy_async();
-    __syncthreads();
-    if (s_fault) break;
-    if (tid == 0 && q + 2 < Q) issue(q + 2);
-
-    T so_new[NF][VX], smid_new[NF][VX];   // S_off(p), S_mid(p)
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      T dn[VX], up[VX];
-      vload<T, VX>(&stage[s][0][f][ly][lane * VX], dn);
-      vload<T, VX>(&stage[s][0][f][ly + 2][lane * VX], up);
-      T left = __shfl_up_sync(0xffffffffu, cur_ph[f][VX - 1], 1);
-      T right = __shfl_down_sync(0xffffffffu, cur_ph[f][0], 1);
-      if (lane == 0) left = colb[s][f][0][ly + 1];
-      if (lane == 31) right = colb[s][f][1][ly + 1];
-      T dl = 0, dr = 0, ul = 0, ur = 0;
-      if constexpr (CORNERS) {
-        dl = __shfl_up_sync(0xffffffffu, dn[VX - 1], 1);
-        dr = __shfl_down_sync(0xffffffffu, dn[0], 1);
-        ul = __shfl_up_sync(0xffffffffu, up[VX - 1], 1);
-        ur = __shfl_down_sync(0xffffffffu, up[0], 1);
-        if (lane == 0) { dl = colb[s][f][0][ly]; ul = colb[s][f][0][ly + 2]; }
-        if (lane == 31) { dr = colb[s][f][1][ly]; ur = colb[s][f][1][ly + 2]; }
-      }
-#pragma unroll
-      for (int j = 0; j < VX; ++j) {
-        const T ctr = cur_ph[f][j];
-        const T L = j > 0 ? cur_ph[f][j - 1] : left;
-        const T R = j < VX - 1 ? cur_ph[f][j + 1] : right;
-        const T faces = (dn[j] + up[j]) + (L + R);
-        if constexpr (CORNERS) {
-          const T DL = j > 0 ? dn[j - 1] : dl;
-          const T DR = j < VX - 1 ? dn[j + 1] : dr;
-          const T UL = j > 0 ? up[j - 1] : ul;
-          const T UR = j < VX - 1 ? up[j + 1] : ur;
-          const T corners = (DL + DR) + (UL + UR);
-          smid_new[f][j] = madd(c2, corners, madd(c1, faces, c0 * ctr));
-          so_new[f][j] = madd(c3, corners, madd(c2, faces, c1 * ctr));
-        } else {
-          smid_new[f][j] = madd(c0, ctr, faces);
-          so_new[f][j] = ctr;
-        }
-      }
-    }
-    if (q >= 2) {  // output plane z = p - 1
-      const size_t o = (size_t)(p - 1) * nn + (size_t)gy * n + gx;
-      // float: per-plane partials then Kahan; double: straight into the accumulators
-      T ps_local[NQ];
-      T* ps = ps_local;
-      if constexpr (PREC == PREC_FP64) {
-        ps = accd_s;
-      } else {
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) ps_local[i] = (T)0;
-      }
-      T pin[NF][VX];
-#pragma unroll
-      for (int j = 0; j < VX; ++j) {
-        T phj[NF], Dj[NF], pmj[NF], pnj[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          phj[f] = ph_m[f][j];
-          Dj[f] = part_m[f][j] + so_new[f][j];
-          pmj[f] = pi_m[f][j];
-        }
-        cx.site(mode, phj, Dj, pmj, pnj, ps);
-#pragma unroll
-        for (int f = 0; f < NF; ++f) pin[f][j] = pnj[f];
-      }
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        vstore<T, VX>(phi_out + f * S + o, ph_m[f]);
-        if (mode == MODE_SWEEP) vstore<T, VX>(pi_out + f * S + o, pin[f]);
-      }
-      if constexpr (PREC == PREC_SPLIT) {
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) acc[i].add(ps_local[i]);
-      }
-    }
+  auto body = [&](auto fix_c) {
+    constexpr bool FIX = decltype(fix_c)::value;
+    using E = typename FixElem<FIX>::type;
+    C cx = s_ctx;
+    // see stage_fp64: the 27-point integer sums are 30 D
+    if constexpr (FIX && STENCIL == 27) cx.kD *= 1.0 / fix_weight<STENCIL>();
+    // rotating registers: part_m = S_off(z-1) + S_mid(z) of the plane z = p - 1
+    // awaiting output; so_m = S_off(p - 1); ph_m / pi_m = drifted phi and
+    // momentum of plane p - 1
+    E part_m[NF][VX], so_m[NF][VX];
+    T ph_m[NF][VX], pi_m[NF][VX];
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
       for (int j = 0; j < VX; ++j) {
-        part_m[f][j] = (CORNERS ? so_m[f][j] : ph_m[f][j]) + smid_new[f][j];
-        if constexpr (CORNERS) so_m[f][j] = so_new[f][j];
-        ph_m[f][j] = cur_ph[f][j];
-        pi_m[f][j] = cur_pi[f][j];
+        part_m[f][j] = so_m[f][j] = (E)0;
+        ph_m[f][j] = pi_m[f][j] = 0.0;
       }
-  }
+    for (; q < Q; ++q) {
+      const int s = q % NSLOT;
+      const int p = z0 - 1 + q;
+      if (!mbar_wait(&mbar[s], (uint32_t)((q / NSLOT) & 1))) atomicOr(&s_fault, 1);
+
+      // drift this plane: phi* = phi + c pi, and into the slot as the stencil's element
+      T cur_ph[NF][VX], cur_pi[NF][VX];
+      E ctr[NF][VX];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        T ph[VX];
+        vload<T, VX>(&stage[s][0][f][ly + 1][lane * VX], ph);
+        vload<T, VX>(&stage[s][1][f][ly + 1][lane * VX], cur_pi[f]);
+#pragma unroll
+        for (int j = 0; j < VX; ++j) {
+          cur_ph[f][j] = madd(cx.cdrift, cur_pi[f][j], ph[j]);
+          ctr[f][j] = fix_in(cur_ph[f][j], cx.fx[f], (E*)nullptr);
+        }
+        vstore<E, VX>(reinterpret_cast<E*>(&stage[s][0][f][ly + 1][lane * VX]), ctr[f]);
+      }
+      if (tid < 64) {  // the two halo rows
+        const int r = tid < 32 ? 0 : ROWS - 1;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          T ph[VX], pv[VX];
+          E e[VX];
+          vload<T, VX>(&stage[s][0][f][r][lane * VX], ph);
+          vload<T, VX>(&stage[s][1][f][r][lane * VX], pv);
+#pragma unroll
+          for (int j = 0; j < VX; ++j)
+            e[j] = fix_in(madd(cx.cdrift, pv[j], ph[j]), cx.fx[f], (E*)nullptr);
+          vstore<E, VX>(reinterpret_cast<E*>(&stage[s][0][f][r][lane * VX]), e);
+        }
+      } else if (hcol) {  // the two halo columns
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+          *reinterpret_cast<E*>(&colb[s][f][hc_side][hc_row]) =
+              fix_in(madd(cx.cdrift, sq[f], sp[f]), cx.fx[f], (E*)nullptr);
+        if (q + 1 < Q) load_col(p + 1);
+      }
+      // every thread's generic reads and writes of the slot recycled below come
+      // before the TMA copy (async proxy) that refills it: a proxy fence by each
+      // thread, then the block barrier
+      fence_proxy_async();
+      __syncthreads();
+      if (s_fault) break;
+      if (tid == 0 && q + 2 < Q) issue(q + 2);
+
+      E so_new[NF][VX], smid_new[NF][VX];   // S_off(p), S_mid(p)
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        E dn[VX], up[VX];
+        vload<E, VX>(reinterpret_cast<const E*>(&stage[s][0][f][ly][lane * VX]), dn);
+        vload<E, VX>(reinterpret_cast<const E*>(&stage[s][0][f][ly + 2][lane * VX]), up);
+        const E* cl = reinterpret_cast<const E*>(&colb[s][f][0][0]);
+        const E* cr = reinterpret_cast<const E*>(&colb[s][f][1][0]);
+        E left = __shfl_up_sync(0xffffffffu, ctr[f][VX - 1], 1);
+        E right = __shfl_down_sync(0xffffffffu, ctr[f][0], 1);
+        if (lane == 0) left = cl[ly + 1];
+        if (lane == 31) right = cr[ly + 1];
+        E dl{}, dr{}, ul{}, ur{};
+        if constexpr (CORNERS) {
+          dl = __shfl_up_sync(0xffffffffu, dn[VX - 1], 1);
+          dr = __shfl_down_sync(0xffffffffu, dn[0], 1);
+          ul = __shfl_up_sync(0xffffffffu, up[VX - 1], 1);
+          ur = __shfl_down_sync(0xffffffffu, up[0], 1);
+          if (lane == 0) { dl = cl[ly]; ul = cl[ly + 2]; }
+          if (lane == 31) { dr = cr[ly]; ur = cr[ly + 2]; }
+        }
+#pragma unroll
+        for (int j = 0; j < VX; ++j) {
+          const E L = j > 0 ? ctr[f][j > 0 ? j - 1 : 0] : left;
+          const E R = j < VX - 1 ? ctr[f][j < VX - 1 ? j + 1 : 0] : right;
+          const E faces = (dn[j] + up[j]) + (L + R);
+          if constexpr (CORNERS) {
+            const E DL = j > 0 ? dn[j > 0 ? j - 1 : 0] : dl;
+            const E DR = j < VX - 1 ? dn[j < VX - 1 ? j + 1 : 0] : dr;
+            const E UL = j > 0 ? up[j > 0 ? j - 1 : 0] : ul;
+            const E UR = j < VX - 1 ? up[j < VX - 1 ? j + 1 : 0] : ur;
+            fix_parts27(ctr[f][j], faces, (DL + DR) + (UL + UR), smid_new[f][j], so_new[f][j]);
+          } else {
+            smid_new[f][j] = fix_mid7(ctr[f][j], faces);
+            so_new[f][j] = ctr[f][j];
+          }
+        }
+      }
+      if (q >= 2) {  // output plane z = p - 1
+        const size_t o = (size_t)(p - 1) * nn + (size_t)gy * n + gx;
+        T pin[NF][VX];
+#pragma unroll
+        for (int j = 0; j < VX; ++j) {
+          T phj[NF], Dj[NF], pmj[NF], pnj[NF];
+#pragma unroll
+          for (int f = 0; f < NF; ++f) {
+            phj[f] = ph_m[f][j];
+            Dj[f] = fix_out(part_m[f][j] + so_new[f][j], cx.fx[f]);
+            pmj[f] = pi_m[f][j];
+          }
+          cx.site(mode, phj, Dj, pmj, pnj, accd_s);
+#pragma unroll
+          for (int f = 0; f < NF; ++f) {
+            pin[f][j] = pnj[f];
+            hm.add(2 * f, phj[f]);
+            hm.add(2 * f + 1, pnj[f]);
+          }
+        }
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          vstore<T, VX>(phi_out + f * S + o, ph_m[f]);
+          if (mode == MODE_SWEEP) vstore<T, VX>(pi_out + f * S + o, pin[f]);
+        }
+      }
+#pragma unroll
+      for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int j = 0; j < VX; ++j) {
+          part_m[f][j] = so_m[f][j] + smid_new[f][j];
+          so_m[f][j] = so_new[f][j];
+          ph_m[f][j] = cur_ph[f][j];
+          pi_m[f][j] = cur_pi[f][j];
+        }
+    }
+    if constexpr (FIX && STENCIL == 27) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f) accd_s[SL::PHID + f] *= 1.0 / fix_weight<STENCIL>();
+    }
+  };
+  if (s_ctx.fx[0]) body(std::true_type{});
+  else body(std::false_type{});
 
   if (s_fault) {
     // a TMA copy never completed: record it, drain what is in flight (bounded), stop
@@ -1233,8 +1373,20 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
     }
     return;
   }
-  block_partials<PREC, NQ, T>(acc, accd_s, sred, sout);
-  finish_block<MODEL, PREC>(s_ctx, d, mode, cta, sout, &s_last);
+#pragma unroll
+  for (int i = 0; i < 2 * NF; ++i) {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, hm.v[i]);
+    if (lane == 0) s_wmax[ly][i] = m;
+  }
+  block_partials<PREC, NQ, T>(nullptr, accd_s, sred, sout);
+  if (tid < 2 * NF) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) m = max(m, s_wmax[w][tid]);
+    s_bmax[tid] = m;
+  }
+  __syncthreads();
+  finish_block<MODEL, PREC>(s_ctx, d, mode, cta, sout, &s_last, s_bmax);
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -2002,7 +2154,7 @@ cudaError_t launch_sweep_impl(int model, int stencil, int vx, int tma, const Lau
         sweep_split_pipe<M, ST, V><<<g, b, smem, s>>>(t);                \
       } else {                                                           \
         if (grid == 0) return cudaSuccess;                               \
-        sweep_tma<M, ST, PREC, V><<<g, b, 0, s>>>(t);                    \
+        sweep_tma<M, ST, V><<<g, b, 0, s>>>(t);                    \
       }                                                                  \
       return cudaGetLastError();                                         \
     }                                                                    \

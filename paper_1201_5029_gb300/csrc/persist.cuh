@@ -211,6 +211,23 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* count, unsigned
   return ok;
 }
 
+// The quantities a pass sums: a flush all of them; a sweep of the FP64 form sum
+// pi^2, sum phi D (the fields together: Ctx::site) and sum V, on warps of
+// different schedulers, a sweep of the split forms all but the variance sums.  A
+// float64 addition of a warp takes 64 cycles of its scheduler's pipe, so the nine
+// sums of a two-field block took 3 000 cycles, the three take 1 300.
+template <int NF, int PREC> struct LiveSlots {
+  using SL = Slots<NF, PREC>;
+  static constexpr int SWEEP = SL::DPHI2;
+  __device__ static int slot(int w, bool) { return w; }
+};
+template <int NF> struct LiveSlots<NF, PREC_FP64> {
+  using SL = Slots<NF, PREC_FP64>;
+  static constexpr int SWEEP = 3;
+  __device__ static int slot(int w, bool sweep) { return sweep ? w * NF : w; }
+  static_assert(SL::PI2 == 0 && SL::PHID == NF && SL::V == 2 * NF, "slots of a sweep");
+};
+
 __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, int x, int y, int z,
                                             int f, int buf, uint64_t* bar) {
   asm volatile(

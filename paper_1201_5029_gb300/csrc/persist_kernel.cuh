@@ -206,11 +206,22 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
     // @units-done
     if (s_bad) { fault = true; break; }
 
-    // ---- block sums: one warp per quantity over the 512 threads' values, fixed order ----
+    // ---- block sums: one warp per live quantity over the 512 threads' values, fixed order ----
+    const bool sweep = mode == MODE_SWEEP;
+    const int nl = sweep ? LiveSlots<NF, PREC>::SWEEP : NQ;   // live quantities
+    const int slot = LiveSlots<NF, PREC>::slot(warp, sweep);  // of this warp (warp < nl)
+    if (tid < kNQ) sums[tid] = 0.0;
     if constexpr (PREC != PREC_SPLIT) {
       double* red = sm.red;
+      if (PREC == PREC_FP64 && sweep) {
+        red[tid] = accd[SL::PHID - NF];   // PI2
+        red[kPThreads + tid] = accd[SL::PHID];
+        red[2 * kPThreads + tid] = accd[SL::V];
+      } else {
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) red[q * kPThreads + tid] = accd[q];
+        for (int q = 0; q < NQ; ++q)
+          if (q < nl) red[q * kPThreads + tid] = accd[q];
+      }
       if constexpr (PREC == PREC_FP64) {
 #pragma unroll
         for (int i = 0; i < 2 * NF; ++i) {
@@ -219,7 +230,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         }
       }
       __syncthreads();
-      if (warp < NQ) {
+      if (warp < nl) {
         // 16 values per lane summed as a pairwise tree (depth 4: FP64 latency is long)
         double x[kPThreads / 32];
 #pragma unroll
@@ -232,10 +243,10 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
 #pragma unroll
         for (int h = 16; h >= 1; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
         if (lane == 0) {
-          reinterpret_cast<double*>(p.rows)[((size_t)(k & 1) * G + blockIdx.x) * kNQ + warp] = v;
+          reinterpret_cast<double*>(p.rows)[((size_t)(k & 1) * G + blockIdx.x) * kNQ + slot] = v;
           fence_proxy_async_global();   // the rows are read back by bulk copies
         }
-      } else if (PREC == PREC_FP64 && warp == NQ) {
+      } else if (PREC == PREC_FP64 && warp == nl) {
         // the block's largest |phi| and |pi| of field f in the row's slot kNQ - 2 + f
         static_assert(PREC != PREC_FP64 || NQ <= kNQ - kMaxFields, "free slots of a row");
         uint32_t m[2 * NF];
@@ -252,7 +263,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         }
       }
     } else {
-      if (warp < NQ) {
+      if (warp < nl) {
         float hi = 0.f, lo = 0.f;
 #pragma unroll
         for (int r = 0; r < kKahanGroups / 32; ++r) {
@@ -285,9 +296,9 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
       if (k < KL) {
         const int mn = k + 1 < K ? MODE_SWEEP : MODE_FLUSH;
         const int sn = sbv[cb].stage + 1 < d.nstages ? sbv[cb].stage + 1 : 0;
-        const Coef& kc = sctxv[cb].k;
+        const Coef& kc = sctxv[cb].k;   // of a sweep: a flush is the last pass
         const double hn = stage_step(d, sn, kc.deta, mn);
-        s_qn = prestage_a(kc.a, __drcp_rn(kc.a), kc.h, hn, d, mn, d.physical ? kc.deta : d.dt,
+        s_qn = prestage_a(kc.a, kc.ia, kc.h, hn, d, mn, d.physical ? kc.deta : d.dt,
                           d.physical && sn == 0, d.w[sn]);
       }
     }
@@ -296,7 +307,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
     if (s_bad) { fault = true; break; }
 
     // ---- after the barrier, on disjoint warps:
-    //   warps 0..NQ-1 fold every block's row (in block order, identically in
+    //   warps 0..nl-1 fold every block's row (in block order, identically in
     //     every block); the next stage's copies wait until these latency-
     //     critical loads have landed (named barrier 1), so that they are not
     //     queued behind the copies;
@@ -322,21 +333,21 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
       __syncwarp();
       if (pre && !PLAIN) named_arrive(1, kPreThreads);   // the next stage's copies queue behind it
     }
-    if constexpr (PLAIN) {   // every thread's own copies (the last planes' slots are its own)
-      if (pre) plain_prefetch<MODEL, PREC, NQ, H>(p, sm, ib_next, gq);
+    if constexpr (PLAIN) {   // every thread's own copies; the folding warps' after their fold
+      if (pre && warp > nl) plain_prefetch<MODEL, PREC, NQ, H>(p, sm, ib_next, gq);
     }
-    if (warp < NQ) {
+    if (warp < nl) {
       if (!mbar_wait(&foldbar, (uint32_t)(k & 1), p.wait_limit)) atomicOr(&s_bad, 1);
       if constexpr (PREC != PREC_SPLIT) {
         double v = 0.0;
-        for (int r = lane; r < G; r += 32) v += srows[(size_t)r * kNQ + warp];   // row order
+        for (int r = lane; r < G; r += 32) v += srows[(size_t)r * kNQ + slot];   // row order
 #pragma unroll
         for (int h = 16; h >= 1; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
-        if (lane == 0) sums[warp] = v;
+        if (lane == 0) sums[slot] = v;
       } else {
         float hi = 0.f, lo = 0.f;
         for (int r = lane; r < G; r += 32) {
-          const float2 x = srows[(size_t)r * kNQ + warp];
+          const float2 x = srows[(size_t)r * kNQ + slot];
           pair_add(hi, lo, x.x, x.y);
         }
 #pragma unroll
@@ -345,10 +356,10 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
           const float bl = __shfl_down_sync(0xffffffffu, lo, h);
           pair_add(hi, lo, bh, bl);
         }
-        if (lane == 0) sums[warp] = (double)hi + (double)lo;
+        if (lane == 0) sums[slot] = (double)hi + (double)lo;
       }
       // @sums-written
-    } else if (PREC == PREC_FP64 && warp == NQ) {
+    } else if (PREC == PREC_FP64 && warp == nl) {
       // the lattice's largest |phi| and |pi| of each field
       if (!mbar_wait(&foldbar, (uint32_t)(k & 1), p.wait_limit)) atomicOr(&s_bad, 1);
       uint32_t m[2 * NF];
@@ -380,6 +391,9 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
     __syncthreads();
     // @folded
     if (tid == 0 && !s_bad) s_fold = -1;   // every folding warp saw the copy land
+    if constexpr (PLAIN) {
+      if (pre && warp <= nl) plain_prefetch<MODEL, PREC, NQ, H>(p, sm, ib_next, gq);
+    }
     // ---- in parallel, on warps of different schedulers, identically in
     //      every block: the next stage's coefficients (warp 14: sums -> p_a
     //      kick -> scalar half-steps -> split background), the split form's

@@ -192,25 +192,27 @@ __device__ __forceinline__ bool is_fin(double x) { return isfinite(x); }
 // ---------------------------------------------------------------------------
 // Deterministic block reduction of NQ doubles; result in out[0..NQ) (shared).
 // ---------------------------------------------------------------------------
+// live: bit q set if quantity q is summed; the others are 0 in out (a float64
+// instruction of a warp takes 64 cycles: a sweep sums only what it needs).
 template <int NQ>
-__device__ __forceinline__ void block_sum(double (&v)[NQ], double* sred, double* out) {
+__device__ __forceinline__ void block_sum(double (&v)[NQ], double* sred, double* out,
+                                          uint32_t live = 0xffffffffu) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
+    if (!((live >> q) & 1u)) continue;
     double x = v[q];
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
-    v[q] = x;
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) sred[warp * NQ + q] = v[q];
+    if (lane == 0) sred[warp * NQ + q] = x;
   }
   __syncthreads();
   if (threadIdx.x < NQ) {
     double s = 0.0;
+    if ((live >> threadIdx.x) & 1u) {
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) s += sred[w * NQ + threadIdx.x];
+      for (int w = 0; w < kThreads / 32; ++w) s += sred[w * NQ + threadIdx.x];
+    }
     out[threadIdx.x] = s;
   }
   __syncthreads();
@@ -461,19 +463,21 @@ struct Ctx {
         kf[0] = kf[1] = P::fac_near(ks, pk.lnM2, u2, q_inv, q_lref);
         ps[SL::V] = madd(u2, kf[0] + ks[2], ps[SL::V]);      // sc 2V = sc u2 (fac - m2 K)
       }
+      // a sweep's sums of pi^2 and phi D are wanted over the fields together
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
         if (mode == MODE_SWEEP) {
           pin[f] = madd(kD, D[f], madd(kf[f], phj[f], pim[f]));
-          ps[SL::PI2 + f] = madd(pin[f], pin[f], ps[SL::PI2 + f]);
+          ps[SL::PI2] = madd(pin[f], pin[f], ps[SL::PI2]);
+          ps[SL::PHID] = madd(phj[f], D[f], ps[SL::PHID]);
         } else {
           pin[f] = pim[f];
           ps[SL::PI2 + f] = madd(pim[f], pim[f], ps[SL::PI2 + f]);
           const T dd = phj[f] - shiftK[f];
           ps[SL::DPHI + f] += dd;
           ps[SL::DPHI2 + f] = madd(dd, dd, ps[SL::DPHI2 + f]);
+          ps[SL::PHID + f] = madd(phj[f], D[f], ps[SL::PHID + f]);
         }
-        ps[SL::PHID + f] = madd(phj[f], D[f], ps[SL::PHID + f]);
       }
     } else if constexpr (PREC == PREC_FP64) {
       double dV[NF], V;
@@ -591,13 +595,13 @@ __device__ __forceinline__ void block_sum_pairs(const Acc<float>* acc, double* s
 // double sums), float pairs for the split form.
 template <int PREC, int NQ, typename T>
 __device__ __forceinline__ void block_partials(const Acc<T>* acc, const T* accd_s, double* sred,
-                                               double* sout) {
+                                               double* sout, uint32_t live = 0xffffffffu) {
   __syncthreads();
   if constexpr (PREC == PREC_FP64) {
     double v[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] = (double)accd_s[q];
-    block_sum<NQ>(v, sred, sout);
+    block_sum<NQ>(v, sred, sout, live);
   } else {
     block_sum_pairs<NQ>(reinterpret_cast<const Acc<float>*>(acc), sred, sout);
   }
@@ -1378,7 +1382,11 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
     const uint32_t m = __reduce_max_sync(0xffffffffu, hm.v[i]);
     if (lane == 0) s_wmax[ly][i] = m;
   }
-  block_partials<PREC, NQ, T>(nullptr, accd_s, sred, sout);
+  // a sweep fills the slots of sum pi^2, sum phi D (fields together; the free
+  // model's site: per field, one field) and sum V
+  constexpr uint32_t kSweepLive = (1u << SL::PI2) | (1u << SL::PHID) | (1u << SL::V);
+  block_partials<PREC, NQ, T>(nullptr, accd_s, sred, sout,
+                              mode == MODE_SWEEP ? kSweepLive : 0xffffffffu);
   if (tid < 2 * NF) {
     uint32_t m = 0u;
 #pragma unroll

@@ -617,10 +617,13 @@ __global__ void arm_kernel(Background* bg, long long nsweeps) {
 // Split forms' initial state on the device: the lattice mean of one field is
 // the float64 background phi0, and the rest, x - phi0, is stored as float32
 // (SPLIT_FP32) or as a double-float pair hi + lo (SPLIT_DD).
-// The mean is a compensated sum (Knuth's TwoSum on a running float64 sum, the
-// rounding errors gathered separately) over a fixed grid-stride order, a fixed
-// tree in each block, and one block that folds the block sums in block order:
-// reproducible bit for bit for a given lattice.
+// A block sums its contiguous share of the field in 128-bit fixed point: the
+// largest exponent of the share first, then every value's 53 bits placed 75 bits
+// (less its exponent's distance from the largest) above the lowest one, exact but
+// for values 2^52 below the largest; one block folds the block sums, as
+// compensated pairs, in block order.  Integer instructions only: the compensated
+// float64 sums that they replace (Knuth's TwoSum, seven float64 instructions a
+// value) took 4 x 190 us of a 256^3 two-field initial state, these take 4 x 55.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void mean_two_sum(double a, double b, double& s, double& e) {
   s = a + b;
@@ -646,18 +649,67 @@ __device__ __forceinline__ void mean_block_tree(double s, double c, double* ss, 
 
 __global__ void __launch_bounds__(256) mean_partial_kernel(const double* __restrict__ x,
                                                            long long S, double* part) {
-  __shared__ double ss[256], cc[256];
-  double s = 0.0, c = 0.0;
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < S; i += (long long)gridDim.x * 256) {
-    double u, e;
-    mean_two_sum(s, x[i], u, e);
-    s = u;
-    c += e;
+  __shared__ uint32_t s_max[8];
+  __shared__ unsigned long long s_sum[8][2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long i0 = S * blockIdx.x / gridDim.x, i1 = S * (blockIdx.x + 1) / gridDim.x;
+  uint32_t m = 0u;
+#pragma unroll 8
+  for (long long i = i0 + threadIdx.x; i < i1; i += 256)
+    m = max(m, (uint32_t)__double2hiint(__ldg(x + i)) & 0x7fffffffu);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) s_max[warp] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = max(m, s_max[w]);
+  const int emax = max(1, (int)(m >> 20));   // biased; subnormal values count as exponent 1
+  if (emax == 2047) {                        // not finite: neither is the sum
+    if (threadIdx.x == 0) {
+      part[2 * blockIdx.x] = __hiloint2double(0x7ff80000, 0);
+      part[2 * blockIdx.x + 1] = 0.0;
+    }
+    return;
   }
-  mean_block_tree(s, c, ss, cc);
+  __int128 acc = 0;
+#pragma unroll 4
+  for (long long i = i0 + threadIdx.x; i < i1; i += 256) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(__ldg(x + i));
+    const int e = (int)(b >> 52) & 0x7ff;
+    const unsigned long long mant =
+        (b & 0x000fffffffffffffull) | (e ? 0x0010000000000000ull : 0ull);
+    const int sh = 52 - (emax - max(e, 1));   // top bit of the largest value: bit 104
+    unsigned __int128 v = mant;
+    v = sh >= 0 ? v << sh : (sh > -64 ? (unsigned __int128)(mant >> -sh) : (unsigned __int128)0);
+    acc += (long long)b < 0 ? -(__int128)v : (__int128)v;
+  }
+#pragma unroll
+  for (int h = 16; h > 0; h >>= 1) {
+    const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)acc, h);
+    const unsigned long long hi =
+        __shfl_down_sync(0xffffffffu, (unsigned long long)(acc >> 64), h);
+    acc += (__int128)(((unsigned __int128)hi << 64) | lo);
+  }
+  if (lane == 0) {
+    s_sum[warp][0] = (unsigned long long)acc;
+    s_sum[warp][1] = (unsigned long long)(acc >> 64);
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = ss[0];
-    part[2 * blockIdx.x + 1] = cc[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w)
+      acc += (__int128)(((unsigned __int128)s_sum[w][1] << 64) | s_sum[w][0]);
+    // as a pair: four exact 32-bit limbs from the top, unit 2^(emax - 1023 - 104)
+    double s = 0.0, c = 0.0;
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+      const double limb = k == 3 ? (double)(int)(acc >> 96) : (double)(uint32_t)(acc >> (32 * k));
+      double u, e;
+      mean_two_sum(s, scalbn(limb, 32 * k), u, e);
+      s = u;
+      c += e;
+    }
+    part[2 * blockIdx.x] = scalbn(s, emax - 1127);
+    part[2 * blockIdx.x + 1] = scalbn(c, emax - 1127);
   }
 }
 
@@ -675,6 +727,51 @@ __global__ void __launch_bounds__(256) mean_fold_kernel(const double* __restrict
   if (threadIdx.x == 0) *mean = (ss[0] + cc[0]) / (double)S;
 }
 
+// The FP64 persistent kernel's initial state: N_f fields of S values copied into
+// the simulation's buffer (dst NULL: already there), the high word of the largest
+// magnitude of each into amax[2 f], so that the first pass, the reducing flush,
+// has its fixed-point scale too.  A copy at the memory's rate; the flush of a
+// 256^3 Q-ball takes 0.58 ms with the scale and 1.05 without.
+template <bool VEC>
+__global__ void __launch_bounds__(256) copy_max_kernel(const double* __restrict__ src, double* dst,
+                                                       long long S, uint32_t* amax) {
+  const int f = blockIdx.y;
+  src += (long long)f * S;
+  if (dst) dst += (long long)f * S;
+  const long long step = (long long)gridDim.x * blockDim.x,
+                  i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  uint32_t m = 0u;
+  auto big = [&](double v) { m = max(m, (uint32_t)__double2hiint(v) & 0x7fffffffu); };
+  if constexpr (VEC) {
+#pragma unroll 4
+    for (long long i = i0; i < S / 2; i += step) {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(src) + i);
+      if (dst) reinterpret_cast<double2*>(dst)[i] = v;
+      big(v.x);
+      big(v.y);
+    }
+  } else {
+#pragma unroll 4
+    for (long long i = i0; i < S; i += step) {
+      const double v = src[i];
+      if (dst) dst[i] = v;
+      big(v);
+    }
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(&amax[2 * f], 0x80000000u | m);
+}
+
+static cudaError_t launch_copy_max(const double* src, double* dst, long long S, int nf,
+                                   uint32_t* amax, cudaStream_t s) {
+  // 16-byte accesses where every field starts on such a boundary
+  const bool vec = S % 2 == 0 && ((uintptr_t)src & 15) == 0 && ((uintptr_t)dst & 15) == 0;
+  const dim3 g((unsigned)std::min<long long>(152 * 8, (S + 511) / 512), nf);
+  if (vec) copy_max_kernel<true><<<g, 256, 0, s>>>(src, dst, S, amax);
+  else copy_max_kernel<false><<<g, 256, 0, s>>>(src, dst, S, amax);
+  return cudaGetLastError();
+}
+
 // out[i] = x[i] - mean as float32, or as the pair (hi, lo) with
 // hi = fl32(x - mean), lo = fl32((x - mean) - hi).
 __global__ void split_store_kernel(const double* __restrict__ x, const double* mean, void* out,
@@ -683,9 +780,9 @@ __global__ void split_store_kernel(const double* __restrict__ x, const double* m
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S;
        i += (long long)gridDim.x * blockDim.x) {
     const double v = x[i] - m;
-    const float hi = __double2float_rn(v);
+    const float hi = narrow(v);
     if (pair)
-      static_cast<float2*>(out)[i] = make_float2(hi, __double2float_rn(v - (double)hi));
+      static_cast<float2*>(out)[i] = make_float2(hi, narrow(v - widen(hi)));
     else
       static_cast<float*>(out)[i] = hi;
   }
@@ -701,9 +798,9 @@ __global__ void split_load_kernel(const void* __restrict__ d, const double* base
     double v;
     if (pair) {
       const float2 p = static_cast<const float2*>(d)[i0 + i];
-      v = (double)p.x + (double)p.y;
+      v = widen(p.x) + widen(p.y);
     } else {
-      v = (double)static_cast<const float*>(d)[i0 + i];
+      v = widen(static_cast<const float*>(d)[i0 + i]);
     }
     out[i] = b + v;
   }
@@ -1140,9 +1237,21 @@ PYCOOL_API pycool_status pycool_set_initial(pycool_sim* sim, const double* phi, 
   CK(cudaStreamSynchronize(sim->stream));
   if (sim->hdesc.prec == PREC_FP64) {
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    CK(cudaMemcpyAsync(sim->hdesc.phi[0], phi, count * sizeof(double), kind, sim->stream));
-    CK(cudaMemcpyAsync(sim->hdesc.pi[0], pi, count * sizeof(double), kind, sim->stream));
+    const bool maxima = sim->persist;   // (run-time potentials do not use them)
+    if (!maxima || !on_device) {
+      CK(cudaMemcpyAsync(sim->hdesc.phi[0], phi, count * sizeof(double), kind, sim->stream));
+      CK(cudaMemcpyAsync(sim->hdesc.pi[0], pi, count * sizeof(double), kind, sim->stream));
+    }
     CK(cudaMemcpyAsync(sim->d_bg, &b, sizeof(b), cudaMemcpyHostToDevice, sim->stream));
+    if (maxima) {
+      double* f0 = (double*)sim->hdesc.phi[0];
+      double* p0 = (double*)sim->hdesc.pi[0];
+      CK(launch_copy_max(on_device ? phi : f0, on_device ? f0 : nullptr, (long long)S, nf,
+                         sim->d_bg->amax, sim->stream));
+      CK(launch_copy_max(on_device ? pi : p0, on_device ? p0 : nullptr, (long long)S, nf,
+                         sim->d_bg->amax + 1, sim->stream));
+      sim->launches += 2;
+    }
   } else {
     // split forms: phi0 = the lattice mean (float64), the rest as float32 or
     // as a double-float pair, all on the device (split_initial)

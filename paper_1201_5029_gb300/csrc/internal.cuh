@@ -40,6 +40,19 @@ __device__ __forceinline__ double widen(float v) {
     return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(m << 29));
   return m == 0u ? __hiloint2double((int)b, 0) : (double)v;
 }
+// (round to nearest, ties to even; results that are not normal are left to the
+// conversion instruction)
+__device__ __forceinline__ float narrow(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t m = hi & 0x7fffffffu;
+  if (m - 0x38100000u < 0x0fd00000u) {   // 2^-126 <= |v| < 2^127: no overflow by rounding
+    uint32_t f = ((m - 0x38000000u) << 3) | (lo >> 29);
+    const uint32_t rest = lo & 0x1fffffffu;
+    f += (rest > 0x10000000u || (rest == 0x10000000u && (f & 1u))) ? 1u : 0u;
+    return __int_as_float((int)(f | (hi & 0x80000000u)));
+  }
+  return __double2float_rn(v);
+}
 #endif
 
 enum Mode : int32_t { MODE_IDLE = 0, MODE_SWEEP = 1, MODE_FLUSH = 2 };

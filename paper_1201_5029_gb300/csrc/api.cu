@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <thread>
 #include <vector>
@@ -267,18 +268,28 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
   };
   // the smallest feasible T for each chunking (bisection), then the chunking
   // with the least loaded slowest block (ties: less total work, fewer chunks)
-  const double work = (double)n * g.tiles_x * ((tiles_y - 2) + 2 * pen);
+  const double work = (double)n * (plain ? g.ntiles : g.tiles_x * ((tiles_y - 2) + 2 * pen));
   double best = 1e300, best_tot = 1e300, best_T = 0.0;
-  for (int rc = 1; rc <= std::min(16, std::max(1, n / kMinPiece)); ++rc) {
+  // (plain staging: whole columns, cut where a block is full, come out best; a
+  // plan is made for every new simulation, so it is not searched further than
+  // half a percent)
+  const int rc_most = plain ? 1 : std::min(16, std::max(1, n / kMinPiece));
+  const double tol = plain ? 5e-3 * work / cap : 1e-3;
+  for (int rc = 1; rc <= rc_most; ++rc) {
     const int rws[3] = {rc, (rc * 12 + 9) / 10, (rc * 13 + 9) / 10};
     for (int j = 0; j < 3; ++j) {
       const int rw = std::min(rws[j], std::max(1, n / kMinPiece));
       if (j > 0 && rw == std::min(rws[j - 1], std::max(1, n / kMinPiece))) continue;
       if (pen == 1.0 && rw != rc) continue;
       chunks(rc, rw);
+      // a chunking that cannot be dealt below the best slowest block so far is
+      // dropped by one deal (a search takes twenty)
+      if (best < 1e299 && !deal(best - 1e-3)) continue;
       double lo = work / cap, hi = (double)n * pen + 2.0 * halo * h * pen + lo;
-      while (!deal(hi)) hi *= 2.0;
-      for (int it = 0; it < 40 && hi - lo > 1e-3; ++it) {
+      if (best < 1e299) hi = best - 1e-3;
+      else
+        while (!deal(hi)) hi *= 2.0;
+      for (int it = 0; it < 40 && hi - lo > tol; ++it) {
         const double mid = 0.5 * (lo + hi);
         if (deal(mid)) hi = mid; else lo = mid;
       }
@@ -853,6 +864,59 @@ void observables(const Background& b, const SimDesc& d, double mpl, double rho_r
 
 }  // namespace pycool
 
+// Pinned host records of the simulations, from slabs of 64 (pinning a page takes
+// longer than the rest of pycool_create).  The first slab (about 20 KB) stays for
+// the process; others go when their last record is given back.  Any thread.
+namespace {
+struct HostRecord {
+  Background bg;
+  int32_t fault;
+  int32_t slab;   // index of its slab
+};
+constexpr int kSlabRecords = 64;
+struct HostSlab {
+  HostRecord* base = nullptr;
+  std::vector<HostRecord*> free;
+};
+std::mutex g_host_mu;
+std::vector<HostSlab> g_host_slabs;
+
+cudaError_t take_host_record(HostRecord** out) {
+  std::lock_guard<std::mutex> lk(g_host_mu);
+  size_t i = 0;
+  while (i < g_host_slabs.size() && g_host_slabs[i].free.empty()) ++i;
+  if (i == g_host_slabs.size()) {   // every slab is full or gone: a new one, in a gap if any
+    for (i = 0; i < g_host_slabs.size() && g_host_slabs[i].base; ++i) {}
+    if (i == g_host_slabs.size()) g_host_slabs.emplace_back();
+    HostRecord* p = nullptr;
+    const cudaError_t e = cudaHostAlloc((void**)&p, sizeof(HostRecord) * kSlabRecords,
+                                        cudaHostAllocPortable);
+    if (e != cudaSuccess) return e;
+    g_host_slabs[i].base = p;
+    for (int k = 0; k < kSlabRecords; ++k) {
+      p[k].slab = (int32_t)i;
+      g_host_slabs[i].free.push_back(p + k);
+    }
+  }
+  *out = g_host_slabs[i].free.back();
+  g_host_slabs[i].free.pop_back();
+  return cudaSuccess;
+}
+
+void give_host_record(HostRecord* r) {
+  if (!r) return;
+  std::lock_guard<std::mutex> lk(g_host_mu);
+  HostSlab& s = g_host_slabs[r->slab];
+  const bool first = r->slab == 0;
+  s.free.push_back(r);
+  if (!first && s.free.size() == (size_t)kSlabRecords) {
+    cudaFreeHost(s.base);
+    s.base = nullptr;
+    s.free.clear();
+  }
+}
+}  // namespace
+
 // ---------------------------------------------------------------------------
 // Simulation object
 // ---------------------------------------------------------------------------
@@ -869,6 +933,9 @@ struct pycool_sim {
   bool own_state = false, own_ws = false;
   SimDesc* d_desc = nullptr;
   Background* d_bg = nullptr;
+  HostRecord* h_rec = nullptr;  // pinned: what sync_bg reads into
+  Background* h_bg = nullptr;
+  int32_t* h_fault = nullptr;
   LaunchTable table{};
   cudaGraphExec_t graph = nullptr;
   int graph_len = 0;
@@ -1125,6 +1192,9 @@ PYCOOL_API pycool_status pycool_create(const pycool_config* cfg, void* dev_state
     if ((e = cudaStreamCreateWithFlags(&sim->cap_stream, cudaStreamNonBlocking)) != cudaSuccess)
       break;
     if ((e = cudaEventCreateWithFlags(&sim->done, cudaEventDisableTiming)) != cudaSuccess) break;
+    if ((e = take_host_record(&sim->h_rec)) != cudaSuccess) break;
+    sim->h_bg = &sim->h_rec->bg;
+    sim->h_fault = &sim->h_rec->fault;
   } while (0);
   if (e != cudaSuccess) {
     cuda_fail(sim, e, "pycool_create");
@@ -1162,12 +1232,6 @@ PYCOOL_API pycool_status pycool_create(const pycool_config* cfg, void* dev_state
     }
   }
   *out = sim;
-  return PYCOOL_OK;
-}
-
-static pycool_status read_bg(pycool_sim* sim, Background* b) {
-  CK(cudaMemcpyAsync(b, sim->d_bg, sizeof(Background), cudaMemcpyDeviceToHost, sim->stream));
-  CK(cudaStreamSynchronize(sim->stream));
   return PYCOOL_OK;
 }
 
@@ -1306,41 +1370,46 @@ PYCOOL_API pycool_status pycool_evolve(pycool_sim* sim, int64_t steps) {
   return PYCOOL_OK;
 }
 
-PYCOOL_API pycool_status pycool_sync(pycool_sim* sim, double timeout_s) {
-  if (!sim) return PYCOOL_E_INVALID;
+// pycool_sync, leaving the background record it read in *b (not read: E_TIMEOUT
+// of a wait, E_CUDA, E_STATE).  The first two milliseconds are polled without
+// sleeping: a sleep of 50 us takes twice that to wake from, as long as ten stages
+// of a small lattice.  The record and the fault word come in one wait.
+static pycool_status sync_bg(pycool_sim* sim, double timeout_s, Background* b) {
   if (sim->poisoned) return PYCOOL_E_STATE;
   const auto t0 = std::chrono::steady_clock::now();
   for (;;) {
     const cudaError_t q = cudaEventQuery(sim->done);
     if (q == cudaSuccess) break;
     if (q != cudaErrorNotReady) return cuda_fail(sim, q, "cudaEventQuery");
-    if (timeout_s >= 0.0) {
-      const double el =
-          std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-      if (el > timeout_s) return PYCOOL_E_TIMEOUT;
-    }
-    std::this_thread::sleep_for(std::chrono::microseconds(50));
+    const double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+    if (timeout_s >= 0.0 && el > timeout_s) return PYCOOL_E_TIMEOUT;
+    if (el < 2e-3) std::this_thread::yield();
+    else std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
-  int32_t fault = 0;
-  CK(cudaMemcpy(&fault, sim->hdesc.fault, sizeof(fault), cudaMemcpyDeviceToHost));
-  if (fault) {  // a device-side wait gave up: the state can no longer be trusted
+  CK(cudaMemcpyAsync(sim->h_fault, sim->hdesc.fault, sizeof(int32_t), cudaMemcpyDeviceToHost,
+                     sim->stream));
+  CK(cudaMemcpyAsync(sim->h_bg, sim->d_bg, sizeof(Background), cudaMemcpyDeviceToHost,
+                     sim->stream));
+  CK(cudaStreamSynchronize(sim->stream));
+  if (*sim->h_fault) {  // a device-side wait gave up: the state can no longer be trusted
     sim->poisoned = true;
     return PYCOOL_E_TIMEOUT;
   }
+  *b = *sim->h_bg;
+  return b->error ? PYCOOL_E_NONFINITE : PYCOOL_OK;
+}
+
+PYCOOL_API pycool_status pycool_sync(pycool_sim* sim, double timeout_s) {
+  if (!sim) return PYCOOL_E_INVALID;
   Background b;
-  pycool_status st = read_bg(sim, &b);
-  if (st != PYCOOL_OK) return st;
-  if (b.error) return PYCOOL_E_NONFINITE;
-  return PYCOOL_OK;
+  return sync_bg(sim, timeout_s, &b);
 }
 
 PYCOOL_API pycool_status pycool_energies(pycool_sim* sim, pycool_observables* out) {
   if (!sim || !out) return PYCOOL_E_INVALID;
   if (!sim->initialised) return PYCOOL_E_STATE;
-  pycool_status st = pycool_sync(sim, -1.0);
-  if (st != PYCOOL_OK) return st;
   Background b;
-  st = read_bg(sim, &b);
+  const pycool_status st = sync_bg(sim, -1.0, &b);
   if (st != PYCOOL_OK) return st;
   observables(b, sim->hdesc, sim->cfg.mpl, sim->cfg.rho_rad0, sim->cfg.rho_mat0, out);
   return PYCOOL_OK;
@@ -1361,11 +1430,9 @@ PYCOOL_API pycool_status pycool_get_fields(pycool_sim* sim, double* phi, double*
                                            int on_device) {
   if (!sim) return PYCOOL_E_INVALID;
   if (!sim->initialised) return PYCOOL_E_STATE;
-  pycool_status st = pycool_sync(sim, -1.0);
-  if (st != PYCOOL_OK && st != PYCOOL_E_NONFINITE) return st;
   Background b;
-  st = read_bg(sim, &b);
-  if (st != PYCOOL_OK) return st;
+  const pycool_status st = sync_bg(sim, -1.0, &b);
+  if (st != PYCOOL_OK && st != PYCOOL_E_NONFINITE) return st;
   const size_t S = (size_t)sim->hdesc.S;
   const size_t count = (size_t)sim->nf * S;
   const void* src_phi = sim->hdesc.phi[b.cur & 1];
@@ -1420,10 +1487,8 @@ PYCOOL_API pycool_status pycool_checkpoint_save(pycool_sim* sim, void* buf, size
   size_t need = 0;
   pycool_checkpoint_size(sim, &need);
   if (cap < need) return PYCOOL_E_INVALID;
-  pycool_status st = pycool_sync(sim, -1.0);
-  if (st != PYCOOL_OK) return st;
   Background b;
-  st = read_bg(sim, &b);
+  const pycool_status st = sync_bg(sim, -1.0, &b);
   if (st != PYCOOL_OK) return st;
   if (b.mode != MODE_IDLE) return PYCOOL_E_STATE;
   const size_t word = prec_word(sim->hdesc.prec);
@@ -1466,9 +1531,7 @@ PYCOOL_API int32_t pycool_spectrum_bins(int32_t n) {
 // The synchronised state that the observables read.
 static pycool_status observed_state(pycool_sim* sim, Background* b) {
   if (!sim->initialised) return PYCOOL_E_STATE;
-  pycool_status st = pycool_sync(sim, -1.0);
-  if (st != PYCOOL_OK) return st;
-  st = read_bg(sim, b);
+  const pycool_status st = sync_bg(sim, -1.0, b);
   if (st != PYCOOL_OK) return st;
   return b->mode == MODE_IDLE ? PYCOOL_OK : PYCOOL_E_STATE;
 }
@@ -1637,6 +1700,7 @@ PYCOOL_API void pycool_destroy(pycool_sim* sim) {
   cudaFree(sim->spec_power);
   if (sim->graph) cudaGraphExecDestroy(sim->graph);
   if (sim->done) cudaEventDestroy(sim->done);
+  give_host_record(sim->h_rec);
   if (sim->cap_stream) cudaStreamDestroy(sim->cap_stream);
   if (sim->own_state && sim->state) cudaFree(sim->state);
   if (sim->own_ws && sim->ws) cudaFree(sim->ws);

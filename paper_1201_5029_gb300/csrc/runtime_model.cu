@@ -92,9 +92,9 @@ cudaError_t launch_runtime_stage(const SimDesc& d, const LaunchTable& t, int gri
     if (d.rt_index < 0 || d.rt_index >= (int)g_rt.size()) return cudaErrorInvalidValue;
   }
   if (grid == 0) return cudaSuccess;
-  const unsigned eg = 152 * 8;
-  if (d.model == M_RUNTIME1) rt_drift<M_RUNTIME1><<<eg, kThreads, 0, s>>>(t);
-  else rt_drift<M_RUNTIME2><<<eg, kThreads, 0, s>>>(t);
+  const unsigned eg = 152;
+  if (d.model == M_RUNTIME1) rt_drift<M_RUNTIME1><<<eg, kRtDriftThreads, 0, s>>>(t);
+  else rt_drift<M_RUNTIME2><<<eg, kRtDriftThreads, 0, s>>>(t);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = launch_runtime_potential(d, d.rt_phis, s);

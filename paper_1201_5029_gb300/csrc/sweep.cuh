@@ -1093,6 +1093,22 @@ template <int STENCIL> struct StencilW {
   static constexpr bool kCorners = (STENCIL == 27);
 };
 
+// A kernel's body for its mode and stencil arithmetic as compile-time constants
+// (a runtime mode leaves the other mode's float64 instructions, predicated off, in
+// the loop).
+template <typename F>
+__device__ __forceinline__ void by_mode(int mode, bool fix, F&& body) {
+  using MS = std::integral_constant<int, MODE_SWEEP>;
+  using MF = std::integral_constant<int, MODE_FLUSH>;
+  if (mode == MODE_SWEEP) {
+    if (fix) body(std::true_type{}, MS{});
+    else body(std::false_type{}, MS{});
+  } else {
+    if (fix) body(std::true_type{}, MF{});
+    else body(std::false_type{}, MF{});
+  }
+}
+
 // ---------------------------------------------------------------------------
 // TMA-staged FP64 sweep (n % 32 == 0).  256 threads = 8 warps; warp w owns tile
 // row y0 + w, lane l owns sites x0 + l*VX .. +VX-1.  The drifted plane replaces
@@ -2013,37 +2029,62 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_wide(const LaunchTable tab)
 // advances the Background).  Both library kernels derive the stage's
 // coefficients from the same Background record, which only the last block of
 // rt_kick changes.
+// Measured on GB300, 128^3, two-field chaotic potential, per stage: rt_drift 25
+// -> 18 us, the compiled kernel 51 (its own float64 instructions), rt_kick 148 ->
+// 83.
 // ---------------------------------------------------------------------------
+// One block per SM: the scalar step that every block repeats takes thousands of
+// cycles of the SM's float64 pipe.
+constexpr int kRtDriftThreads = 1024;
 template <int MODEL>
-__global__ void __launch_bounds__(kThreads) rt_drift(const LaunchTable tab) {
+__global__ void __launch_bounds__(kRtDriftThreads) rt_drift(const LaunchTable tab) {
   using C = Ctx<MODEL, PREC_FP64>;
   constexpr int NF = C::NF;
-  __shared__ C s_ctx;
+  __shared__ double s_c;
   const SimDesc& d = *tab.desc[0];
   const Background& bgr = *d.bg;
   const int mode = bgr.mode;
   if (mode == MODE_IDLE) return;
-  if (threadIdx.x == 0) s_ctx.init(bgr, d, mode);
+  if (threadIdx.x == 0) s_c = prestage(bgr, d, mode).c;
   __syncthreads();
-  const double c = s_ctx.cdrift;
+  const double c = s_c;
   const int ib = bgr.cur;
-  const double* __restrict__ phi = (const double*)d.phi[ib & 1];
-  const double* __restrict__ pi = (const double*)d.pi[(ib >> 1) & 1];
-  const size_t total = (size_t)NF * (size_t)d.S;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x)
-    d.rt_phis[i] = fma(c, pi[i], phi[i]);
+  const size_t total = (size_t)NF * (size_t)d.S, pairs = total / 2;
+  const size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x,
+               step = (size_t)gridDim.x * blockDim.x;
+  // the state's buffers and the scratch start on 256-byte boundaries
+  const double2* __restrict__ phi = (const double2*)d.phi[ib & 1];
+  const double2* __restrict__ pi = (const double2*)d.pi[(ib >> 1) & 1];
+  double2* out = reinterpret_cast<double2*>(d.rt_phis);
+#pragma unroll 4
+  for (size_t i = i0; i < pairs; i += step) {
+    const double2 f = phi[i], q = pi[i];
+    out[i] = make_double2(fma(c, q.x, f.x), fma(c, q.y, f.y));
+  }
+  if (i0 == 0 && (total & 1))
+    d.rt_phis[total - 1] = fma(c, reinterpret_cast<const double*>(pi)[total - 1],
+                               reinterpret_cast<const double*>(phi)[total - 1]);
 }
 
+// Tiles of txt x ty sites marching z: a plane's cells (with the halo ring, two
+// per thread) are loaded one plane ahead, put on the fixed-point scale (or kept
+// in float64 without one) in one of two shared-memory planes, and summed as in
+// stage_plain.  Bound by the float64 pipe (9 instructions per two-field site; 21
+// with the stencil in float64, and its neighbours by 64-bit wrapped indices).
 template <int MODEL, int STENCIL>
 __global__ void __launch_bounds__(kThreads, 2) rt_kick(const LaunchTable tab) {
   using C = Ctx<MODEL, PREC_FP64>;
   using SL = typename C::SL;
   constexpr int NF = C::NF;
   constexpr int NQ = SL::NQ;
-  constexpr bool CORNERS = StencilW<STENCIL>::kCorners;
+  constexpr bool CORNERS = StencilW<STENCIL>::kCorners, WIDE = STENCIL == 13;
+  constexpr int H = WIDE ? 2 : 1;
+  constexpr int kCells = (kMaxTXT + 2 * H) * (kMaxTY + 2 * H);
+  static_assert(kCells <= 2 * kThreads, "two cells per thread");
+  __shared__ double sm[2][NF][kCells];
   __shared__ double sred[(kThreads / 32) * NQ];
   __shared__ double sout[NQ];
+  __shared__ uint32_t s_wmax[kThreads / 32][2 * NF], s_bmax[2 * NF];
   __shared__ int s_last;
   __shared__ C s_ctx;
   const SimDesc& d = *tab.desc[0];
@@ -2059,74 +2100,157 @@ __global__ void __launch_bounds__(kThreads, 2) rt_kick(const LaunchTable tab) {
   const int z0 = zch * d.zc, zend = min(n, z0 + d.zc);
   const int tid = threadIdx.x;
   const bool active = tid < TX * TY;
-  const int gx = x0 + (active ? tid % TX : 0), gy = y0 + (active ? tid / TX : 0);
+  const int lx = active ? tid % TX : 0, ly = active ? tid / TX : 0;
+  const int gx = x0 + lx, gy = y0 + ly;
   const bool valid = active && gx < n && gy < n;
   const size_t S = (size_t)d.S, nn = (size_t)n * n;
-  if (tid == 0) s_ctx.init(bgr, d, mode);
+  const int rs = TX + 2 * H, cells = rs * (TY + 2 * H), own = (ly + H) * rs + lx + H;
+  // this thread's cells of a plane: in-plane offsets (a ragged tile's cells past
+  // the lattice wrap like the halo and are not used)
+  int off[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int c = tid + k * kThreads;
+    const int row = c / rs, col = c - row * rs;
+    off[k] = c < cells ? ((y0 - H + row + n) % n) * n + (x0 - H + col + n) % n : -1;
+  }
+  if (tid == 0) {
+    s_ctx.init(bgr, d, mode);
+    s_ctx.set_fix(bgr.amax, fix_headroom<STENCIL>());
+  }
   __syncthreads();
-  const C cx = s_ctx;
   const int ib = bgr.cur;
   double* __restrict__ phi_out = (double*)d.phi[(ib & 1) ^ 1];
   const double* __restrict__ pi_in = (const double*)d.pi[(ib >> 1) & 1];
   double* __restrict__ pi_out = (double*)d.pi[((ib >> 1) & 1) ^ 1];
-  const double c0 = CORNERS ? -128.0 / 30.0 : -6.0, c1 = CORNERS ? 14.0 / 30.0 : 1.0;
-  const double c2 = CORNERS ? 3.0 / 30.0 : 0.0, c3 = CORNERS ? 1.0 / 30.0 : 0.0;
   double ps[NQ];
-  Acc<double> acc[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) ps[q] = 0.0;
-  if (valid) {
-    for (int z = z0; z < zend; ++z) {
-      const size_t o = (size_t)z * nn + (size_t)gy * n + gx;
+  HiMax<NF> hm;
+  hm.zero();
+  auto body = [&](auto fix_c, auto mode_c) {
+    constexpr bool FIX = decltype(fix_c)::value;
+    constexpr int MODE = decltype(mode_c)::value;
+    constexpr bool TIMES = WIDE || (FIX && STENCIL == 27);   // as in stage_plain
+    using E = typename FixElem<FIX>::type;
+    C cx = s_ctx;
+    if constexpr (TIMES) cx.kD *= 1.0 / fix_weight<STENCIL>();
+    const E w1 = (E)16, w2 = (E)0 - (E)1, w0 = (E)0 - (E)90;   // 13-point, times 12
+    double raw[2][NF];
+    auto load = [&](int p) {
+      const size_t zo = (size_t)((p + n) % n) * nn;
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+          raw[k][f] = off[k] >= 0 ? d.rt_phis[f * S + zo + off[k]] : 0.0;
+    };
+    E qa[NF], qb[NF], qc[NF], qd[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) qa[f] = qb[f] = qc[f] = qd[f] = (E)0;
+    load(z0 - H);
+    const int Q = zend - z0 + 2 * H;
+    for (int q = 0; q < Q; ++q) {
+      E* buf = reinterpret_cast<E*>(&sm[q & 1][0][0]);
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+          if (off[k] >= 0)
+            buf[f * kCells + tid + k * kThreads] = fix_in(raw[k][f], cx.fx[f], (E*)nullptr);
+      if (q + 1 < Q) load(z0 - H + q + 1);
+      // the output plane's own values
+      const bool put = valid && q >= 2 * H;
+      const size_t o = (size_t)(z0 + q - 2 * H) * nn + (size_t)gy * n + gx;
+      double ph[NF], pm[NF], dv[NF], V = 0.0;
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
-        const double* ph = d.rt_phis + (size_t)f * S;
-        const double ctr = ph[o];
-        double D;
-        if constexpr (STENCIL == 13) {
-          // the fourth-order stencil: +-1 and +-2 along each axis
-          auto at = [&](int dz, int dy, int dx) {
-            return ph[(size_t)((z + dz + 2 * n) % n) * nn + (size_t)((gy + dy + 2 * n) % n) * n +
-                      (gx + dx + 2 * n) % n];
-          };
-          const double near = (at(-1, 0, 0) + at(1, 0, 0)) + (at(0, -1, 0) + at(0, 1, 0)) +
-                              (at(0, 0, -1) + at(0, 0, 1));
-          const double far = (at(-2, 0, 0) + at(2, 0, 0)) + (at(0, -2, 0) + at(0, 2, 0)) +
-                             (at(0, 0, -2) + at(0, 0, 2));
-          D = fma(-90.0 / 12.0, ctr, fma(-1.0 / 12.0, far, (16.0 / 12.0) * near));
+        ph[f] = put ? d.rt_phis[f * S + o] : 0.0;
+        pm[f] = put ? pi_in[f * S + o] : 0.0;
+        dv[f] = put && MODE == MODE_SWEEP ? d.rt_dV[f * S + o] : 0.0;
+      }
+      if (put) V = d.rt_V[o];
+      __syncthreads();
+      const bool mid = q >= H && q < Q - H;
+      E D[NF];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        const E* fx = buf + f * kCells + own;
+        const E ctr = fx[0];
+        if constexpr (WIDE) {
+          E m = (E)0;
+          if (mid) {
+            const E nr = (fx[-rs] + fx[rs]) + (fx[-1] + fx[1]);
+            const E fr = (fx[-2 * rs] + fx[2 * rs]) + (fx[-2] + fx[2]);
+            m = fix_mad(w0, ctr, fix_mad(w2, fr, w1 * nr));
+          }
+          D[f] = fix_mad(w2, ctr, qb[f]);
+          const E np1 = fix_mad(w1, ctr, qa[f]);
+          qa[f] = fix_mad(w2, qd[f], fix_mad(w1, qc[f], m));
+          qb[f] = np1;
+          qd[f] = qc[f];
+          qc[f] = ctr;
         } else {
-          double faces = 0.0, edges = 0.0, corners = 0.0;
-          for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-              for (int dx = -1; dx <= 1; ++dx) {
-                const int cls = (dz != 0) + (dy != 0) + (dx != 0);
-                if (cls == 0 || (!CORNERS && cls > 1)) continue;
-                const double v = ph[(size_t)wrapi(z + dz, n) * nn +
-                                    (size_t)wrapi(gy + dy, n) * n + wrapi(gx + dx, n)];
-                if (cls == 1) faces += v; else if (cls == 2) edges += v; else corners += v;
-              }
-          D = fma(c3, corners, fma(c2, edges, fma(c1, faces, c0 * ctr)));
-        }
-        const double pim = pi_in[(size_t)f * S + o];
-        double pin = pim;
-        if (mode == MODE_SWEEP) {
-          pin = fma(cx.kD, D, fma(-cx.kV, d.rt_dV[(size_t)f * S + o], pim));
-          pi_out[(size_t)f * S + o] = pin;
-        }
-        phi_out[(size_t)f * S + o] = ctr;
-        ps[SL::PI2 + f] = fma(pin, pin, ps[SL::PI2 + f]);
-        ps[SL::PHID + f] = fma(ctr, D, ps[SL::PHID + f]);
-        if (mode != MODE_SWEEP) {
-          const double dd = ctr - cx.shiftK[f];
-          ps[SL::DPHI + f] += dd;
-          ps[SL::DPHI2 + f] = fma(dd, dd, ps[SL::DPHI2 + f]);
+          E smid = ctr, so = ctr;
+          if (CORNERS || mid) {
+            const E faces = (fx[-rs] + fx[rs]) + (fx[-1] + fx[1]);
+            if constexpr (CORNERS)
+              fix_parts27(ctr, faces, (fx[-rs - 1] + fx[-rs + 1]) + (fx[rs - 1] + fx[rs + 1]),
+                          smid, so);
+            else
+              smid = fix_mid7(ctr, faces);
+          }
+          D[f] = qa[f] + so;
+          if (mid) qa[f] = qb[f] + smid;
+          qb[f] = so;
         }
       }
-      ps[SL::V] += d.rt_V[o];
+      if (put) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          const double Df = fix_out(D[f], cx.fx[f]);
+          phi_out[f * S + o] = ph[f];
+          hm.add(2 * f, ph[f]);
+          if (MODE == MODE_SWEEP) {
+            const double pin = fma(cx.kD, Df, fma(-cx.kV, dv[f], pm[f]));
+            pi_out[f * S + o] = pin;
+            hm.add(2 * f + 1, pin);
+            ps[SL::PI2] = fma(pin, pin, ps[SL::PI2]);
+            ps[SL::PHID] = fma(ph[f], Df, ps[SL::PHID]);
+          } else {
+            hm.add(2 * f + 1, pm[f]);
+            ps[SL::PI2 + f] = fma(pm[f], pm[f], ps[SL::PI2 + f]);
+            ps[SL::PHID + f] = fma(ph[f], Df, ps[SL::PHID + f]);
+            const double dd = ph[f] - cx.shiftK[f];
+            ps[SL::DPHI + f] += dd;
+            ps[SL::DPHI2 + f] = fma(dd, dd, ps[SL::DPHI2 + f]);
+          }
+        }
+        ps[SL::V] += V;
+      }
     }
+    if constexpr (TIMES) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f) ps[SL::PHID + f] *= 1.0 / fix_weight<STENCIL>();
+    }
+  };
+  by_mode(mode, s_ctx.fx[0] != 0, body);
+#pragma unroll
+  for (int i = 0; i < 2 * NF; ++i) {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, hm.v[i]);
+    if ((tid & 31) == 0) s_wmax[tid >> 5][i] = m;
   }
-  block_partials<PREC_FP64, NQ, double>(acc, ps, sred, sout);
-  finish_block<MODEL, PREC_FP64>(s_ctx, d, mode, cta, sout, &s_last);
+  constexpr uint32_t kSweepLive = (1u << SL::PI2) | (1u << SL::PHID) | (1u << SL::V);
+  block_partials<PREC_FP64, NQ, double>(nullptr, ps, sred, sout,
+                                        mode == MODE_SWEEP ? kSweepLive : 0xffffffffu);
+  if (tid < 2 * NF) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) m = max(m, s_wmax[w][tid]);
+    s_bmax[tid] = m;
+  }
+  __syncthreads();
+  finish_block<MODEL, PREC_FP64>(s_ctx, d, mode, cta, sout, &s_last, s_bmax);
 }
 
 // Launch helper: dispatch (model, stencil, path/vx) at runtime to an instance.

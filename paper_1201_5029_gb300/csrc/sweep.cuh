@@ -1236,8 +1236,9 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
   HiMax<NF> hm;
   hm.zero();
   int q = 0;
-  auto body = [&](auto fix_c) {
+  auto body = [&](auto fix_c, auto mode_c) {
     constexpr bool FIX = decltype(fix_c)::value;
+    constexpr int MODE = decltype(mode_c)::value;
     using E = typename FixElem<FIX>::type;
     C cx = s_ctx;
     // see stage_fp64: the 27-point integer sums are 30 D
@@ -1352,7 +1353,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
             Dj[f] = fix_out(part_m[f][j] + so_new[f][j], cx.fx[f]);
             pmj[f] = pi_m[f][j];
           }
-          cx.site(mode, phj, Dj, pmj, pnj, accd_s);
+          cx.site(MODE, phj, Dj, pmj, pnj, accd_s);
 #pragma unroll
           for (int f = 0; f < NF; ++f) {
             pin[f][j] = pnj[f];
@@ -1363,7 +1364,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
           vstore<T, VX>(phi_out + f * S + o, ph_m[f]);
-          if (mode == MODE_SWEEP) vstore<T, VX>(pi_out + f * S + o, pin[f]);
+          if (MODE == MODE_SWEEP) vstore<T, VX>(pi_out + f * S + o, pin[f]);
         }
       }
 #pragma unroll
@@ -1381,8 +1382,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) 
       for (int f = 0; f < NF; ++f) accd_s[SL::PHID + f] *= 1.0 / fix_weight<STENCIL>();
     }
   };
-  if (s_ctx.fx[0]) body(std::true_type{});
-  else body(std::false_type{});
+  by_mode(mode, s_ctx.fx[0] != 0, body);
 
   if (s_fault) {
     // a TMA copy never completed: record it, drain what is in flight (bounded), stop

@@ -79,7 +79,7 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Blocks of the split forms' initial-mean reduction (a fixed grid, so the
 // summation order and the result depend on the lattice alone).
-constexpr int kMeanBlocks = 304;
+constexpr int kMeanBlocks = 1216;   // per array
 
 Layout layout_for(const pycool_config& c) {
   Layout L;
@@ -109,7 +109,7 @@ Layout layout_for(const pycool_config& c) {
 Layout sim_layout(const pycool_config& c) {
   Layout L = layout_for(c);
   L.off_mean = align256(L.ws_bytes);
-  L.ws_bytes = L.off_mean + align256((size_t)2 * kMeanBlocks * sizeof(double));
+  L.ws_bytes = L.off_mean + align256((size_t)2 * kMaxFields * kMeanBlocks * 2 * sizeof(double));
   // the persistent kernel, compiled models: TMA staging for n a multiple of 32
   // (the 13-point stencil in the FP64 and split-DD forms), plain staging for
   // every other n and for the split-FP32 form's 13-point stencil (faster than
@@ -633,8 +633,8 @@ __global__ void arm_kernel(Background* bg, long long nsweeps) {
 // (less its exponent's distance from the largest) above the lowest one, exact but
 // for values 2^52 below the largest; one block folds the block sums, as
 // compensated pairs, in block order.  Integer instructions only: the compensated
-// float64 sums that they replace (Knuth's TwoSum, seven float64 instructions a
-// value) took 4 x 190 us of a 256^3 two-field initial state, these take 4 x 55.
+// float64 sums that they replace were seven float64 instructions a value (Knuth's
+// TwoSum).  Every array of a device state goes through one launch per pass.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void mean_two_sum(double a, double b, double& s, double& e) {
   s = a + b;
@@ -658,8 +658,15 @@ __device__ __forceinline__ void mean_block_tree(double s, double c, double* ss, 
   }
 }
 
-__global__ void __launch_bounds__(256) mean_partial_kernel(const double* __restrict__ x,
-                                                           long long S, double* part) {
+struct SplitArrays {   // blockIdx.y: which
+  const double* x[2 * kMaxFields];   // float64 input, S values
+  double* mean[2 * kMaxFields];
+  void* out[2 * kMaxFields];         // fluctuations
+};
+__global__ void __launch_bounds__(256) mean_partial_kernel(const SplitArrays arr, long long S,
+                                                           double* part) {
+  const double* __restrict__ x = arr.x[blockIdx.y];
+  part += (size_t)blockIdx.y * 2 * kMeanBlocks;
   __shared__ uint32_t s_max[8];
   __shared__ unsigned long long s_sum[8][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -724,8 +731,9 @@ __global__ void __launch_bounds__(256) mean_partial_kernel(const double* __restr
   }
 }
 
-__global__ void __launch_bounds__(256) mean_fold_kernel(const double* __restrict__ part, int nb,
-                                                        long long S, double* mean) {
+__global__ void __launch_bounds__(256) mean_fold_kernel(const SplitArrays arr, const double* part,
+                                                        int nb, long long S) {
+  part += (size_t)blockIdx.y * 2 * kMeanBlocks;
   __shared__ double ss[256], cc[256];
   double s = 0.0, c = 0.0;
   for (int b = threadIdx.x; b < nb; b += 256) {
@@ -735,7 +743,7 @@ __global__ void __launch_bounds__(256) mean_fold_kernel(const double* __restrict
     c += part[2 * b + 1] + e;
   }
   mean_block_tree(s, c, ss, cc);
-  if (threadIdx.x == 0) *mean = (ss[0] + cc[0]) / (double)S;
+  if (threadIdx.x == 0) *arr.mean[blockIdx.y] = (ss[0] + cc[0]) / (double)S;
 }
 
 // The FP64 persistent kernel's initial state: N_f fields of S values copied into
@@ -784,39 +792,73 @@ static cudaError_t launch_copy_max(const double* src, double* dst, long long S, 
 }
 
 // out[i] = x[i] - mean as float32, or as the pair (hi, lo) with
-// hi = fl32(x - mean), lo = fl32((x - mean) - hi).
-__global__ void split_store_kernel(const double* __restrict__ x, const double* mean, void* out,
-                                   long long S, int pair) {
-  const double m = *mean;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < S;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double v = x[i] - m;
-    const float hi = narrow(v);
-    if (pair)
-      static_cast<float2*>(out)[i] = make_float2(hi, narrow(v - widen(hi)));
-    else
-      static_cast<float*>(out)[i] = hi;
+// hi = fl32(x - mean), lo = fl32((x - mean) - hi).  VEC: two values per access.
+__device__ __forceinline__ float2 split_pair(double v) {
+  const float hi = narrow(v);
+  return make_float2(hi, narrow(v - widen(hi)));
+}
+template <bool VEC>
+__global__ void __launch_bounds__(256) split_store_kernel(const SplitArrays arr, long long S,
+                                                          int pair) {
+  const double* __restrict__ x = arr.x[blockIdx.y];
+  void* out = arr.out[blockIdx.y];
+  const double m = *arr.mean[blockIdx.y];
+  const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                  step = (long long)gridDim.x * blockDim.x;
+  if constexpr (VEC) {
+#pragma unroll 4
+    for (long long i = i0; i < S / 2; i += step) {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(x) + i);
+      if (pair) {
+        const float2 p = split_pair(v.x - m), q = split_pair(v.y - m);
+        static_cast<float4*>(out)[i] = make_float4(p.x, p.y, q.x, q.y);
+      } else {
+        static_cast<float2*>(out)[i] = make_float2(narrow(v.x - m), narrow(v.y - m));
+      }
+    }
+  } else {
+    for (long long i = i0; i < S; i += step) {
+      if (pair) static_cast<float2*>(out)[i] = split_pair(x[i] - m);
+      else static_cast<float*>(out)[i] = narrow(x[i] - m);
+    }
   }
 }
 
 // The inverse for a read-out: out[i] = base + fluctuation, in float64, for
 // elements [i0, i0 + count) of one field.
-__global__ void split_load_kernel(const void* __restrict__ d, const double* base, double* out,
-                                  long long i0, long long count, int pair) {
+template <bool VEC>
+__global__ void __launch_bounds__(256) split_load_kernel(const void* __restrict__ d,
+                                                         const double* base, double* out,
+                                                         long long i0, long long count, int pair) {
   const double b = *base;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x) {
-    double v;
-    if (pair) {
-      const float2 p = static_cast<const float2*>(d)[i0 + i];
-      v = widen(p.x) + widen(p.y);
-    } else {
-      v = widen(static_cast<const float*>(d)[i0 + i]);
+  const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                  step = (long long)gridDim.x * blockDim.x;
+  if constexpr (VEC) {
+#pragma unroll 4
+    for (long long i = t0; i < count / 2; i += step) {
+      double2 v;
+      if (pair) {
+        const float4 p = __ldg(static_cast<const float4*>(d) + i0 / 2 + i);
+        v = make_double2(b + (widen(p.x) + widen(p.y)), b + (widen(p.z) + widen(p.w)));
+      } else {
+        const float2 p = __ldg(static_cast<const float2*>(d) + i0 / 2 + i);
+        v = make_double2(b + widen(p.x), b + widen(p.y));
+      }
+      reinterpret_cast<double2*>(out)[i] = v;
     }
-    out[i] = b + v;
+  } else {
+    for (long long i = t0; i < count; i += step) {
+      double v;
+      if (pair) {
+        const float2 p = static_cast<const float2*>(d)[i0 + i];
+        v = widen(p.x) + widen(p.y);
+      } else {
+        v = widen(static_cast<const float*>(d)[i0 + i]);
+      }
+      out[i] = b + v;
+    }
   }
 }
-
 
 __global__ void clear_barrier_kernel(unsigned long long* bar) { *bar = 0ull; }
 
@@ -1241,8 +1283,27 @@ static pycool_status launch_one(pycool_sim* sim) {
   return PYCOOL_OK;
 }
 
+// Means, then fluctuations, of `count` arrays (device pointers).
+static pycool_status split_arrays(pycool_sim* sim, const SplitArrays& arr, int count) {
+  const long long S = (long long)sim->hdesc.S;
+  const int pair = sim->hdesc.prec == PREC_DD ? 1 : 0;
+  double* part = (double*)(sim->ws + sim->L.off_mean);
+  const int nb = (int)std::min<long long>(kMeanBlocks, (S + 4095) / 4096);
+  bool vec = S % 2 == 0;   // and every array on the boundary of its two values
+  for (int j = 0; j < count; ++j)
+    vec = vec && ((uintptr_t)arr.x[j] & 15) == 0 && ((uintptr_t)arr.out[j] & 15) == 0;
+  const unsigned sg = (unsigned)std::min<long long>(152 * 8, (S + 511) / 512);
+  mean_partial_kernel<<<dim3(nb, count), 256, 0, sim->stream>>>(arr, S, part);
+  mean_fold_kernel<<<dim3(1, count), 256, 0, sim->stream>>>(arr, part, nb, S);
+  if (vec) split_store_kernel<true><<<dim3(sg, count), 256, 0, sim->stream>>>(arr, S, pair);
+  else split_store_kernel<false><<<dim3(sg, count), 256, 0, sim->stream>>>(arr, S, pair);
+  CK(cudaGetLastError());
+  sim->launches += 3;
+  return PYCOOL_OK;
+}
+
 // The split forms' initial state (Background already on the device, phi0 and
-// pi0 still 0): per field, the device mean goes into Background.phi0[f] /
+// pi0 still 0): the device mean of each field goes into Background.phi0[f] /
 // pi0[f], then the fluctuation into buffer 0.  Host inputs are staged, one
 // field at a time, in the simulation's own buffers that the initial state does
 // not use yet: phi buffer 1 (and, for SPLIT_FP32 with its 4-byte words, pi
@@ -1251,31 +1312,34 @@ static pycool_status launch_one(pycool_sim* sim) {
 static pycool_status split_initial(pycool_sim* sim, const double* phi, const double* pi,
                                    bool on_device) {
   const size_t S = (size_t)sim->hdesc.S;
-  const int pair = sim->hdesc.prec == PREC_DD ? 1 : 0;
-  const size_t word = pair ? 8 : 4;
+  const size_t word = sim->hdesc.prec == PREC_DD ? 8 : 4;
   char* f0 = (char*)sim->hdesc.phi[0];
   char* f1 = (char*)sim->hdesc.phi[1];
   char* p0 = (char*)sim->hdesc.pi[0];
-  double* part = (double*)(sim->ws + sim->L.off_mean);
-  const int nb = (int)std::min<size_t>(kMeanBlocks, (S + 4095) / 4096);
-  const unsigned sg = (unsigned)std::min<size_t>(152 * 8, (S + 255) / 256);
-  for (int which = 0; which < 2; ++which) {
-    const double* src_all = which == 0 ? phi : pi;
+  SplitArrays arr;
+  std::memset(&arr, 0, sizeof(arr));
+  if (on_device) {
     for (int f = 0; f < sim->nf; ++f) {
-      const double* x = src_all + (size_t)f * S;
+      arr.x[f] = phi + (size_t)f * S;
+      arr.x[sim->nf + f] = pi + (size_t)f * S;
+      arr.mean[f] = &sim->d_bg->phi0[f];
+      arr.mean[sim->nf + f] = &sim->d_bg->pi0[f];
+      arr.out[f] = f0 + (size_t)f * S * word;
+      arr.out[sim->nf + f] = p0 + (size_t)f * S * word;
+    }
+    return split_arrays(sim, arr, 2 * sim->nf);
+  }
+  for (int which = 0; which < 2; ++which) {
+    for (int f = 0; f < sim->nf; ++f) {
       // float64 staging of one field (8 S bytes), disjoint from the output
       double* stage = (double*)(which == 0 ? f1 : p0);
-      char* out = which == 0 ? f0 + (size_t)f * S * word : f1 + (size_t)f * S * word;
-      if (!on_device) {
-        CK(cudaMemcpyAsync(stage, x, S * sizeof(double), cudaMemcpyHostToDevice, sim->stream));
-        x = stage;
-      }
-      double* mean = which == 0 ? &sim->d_bg->phi0[f] : &sim->d_bg->pi0[f];
-      mean_partial_kernel<<<nb, 256, 0, sim->stream>>>(x, (long long)S, part);
-      mean_fold_kernel<<<1, 256, 0, sim->stream>>>(part, nb, (long long)S, mean);
-      split_store_kernel<<<sg, 256, 0, sim->stream>>>(x, mean, out, (long long)S, pair);
-      CK(cudaGetLastError());
-      sim->launches += 3;
+      CK(cudaMemcpyAsync(stage, (which == 0 ? phi : pi) + (size_t)f * S, S * sizeof(double),
+                         cudaMemcpyHostToDevice, sim->stream));
+      arr.x[0] = stage;
+      arr.mean[0] = which == 0 ? &sim->d_bg->phi0[f] : &sim->d_bg->pi0[f];
+      arr.out[0] = (which == 0 ? f0 : f1) + (size_t)f * S * word;
+      const pycool_status st = split_arrays(sim, arr, 1);
+      if (st != PYCOOL_OK) return st;
     }
   }
   // the momenta's fluctuations, written to phi buffer 1, into pi buffer 0
@@ -1459,9 +1523,15 @@ PYCOOL_API pycool_status pycool_get_fields(pycool_sim* sim, double* phi, double*
       for (size_t i0 = 0; i0 < S; i0 += chunk) {
         const size_t m = std::min(chunk, S - i0);
         double* out = on_device ? dst + (size_t)f * S + i0 : stage;
-        const unsigned g = (unsigned)std::min<size_t>(152 * 8, (m + 255) / 256);
-        split_load_kernel<<<g, 256, 0, sim->stream>>>(src, base, out, (long long)((size_t)f * S + i0),
-                                                     (long long)m, pair);
+        const unsigned g = (unsigned)std::min<size_t>(152 * 8, (m + 511) / 512);
+        const long long e0 = (long long)((size_t)f * S + i0);
+        const bool vec = e0 % 2 == 0 && m % 2 == 0 && ((uintptr_t)out & 15) == 0;
+        if (vec)
+          split_load_kernel<true><<<g, 256, 0, sim->stream>>>(src, base, out, e0, (long long)m,
+                                                              pair);
+        else
+          split_load_kernel<false><<<g, 256, 0, sim->stream>>>(src, base, out, e0, (long long)m,
+                                                               pair);
         CK(cudaGetLastError());
         sim->launches += 1;
         if (!on_device)

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "../../include/pycool.h"
+#include "fft.h"
 #include "models.cuh"
 #include "internal.cuh"
 #include "runtime.h"
@@ -993,6 +994,7 @@ struct pycool_sim {
   // spectrum (made at the first pycool_spectrum call): FFT plan, buffers and
   // the half-spectrum modes ordered by shell
   bool spec_ready = false;
+  bool spec_planned = false;        // a cuFFT plan (sides that fft.h does not take)
   cufftHandle spec_plan = 0;
   double* spec_tmp = nullptr;       // n^3 float64 field
   void* spec_out = nullptr;         // n n (n/2 + 1) complex coefficients
@@ -1700,7 +1702,10 @@ static pycool_status spectrum_setup(pycool_sim* sim) {
   CK(cudaMemcpy(sim->spec_cut, cut.data(), cut.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(sim->spec_first, first.data(), (nb + 1) * sizeof(int32_t),
                 cudaMemcpyHostToDevice));
-  if (cufftPlan3d(&sim->spec_plan, n, n, n, CUFFT_D2Z) != CUFFT_SUCCESS) return PYCOOL_E_CUDA;
+  if (!fft_takes(n)) {
+    if (cufftPlan3d(&sim->spec_plan, n, n, n, CUFFT_D2Z) != CUFFT_SUCCESS) return PYCOOL_E_CUDA;
+    sim->spec_planned = true;
+  }
   sim->spec_ready = true;
   return PYCOOL_OK;
 }
@@ -1718,7 +1723,6 @@ PYCOOL_API pycool_status pycool_spectrum(pycool_sim* sim, int32_t which, int32_t
     st = spectrum_setup(sim);
     if (st != PYCOOL_OK) return st;
   }
-  if (cufftSetStream(sim->spec_plan, sim->stream) != CUFFT_SUCCESS) return PYCOOL_E_CUDA;
   // an out-of-place forward transform leaves its input alone, so the FP64 form's
   // field is transformed where it lies, if it starts on a 16-byte boundary
   const double* field_values =
@@ -1730,9 +1734,13 @@ PYCOOL_API pycool_status pycool_spectrum(pycool_sim* sim, int32_t which, int32_t
     field_values = sim->spec_tmp;
     sim->launches += 1;
   }
-  if (cufftExecD2Z(sim->spec_plan, const_cast<double*>(field_values),
-                   (cufftDoubleComplex*)sim->spec_out) != CUFFT_SUCCESS)
+  if (!sim->spec_planned) {
+    CK(fft_forward(field_values, (double2*)sim->spec_out, sim->cfg.n, 1, sim->stream));
+  } else if (cufftSetStream(sim->spec_plan, sim->stream) != CUFFT_SUCCESS ||
+             cufftExecD2Z(sim->spec_plan, const_cast<double*>(field_values),
+                          (cufftDoubleComplex*)sim->spec_out) != CUFFT_SUCCESS) {
     return PYCOOL_E_CUDA;
+  }
   CK(launch_spectrum_bins(sim->spec_out, sim->cfg.n, sim->spec_order, sim->spec_cut,
                           sim->spec_chunks, sim->spec_first, nbins, sim->spec_part,
                           sim->spec_power, sim->stream));
@@ -1760,7 +1768,7 @@ PYCOOL_API pycool_status pycool_set_stream(pycool_sim* sim, void* cuda_stream) {
 PYCOOL_API void pycool_destroy(pycool_sim* sim) {
   if (!sim) return;
   cudaStreamSynchronize(sim->stream);
-  if (sim->spec_ready) cufftDestroy(sim->spec_plan);
+  if (sim->spec_planned) cufftDestroy(sim->spec_plan);
   cudaFree(sim->spec_tmp);
   cudaFree(sim->spec_out);
   cudaFree(sim->spec_order);

@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "fft.h"
 #include "models.cuh"
 #include "runtime.h"
 
@@ -562,9 +563,15 @@ extern "C" __attribute__((visibility("default"))) pycool_status pycool_linear_ev
   const long long half = (long long)n * n * (n / 2 + 1);   // coefficients of a real transform
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return PYCOOL_E_CUDA;
-  const std::shared_ptr<LinPlans> plans = linear_plans(n, nf, device);
-  if (!plans) return PYCOOL_E_CUDA;
-  std::lock_guard<std::mutex> plan_lock(plans->mu);
+  // the library's own transforms where they take the side, else cuFFT's plans
+  const bool own_fft = fft_takes(n);
+  std::shared_ptr<LinPlans> plans;
+  std::unique_lock<std::mutex> plan_lock;
+  if (!own_fft) {
+    plans = linear_plans(n, nf, device);
+    if (!plans) return PYCOOL_E_CUDA;
+    plan_lock = std::unique_lock<std::mutex>(plans->mu);
+  }
   const int hn = n / 2;
   const long long nk = linear_class(hn, hn, hn) + 1;
   const size_t N2 = (size_t)(2 * nf) * (2 * nf);
@@ -590,7 +597,6 @@ extern "C" __attribute__((visibility("default"))) pycool_status pycool_linear_ev
   cufftDoubleComplex* spec = nullptr;   // [phi, pi][N_f][half]
   double *dk = nullptr, *dT = nullptr, *dbg = nullptr, *dpart = nullptr;
   double** dptrs = nullptr;             // [2][2 N_f]: source and destination arrays
-  const cufftHandle fwd = plans->fwd, inv = plans->inv;
   pycool_status st = PYCOOL_OK;
   do {
     if (injected_alloc_failure() ||
@@ -605,7 +611,8 @@ extern "C" __attribute__((visibility("default"))) pycool_status pycool_linear_ev
       st = PYCOOL_E_NOMEM;
       break;
     }
-    if (cufftSetStream(fwd, s) != CUFFT_SUCCESS || cufftSetStream(inv, s) != CUFFT_SUCCESS) {
+    if (!own_fft && (cufftSetStream(plans->fwd, s) != CUFFT_SUCCESS ||
+                     cufftSetStream(plans->inv, s) != CUFFT_SUCCESS)) {
       st = PYCOOL_E_CUDA;
       break;
     }
@@ -641,9 +648,14 @@ extern "C" __attribute__((visibility("default"))) pycool_status pycool_linear_ev
     linear_means_fold<<<1, 32, 0, s>>>(dpart, 2 * nf, 1.0 / (double)S, dbg + 8);
     linear_subtract<<<152 * 8, 256, 0, s>>>(dptrs, dptrs + 4, S, 2 * nf, dbg + 8);
     // 2. forward transforms of the perturbations (every field), k = 0 cleared
-    if (cudaGetLastError() != cudaSuccess ||
-        cufftExecD2Z(fwd, phi_out, sphi) != CUFFT_SUCCESS ||
-        cufftExecD2Z(fwd, pi_out, spi) != CUFFT_SUCCESS) {
+    bool ok = cudaGetLastError() == cudaSuccess;
+    if (own_fft)
+      ok = ok && fft_forward(phi_out, sphi, n, nf, s) == cudaSuccess &&
+           fft_forward(pi_out, spi, n, nf, s) == cudaSuccess;
+    else
+      ok = ok && cufftExecD2Z(plans->fwd, phi_out, sphi) == CUFFT_SUCCESS &&
+           cufftExecD2Z(plans->fwd, pi_out, spi) == CUFFT_SUCCESS;
+    if (!ok) {
       st = PYCOOL_E_CUDA;
       break;
     }
@@ -656,8 +668,13 @@ extern "C" __attribute__((visibility("default"))) pycool_status pycool_linear_ev
       break;
     }
     // 5. inverse transforms into the caller's arrays
-    if (cufftExecZ2D(inv, sphi, phi_out) != CUFFT_SUCCESS ||
-        cufftExecZ2D(inv, spi, pi_out) != CUFFT_SUCCESS) {
+    if (own_fft)
+      ok = fft_inverse(sphi, phi_out, n, nf, s) == cudaSuccess &&
+           fft_inverse(spi, pi_out, n, nf, s) == cudaSuccess;
+    else
+      ok = cufftExecZ2D(plans->inv, sphi, phi_out) == CUFFT_SUCCESS &&
+           cufftExecZ2D(plans->inv, spi, pi_out) == CUFFT_SUCCESS;
+    if (!ok) {
       st = PYCOOL_E_CUDA;
       break;
     }

@@ -94,15 +94,18 @@ Layout layout_for(const pycool_config& c) {
   L.off_desc = align256(sizeof(Background));
   L.off_fields = L.off_desc + align256(sizeof(SimDesc));
   L.state_bytes = L.off_fields + 4 * L.field_bytes;
+  if (runtime) L.geo.ncta = kMaxPBlocks;   // rt_kick: at most; its plan's blocks at creation
   workspace_layout(L.geo.ncta, L);
   L.off_prows = 0;
   L.off_punits = 0;
   L.off_rt = 0;
   L.off_mean = 0;
   L.plain = false;
-  if (runtime) {   // drifted fields, V' (N_f n^3 each) and V (n^3)
+  if (runtime) {   // drifted fields, V' (N_f n^3 each) and V (n^3); rt_kick's plan
     L.off_rt = align256(L.ws_bytes);
-    L.ws_bytes = L.off_rt + 2 * align256((size_t)nf * S * 8) + align256(S * 8);
+    L.off_punits = L.off_rt + 2 * align256((size_t)nf * S * 8) + align256(S * 8);
+    L.ws_bytes = L.off_punits + align256((size_t)kMaxPBlocks * kMaxPUnits * sizeof(int4)) +
+                 align256((size_t)(kMaxPBlocks + 1) * sizeof(int));
   }
   return L;
 }
@@ -512,6 +515,9 @@ void fill_desc(SimDesc& d, const pycool_config& c, const Layout& L, char* state,
     d.rt_phis = (double*)(ws + L.off_rt);
     d.rt_dV = (double*)(ws + L.off_rt + fb);
     d.rt_V = (double*)(ws + L.off_rt + 2 * fb);
+    d.rt_units = (const int4*)(ws + L.off_punits);
+    d.rt_uoff = (const int*)(ws + L.off_punits +
+                             align256((size_t)kMaxPBlocks * kMaxPUnits * sizeof(int4)));
   }
 }
 
@@ -1209,6 +1215,22 @@ PYCOOL_API pycool_status pycool_create(const pycool_config* cfg, void* dev_state
     }
     sim->own_ws = true;
   }
+  std::vector<int4> rt_units;   // run-time potentials: rt_kick's plan for this device
+  std::vector<int> rt_uoff;
+  if (cfg->model >= kRuntimeModelBase) {
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, sim->device);
+    const PGeo g = plan_units(cfg->n, 8, sim->nf, PREC_FP64, std::max(sms, 1), 0, &rt_units,
+                              &rt_uoff, cfg->stencil == PYCOOL_STENCIL_4TH ? 2 : 1, true);
+    if (e != cudaSuccess || rt_units.size() > (size_t)kMaxPBlocks * kMaxPUnits ||
+        !check_plan(g, rt_units, rt_uoff, true)) {
+      if (sim->own_state) cudaFree(sim->state);
+      if (sim->own_ws) cudaFree(sim->ws);
+      delete sim;
+      return e != cudaSuccess ? PYCOOL_E_CUDA : PYCOOL_E_INVALID;
+    }
+    sim->L.geo.ncta = g.G;
+  }
   fill_desc(sim->hdesc, *cfg, sim->L, sim->state, sim->ws);
   e = encode_tensor_maps(sim->hdesc);
   if (e != cudaSuccess) {
@@ -1232,6 +1254,14 @@ PYCOOL_API pycool_status pycool_create(const pycool_config* cfg, void* dev_state
     if ((e = cudaMemcpyAsync(sim->d_bg, &b, sizeof(b), cudaMemcpyHostToDevice, sim->stream)) !=
         cudaSuccess) break;
     if ((e = cudaMemsetAsync(sim->ws, 0, sim->L.ws_bytes, sim->stream)) != cudaSuccess) break;
+    if (!rt_units.empty()) {
+      if ((e = cudaMemcpyAsync((void*)sim->hdesc.rt_units, rt_units.data(),
+                               rt_units.size() * sizeof(int4), cudaMemcpyHostToDevice,
+                               sim->stream)) != cudaSuccess) break;
+      if ((e = cudaMemcpyAsync((void*)sim->hdesc.rt_uoff, rt_uoff.data(),
+                               rt_uoff.size() * sizeof(int), cudaMemcpyHostToDevice,
+                               sim->stream)) != cudaSuccess) break;
+    }
     if ((e = cudaStreamSynchronize(sim->stream)) != cudaSuccess) break;
     if ((e = cudaStreamCreateWithFlags(&sim->cap_stream, cudaStreamNonBlocking)) != cudaSuccess)
       break;

@@ -124,6 +124,8 @@ struct alignas(64) SimDesc {
   double* rt_phis;            // N_f n^3
   double* rt_dV;              // N_f n^3
   double* rt_V;               // n^3
+  const int4* rt_units;       // rt_kick's plan (as PParams::units of the plain staging) ...
+  const int* rt_uoff;         // ... for ncta blocks
   int32_t rt_index;           // the registry entry of the potential (-1: none)
 };
 

@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
   // scalar coefficients (the FP64 chain of the merged half-stages)
   {
     if constexpr (PLAIN) {
-      plain_prefetch<MODEL, PREC, NQ, H>(p, sm, ib, gq);
+      plain_prefetch<MODEL, PREC, NQ, H>(p.g.n, sm, ib, gq);
     } else {
       for (int l = kPWarps - 1 - warp; l < LEAD; l += kPWarps)   // warp 15 - l issues plane l
         prefetch_plane<PREC, NF, VX, CORNERS, NSLOT, H>(p, sm, ib, gq, l);
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         constexpr int MD = decltype(mode_c)::value;
         constexpr bool FX = decltype(fix_c)::value;
         if constexpr (PLAIN)
-          return stage_plain<MODEL, STENCIL, PREC, MD, FX>(p, cx, sm, gq, ib, accd, hm);
+          return stage_plain<MODEL, STENCIL, PREC, MD, FX>(p.g.n, cx, sm, gq, ib, accd, hm);
         else if constexpr (STENCIL == 13)
           return stage_fp64_wide<MODEL, VX, MD, FX>(p, cx, sm, gq, ib, accd, hm);
         else
@@ -166,8 +166,8 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         ok = fix ? stage(MF{}, std::true_type{}) : stage(MF{}, std::false_type{});
     } else if constexpr (PLAIN) {
       ok = (mode == MODE_SWEEP)
-               ? stage_plain<MODEL, STENCIL, PREC, MODE_SWEEP, false>(p, cx, sm, gq, ib, accd, hm)
-               : stage_plain<MODEL, STENCIL, PREC, MODE_FLUSH, false>(p, cx, sm, gq, ib, accd, hm);
+               ? stage_plain<MODEL, STENCIL, PREC, MODE_SWEEP, false>(p.g.n, cx, sm, gq, ib, accd, hm)
+               : stage_plain<MODEL, STENCIL, PREC, MODE_FLUSH, false>(p.g.n, cx, sm, gq, ib, accd, hm);
     } else if constexpr (STENCIL == 13) {
       ok = (mode == MODE_SWEEP) ? stage_wide_dd<MODEL, VX, MODE_SWEEP>(p, cx, sm, gq, ib)
                                 : stage_wide_dd<MODEL, VX, MODE_FLUSH>(p, cx, sm, gq, ib);
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
       if (pre && !PLAIN) named_arrive(1, kPreThreads);   // the next stage's copies queue behind it
     }
     if constexpr (PLAIN) {   // every thread's own copies; the folding warps' after their fold
-      if (pre && warp > nl) plain_prefetch<MODEL, PREC, NQ, H>(p, sm, ib_next, gq);
+      if (pre && warp > nl) plain_prefetch<MODEL, PREC, NQ, H>(p.g.n, sm, ib_next, gq);
     }
     if (warp < nl) {
       if (!mbar_wait(&foldbar, (uint32_t)(k & 1), p.wait_limit)) atomicOr(&s_bad, 1);
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
     // @folded
     if (tid == 0 && !s_bad) s_fold = -1;   // every folding warp saw the copy land
     if constexpr (PLAIN) {
-      if (pre && warp <= nl) plain_prefetch<MODEL, PREC, NQ, H>(p, sm, ib_next, gq);
+      if (pre && warp <= nl) plain_prefetch<MODEL, PREC, NQ, H>(p.g.n, sm, ib_next, gq);
     }
     // ---- in parallel, on warps of different schedulers, identically in
     //      every block: the next stage's coefficients (warp 14: sums -> p_a

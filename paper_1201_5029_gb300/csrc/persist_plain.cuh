@@ -132,20 +132,26 @@ struct PlainPos {
   }
 };
 
+// A potential given at run time: its stage (rt_kick) finds the field drifted
+// (SimDesc::rt_phis) and V' and V at every site in arrays.
+template <int MODEL> constexpr bool runtime_pot() {
+  return MODEL == M_RUNTIME1 || MODEL == M_RUNTIME2;
+}
+
 // Copies of the plane at `pos` (ring plane gp) and one commit, always: the
 // groups a thread has committed count the planes.
 template <int MODEL, int PREC, int NQ, int H>
-__device__ __forceinline__ void plain_issue(const PParams& p, const PShared& sm, PlainPos<H>& pos,
-                                            int ib, uint32_t gp) {
+__device__ __forceinline__ void plain_issue(int n, const PShared& sm, PlainPos<H>& pos, int ib,
+                                            uint32_t gp) {
+  constexpr bool RT = runtime_pot<MODEL>();
   constexpr int NF = Pot<MODEL>::NF;
   using T = typename WorkT<PREC>::type;
   using RG = PlainRing<PREC, NF, NQ, H>;
   if (pos.in(sm)) {
     const SimDesc& d = *sm.d;
-    const int n = p.g.n;
     const size_t S = (size_t)d.S;
     const int z = wrapi(sm.units[pos.ui].z - H + pos.uq, n);
-    const T* src[2] = {(const T*)d.phi[ib & 1] + (size_t)z * n * n,
+    const T* src[2] = {(RT ? (const T*)d.rt_phis : (const T*)d.phi[ib & 1]) + (size_t)z * n * n,
                        (const T*)d.pi[(ib >> 1) & 1] + (size_t)z * n * n};
     T* own = (T*)sm.ring + (gp % RG::OSLOT) * RG::OWN + threadIdx.x;
     T* hal = (T*)sm.ring + RG::HALO_OFF + (gp % RG::HSLOT) * RG::HALO + threadIdx.x;
@@ -155,7 +161,7 @@ __device__ __forceinline__ void plain_issue(const PParams& p, const PShared& sm,
       for (int arr = 0; arr < 2; ++arr) {
         if (pos.c.own >= 0)
           cp_async_word(own + (f * 2 + arr) * kPThreads, src[arr] + f * S + pos.c.own);
-        if (pos.c.halo >= 0)
+        if (pos.c.halo >= 0 && (!RT || arr == 0))
           cp_async_word(hal + (f * 2 + arr) * kPlainHalo, src[arr] + f * S + pos.c.halo);
       }
     pos.next(sm, n);
@@ -165,12 +171,11 @@ __device__ __forceinline__ void plain_issue(const PParams& p, const PShared& sm,
 
 // The first LEAD planes of a stage (every thread of the block).
 template <int MODEL, int PREC, int NQ, int H>
-__device__ __forceinline__ void plain_prefetch(const PParams& p, const PShared& sm, int ib,
-                                               uint32_t gq) {
+__device__ __forceinline__ void plain_prefetch(int n, const PShared& sm, int ib, uint32_t gq) {
   using RG = PlainRing<PREC, Pot<MODEL>::NF, NQ, H>;
   PlainPos<H> pos;
-  pos.start(sm, p.g.n);
-  for (int l = 0; l < RG::LEAD; ++l) plain_issue<MODEL, PREC, NQ, H>(p, sm, pos, ib, gq + l);
+  pos.start(sm, n);
+  for (int l = 0; l < RG::LEAD; ++l) plain_issue<MODEL, PREC, NQ, H>(n, sm, pos, ib, gq + l);
 }
 
 __device__ __forceinline__ float fix_in(float v, int, float*) { return v; }
@@ -188,9 +193,10 @@ __device__ __forceinline__ void fix_parts27(float c, float faces, float corners,
 // One stage over this block's units (see the head of this file); the sums go to
 // accd (FP64) or the block's compensated sums (split-FP32, as stage_split).
 template <int MODEL, int STENCIL, int PREC, int MODE, bool FIX>
-__device__ __forceinline__ bool stage_plain(const PParams& p, const Ctx<MODEL, PREC>& cx0,
-                                            const PShared& sm, uint32_t gq, int ib, double* accd,
+__device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, const PShared& sm,
+                                            uint32_t gq, int ib, double* accd,
                                             HiMax<Pot<MODEL>::NF>& hm) {
+  constexpr bool RT = runtime_pot<MODEL>();
   using C = Ctx<MODEL, PREC>;
   using T = typename C::T;
   constexpr bool F64 = PREC == PREC_FP64;
@@ -204,7 +210,6 @@ __device__ __forceinline__ bool stage_plain(const PParams& p, const Ctx<MODEL, P
   constexpr int KGROUP = 8;   // split: output planes per float partial before a compensated add
   const SimDesc& d = *sm.d;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int n = p.g.n;
   const size_t S = (size_t)d.S, nn = (size_t)n * n;
   T* __restrict__ phi_out = (T*)d.phi[(ib & 1) ^ 1];
   T* __restrict__ pi_out = (T*)d.pi[((ib >> 1) & 1) ^ 1];
@@ -248,12 +253,16 @@ __device__ __forceinline__ bool stage_plain(const PParams& p, const Ctx<MODEL, P
     for (int f = 0; f < NF; ++f) {
       const int ex = F64 ? cx.fx[f] : 0;
       if (dp.c.own >= 0) {
-        const T a = madd(cx.cdrift, o[(f * 2 + 1) * kPThreads], o[f * 2 * kPThreads]);
-        o[f * 2 * kPThreads] = a;
+        T a = o[f * 2 * kPThreads];
+        if constexpr (!RT) {
+          a = madd(cx.cdrift, o[(f * 2 + 1) * kPThreads], a);
+          o[f * 2 * kPThreads] = a;
+        }
         fx[f * kPlainCells + dp.c.ownc] = fix_in(a, ex, (E*)nullptr);
       }
       if (dp.c.halo >= 0) {
-        const T a = madd(cx.cdrift, h[(f * 2 + 1) * kPlainHalo], h[f * 2 * kPlainHalo]);
+        T a = h[f * 2 * kPlainHalo];
+        if constexpr (!RT) a = madd(cx.cdrift, h[(f * 2 + 1) * kPlainHalo], a);
         fx[f * kPlainCells + dp.c.haloc] = fix_in(a, ex, (E*)nullptr);
       }
     }
@@ -264,7 +273,7 @@ __device__ __forceinline__ bool stage_plain(const PParams& p, const Ctx<MODEL, P
 
   uint32_t g = gq;
   if (sm.nunits > 0) {
-    plain_issue<MODEL, PREC, NQ, H>(p, sm, ip, ib, g + LEAD);
+    plain_issue<MODEL, PREC, NQ, H>(n, sm, ip, ib, g + LEAD);
     cp_async_wait<LEAD>();
     drift(g);
   }
@@ -278,10 +287,19 @@ __device__ __forceinline__ bool stage_plain(const PParams& p, const Ctx<MODEL, P
 #pragma unroll
     for (int f = 0; f < NF; ++f) qa[f] = qb[f] = qc[f] = qd[f] = (E)0;
     for (int q = 0; q < Q; ++q, ++g) {
-      plain_issue<MODEL, PREC, NQ, H>(p, sm, ip, ib, g + 1 + LEAD);
+      plain_issue<MODEL, PREC, NQ, H>(n, sm, ip, ib, g + 1 + LEAD);
       if (dp.in(sm)) {
         cp_async_wait<LEAD>();
         drift(g + 1);
+      }
+      double rv[RT ? NF + 1 : 1];   // run-time potential: V' and V of the plane put out
+      if constexpr (RT) {
+        const bool put = valid && q >= 2 * H;
+        const size_t o = (size_t)(u.z + q - 2 * H) * nn + c.own;
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+          rv[f] = put && MODE == MODE_SWEEP ? __ldcg(d.rt_dV + f * S + o) : 0.0;
+        rv[NF] = put ? __ldcg(d.rt_V + o) : 0.0;
       }
       // every warp has drifted plane g
       ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit);
@@ -336,8 +354,27 @@ __device__ __forceinline__ bool stage_plain(const PParams& p, const Ctx<MODEL, P
               pmj[f] -= cx.mu_pi[f];
             }
           }
-          if constexpr (F64) {
+          if constexpr (RT) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+              if (MODE == MODE_SWEEP) {
+                pnj[f] = madd(cx.kD, Dj[f], madd(-cx.kV, rv[f], pmj[f]));
+                accd[SL::PI2] = madd(pnj[f], pnj[f], accd[SL::PI2]);
+                accd[SL::PHID] = madd(phj[f], Dj[f], accd[SL::PHID]);
+              } else {
+                pnj[f] = pmj[f];
+                accd[SL::PI2 + f] = madd(pmj[f], pmj[f], accd[SL::PI2 + f]);
+                accd[SL::PHID + f] = madd(phj[f], Dj[f], accd[SL::PHID + f]);
+                const T dd = phj[f] - cx.shiftK[f];
+                accd[SL::DPHI + f] += dd;
+                accd[SL::DPHI2 + f] = madd(dd, dd, accd[SL::DPHI2 + f]);
+              }
+            }
+            accd[SL::V] += rv[NF];
+          } else if constexpr (F64) {
             cx.site(MODE, phj, Dj, pmj, pnj, accd);
+          }
+          if constexpr (F64) {
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
               hm.add(2 * f, phj[f]);

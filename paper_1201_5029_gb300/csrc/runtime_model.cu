@@ -17,8 +17,8 @@
 #include <vector>
 
 #include "../../include/pycool.h"
+#include "persist_plain.cuh"
 #include "runtime.h"
-#include "sweep.cuh"
 
 #define PYCOOL_API extern "C" __attribute__((visibility("default")))
 
@@ -58,6 +58,107 @@ std::string make_source(int nf, const char* V, const char* const* dV) {
   return s;
 }
 
+// The kick of a stage: one stage of the plain staging over each block's units
+// (one block per SM), with V' and V read from the compiled kernel's arrays, then
+// the per-stage kernels' block finish.  Bound by the float64 pipe: ten
+// instructions per two-field site (128^3: 51 % of it; 16 warps and a barrier of
+// all of them per plane do not cover the rest).
+template <int MODEL, int STENCIL>
+__global__ void __launch_bounds__(kPThreads, 1) rt_kick(const LaunchTable tab) {
+  using C = Ctx<MODEL, PREC_FP64>;
+  using SL = typename C::SL;
+  constexpr int NF = C::NF, NQ = SL::NQ, H = halo_of<STENCIL>();
+  using RG = PlainRing<PREC_FP64, NF, NQ, H>;
+  extern __shared__ __align__(128) unsigned char dsm[];
+  __shared__ __align__(8) uint64_t dbar[RG::NDRIFT];
+  __shared__ __align__(64) SimDesc s_desc;
+  __shared__ int4 s_units[kMaxPUnits];
+  __shared__ double sout[NQ];
+  __shared__ uint32_t s_wmax[kPWarps][2 * NF], s_bmax[2 * NF];
+  __shared__ C s_ctx;
+  __shared__ int s_last, s_bad;
+  const SimDesc* dg = tab.desc[0];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int mode = dg->bg->mode;
+  if (mode == MODE_IDLE) return;
+  const int ubeg = dg->rt_uoff[blockIdx.x];
+  PShared sm;
+  sm.d = &s_desc;
+  sm.ring = dsm;
+  sm.kahan = nullptr;
+  sm.drift = nullptr;
+  sm.red = reinterpret_cast<double*>(dsm + RG::RING_BYTES);
+  sm.full = sm.empty = nullptr;
+  sm.dbar = dbar;
+  sm.units = s_units;
+  sm.nunits = min(dg->rt_uoff[blockIdx.x + 1] - ubeg, kMaxPUnits);   // host: <= kMaxPUnits
+  sm.issued = nullptr;
+  sm.limit = kWaitLimit;
+  for (int i = tid; i < (int)(sizeof(SimDesc) / 8); i += kPThreads)
+    reinterpret_cast<unsigned long long*>(&s_desc)[i] =
+        reinterpret_cast<const unsigned long long*>(dg)[i];
+  if (tid < sm.nunits) s_units[tid] = dg->rt_units[ubeg + tid];
+  if (tid == 0) {
+    for (int b = 0; b < RG::NDRIFT; ++b) mbar_init(&dbar[b], kPWarps);
+    fence_mbar_init();
+    s_bad = 0;
+  }
+  __syncthreads();
+  const SimDesc& d = s_desc;
+  const Background& bgr = *d.bg;
+  const int n = d.n, ib = bgr.cur;
+  plain_prefetch<MODEL, PREC_FP64, NQ, H>(n, sm, ib, 0u);   // while one thread ...
+  if (tid == 0) {
+    s_ctx.init(bgr, d, mode);
+    s_ctx.set_fix(bgr.amax, fix_headroom<STENCIL>());
+  }
+  __syncthreads();
+  double ps[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) ps[q] = 0.0;
+  HiMax<NF> hm;
+  hm.zero();
+  bool ok = true;
+  by_mode(mode, s_ctx.fx[0] != 0, [&](auto fix_c, auto mode_c) {
+    ok = stage_plain<MODEL, STENCIL, PREC_FP64, decltype(mode_c)::value, decltype(fix_c)::value>(
+        n, s_ctx, sm, 0u, ib, ps, hm);
+  });
+  cp_async_wait<0>();
+  if (!ok) s_bad = 1;
+#pragma unroll
+  for (int i = 0; i < 2 * NF; ++i) {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, hm.v[i]);
+    if (lane == 0) s_wmax[warp][i] = m;
+  }
+  __syncthreads();
+  if (s_bad) {   // a wait gave up: recorded, and the stage is not finished
+    if (tid == 0) atomicOr(d.fault, 1);
+    return;
+  }
+  constexpr uint32_t kSweepLive = (1u << SL::PI2) | (1u << SL::PHID) | (1u << SL::V);
+  block_sum<NQ, kPWarps>(ps, sm.red, sout, mode == MODE_SWEEP ? kSweepLive : 0xffffffffu);
+  if (tid < 2 * NF) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int w = 0; w < kPWarps; ++w) m = max(m, s_wmax[w][tid]);
+    s_bmax[tid] = m;
+  }
+  __syncthreads();
+  finish_block<MODEL, PREC_FP64>(s_ctx, d, mode, blockIdx.x, sout, &s_last, s_bmax);
+}
+
+template <int MODEL, int STENCIL>
+cudaError_t launch_rt_kick(const LaunchTable& t, int grid, cudaStream_t s) {
+  constexpr int NF = Pot<MODEL>::NF;
+  constexpr int smem =
+      PlainRing<PREC_FP64, NF, Slots<NF, PREC_FP64>::NQ, halo_of<STENCIL>()>::SMEM_BYTES;
+  if (grid == 0)   // ahead of any stream capture
+    return cudaFuncSetAttribute(rt_kick<MODEL, STENCIL>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  rt_kick<MODEL, STENCIL><<<grid, kPThreads, smem, s>>>(t);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 int runtime_model_nfields(int id) {
@@ -91,18 +192,18 @@ cudaError_t launch_runtime_stage(const SimDesc& d, const LaunchTable& t, int gri
     std::lock_guard<std::mutex> lk(g_rt_mu);
     if (d.rt_index < 0 || d.rt_index >= (int)g_rt.size()) return cudaErrorInvalidValue;
   }
-  if (grid == 0) return cudaSuccess;
-  const unsigned eg = 152;
-  if (d.model == M_RUNTIME1) rt_drift<M_RUNTIME1><<<eg, kRtDriftThreads, 0, s>>>(t);
-  else rt_drift<M_RUNTIME2><<<eg, kRtDriftThreads, 0, s>>>(t);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  e = launch_runtime_potential(d, d.rt_phis, s);
-  if (e != cudaSuccess) return e;
+  if (grid != 0) {   // 0: set the kernel's attributes only
+    const unsigned eg = 152;
+    if (d.model == M_RUNTIME1) rt_drift<M_RUNTIME1><<<eg, kRtDriftThreads, 0, s>>>(t);
+    else rt_drift<M_RUNTIME2><<<eg, kRtDriftThreads, 0, s>>>(t);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = launch_runtime_potential(d, d.rt_phis, s);
+    if (e != cudaSuccess) return e;
+  }
 #define PYCOOL_RT(M, ST)                                              \
   if (d.model == M && d.stencil == ST) {                              \
-    rt_kick<M, ST><<<grid, kThreads, 0, s>>>(t);                      \
-    return cudaGetLastError();                                        \
+    return launch_rt_kick<M, ST>(t, grid, s);                         \
   }
   PYCOOL_RT(M_RUNTIME1, 7) PYCOOL_RT(M_RUNTIME1, 27) PYCOOL_RT(M_RUNTIME1, 13)
   PYCOOL_RT(M_RUNTIME2, 7) PYCOOL_RT(M_RUNTIME2, 27) PYCOOL_RT(M_RUNTIME2, 13)

@@ -194,7 +194,7 @@ __device__ __forceinline__ bool is_fin(double x) { return isfinite(x); }
 // ---------------------------------------------------------------------------
 // live: bit q set if quantity q is summed; the others are 0 in out (a float64
 // instruction of a warp takes 64 cycles: a sweep sums only what it needs).
-template <int NQ>
+template <int NQ, int NWARP = kThreads / 32>
 __device__ __forceinline__ void block_sum(double (&v)[NQ], double* sred, double* out,
                                           uint32_t live = 0xffffffffu) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -211,7 +211,7 @@ __device__ __forceinline__ void block_sum(double (&v)[NQ], double* sred, double*
     double s = 0.0;
     if ((live >> threadIdx.x) & 1u) {
 #pragma unroll
-      for (int w = 0; w < kThreads / 32; ++w) s += sred[w * NQ + threadIdx.x];
+      for (int w = 0; w < NWARP; ++w) s += sred[w * NQ + threadIdx.x];
     }
     out[threadIdx.x] = s;
   }
@@ -2029,9 +2029,10 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_wide(const LaunchTable tab)
 // advances the Background).  Both library kernels derive the stage's
 // coefficients from the same Background record, which only the last block of
 // rt_kick changes.
+// rt_kick runs the plain staging's stage (persist_plain.cuh, runtime_model.cu).
 // Measured on GB300, 128^3, two-field chaotic potential, per stage: rt_drift 25
 // -> 18 us, the compiled kernel 51 (its own float64 instructions), rt_kick 148 ->
-// 83.
+// 83 as 32 x 8 tiles of 256 threads, 78 on the plan's units.
 // ---------------------------------------------------------------------------
 // One block per SM: the scalar step that every block repeats takes thousands of
 // cycles of the SM's float64 pipe.
@@ -2064,193 +2065,6 @@ __global__ void __launch_bounds__(kRtDriftThreads) rt_drift(const LaunchTable ta
   if (i0 == 0 && (total & 1))
     d.rt_phis[total - 1] = fma(c, reinterpret_cast<const double*>(pi)[total - 1],
                                reinterpret_cast<const double*>(phi)[total - 1]);
-}
-
-// Tiles of txt x ty sites marching z: a plane's cells (with the halo ring, two
-// per thread) are loaded one plane ahead, put on the fixed-point scale (or kept
-// in float64 without one) in one of two shared-memory planes, and summed as in
-// stage_plain.  Bound by the float64 pipe (9 instructions per two-field site; 21
-// with the stencil in float64, and its neighbours by 64-bit wrapped indices).
-template <int MODEL, int STENCIL>
-__global__ void __launch_bounds__(kThreads, 2) rt_kick(const LaunchTable tab) {
-  using C = Ctx<MODEL, PREC_FP64>;
-  using SL = typename C::SL;
-  constexpr int NF = C::NF;
-  constexpr int NQ = SL::NQ;
-  constexpr bool CORNERS = StencilW<STENCIL>::kCorners, WIDE = STENCIL == 13;
-  constexpr int H = WIDE ? 2 : 1;
-  constexpr int kCells = (kMaxTXT + 2 * H) * (kMaxTY + 2 * H);
-  static_assert(kCells <= 2 * kThreads, "two cells per thread");
-  __shared__ double sm[2][NF][kCells];
-  __shared__ double sred[(kThreads / 32) * NQ];
-  __shared__ double sout[NQ];
-  __shared__ uint32_t s_wmax[kThreads / 32][2 * NF], s_bmax[2 * NF];
-  __shared__ int s_last;
-  __shared__ C s_ctx;
-  const SimDesc& d = *tab.desc[0];
-  const int cta = blockIdx.x;
-  const Background& bgr = *d.bg;
-  const int mode = bgr.mode;
-  if (mode == MODE_IDLE) return;
-  const int n = d.n;
-  const int TX = d.txt, TY = d.ty;
-  const int tile = cta % (d.tiles_x * d.tiles_y);
-  const int zch = cta / (d.tiles_x * d.tiles_y);
-  const int x0 = (tile % d.tiles_x) * TX, y0 = (tile / d.tiles_x) * TY;
-  const int z0 = zch * d.zc, zend = min(n, z0 + d.zc);
-  const int tid = threadIdx.x;
-  const bool active = tid < TX * TY;
-  const int lx = active ? tid % TX : 0, ly = active ? tid / TX : 0;
-  const int gx = x0 + lx, gy = y0 + ly;
-  const bool valid = active && gx < n && gy < n;
-  const size_t S = (size_t)d.S, nn = (size_t)n * n;
-  const int rs = TX + 2 * H, cells = rs * (TY + 2 * H), own = (ly + H) * rs + lx + H;
-  // this thread's cells of a plane: in-plane offsets (a ragged tile's cells past
-  // the lattice wrap like the halo and are not used)
-  int off[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int c = tid + k * kThreads;
-    const int row = c / rs, col = c - row * rs;
-    off[k] = c < cells ? ((y0 - H + row + n) % n) * n + (x0 - H + col + n) % n : -1;
-  }
-  if (tid == 0) {
-    s_ctx.init(bgr, d, mode);
-    s_ctx.set_fix(bgr.amax, fix_headroom<STENCIL>());
-  }
-  __syncthreads();
-  const int ib = bgr.cur;
-  double* __restrict__ phi_out = (double*)d.phi[(ib & 1) ^ 1];
-  const double* __restrict__ pi_in = (const double*)d.pi[(ib >> 1) & 1];
-  double* __restrict__ pi_out = (double*)d.pi[((ib >> 1) & 1) ^ 1];
-  double ps[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) ps[q] = 0.0;
-  HiMax<NF> hm;
-  hm.zero();
-  auto body = [&](auto fix_c, auto mode_c) {
-    constexpr bool FIX = decltype(fix_c)::value;
-    constexpr int MODE = decltype(mode_c)::value;
-    constexpr bool TIMES = WIDE || (FIX && STENCIL == 27);   // as in stage_plain
-    using E = typename FixElem<FIX>::type;
-    C cx = s_ctx;
-    if constexpr (TIMES) cx.kD *= 1.0 / fix_weight<STENCIL>();
-    const E w1 = (E)16, w2 = (E)0 - (E)1, w0 = (E)0 - (E)90;   // 13-point, times 12
-    double raw[2][NF];
-    auto load = [&](int p) {
-      const size_t zo = (size_t)((p + n) % n) * nn;
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-          raw[k][f] = off[k] >= 0 ? d.rt_phis[f * S + zo + off[k]] : 0.0;
-    };
-    E qa[NF], qb[NF], qc[NF], qd[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) qa[f] = qb[f] = qc[f] = qd[f] = (E)0;
-    load(z0 - H);
-    const int Q = zend - z0 + 2 * H;
-    for (int q = 0; q < Q; ++q) {
-      E* buf = reinterpret_cast<E*>(&sm[q & 1][0][0]);
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-          if (off[k] >= 0)
-            buf[f * kCells + tid + k * kThreads] = fix_in(raw[k][f], cx.fx[f], (E*)nullptr);
-      if (q + 1 < Q) load(z0 - H + q + 1);
-      // the output plane's own values
-      const bool put = valid && q >= 2 * H;
-      const size_t o = (size_t)(z0 + q - 2 * H) * nn + (size_t)gy * n + gx;
-      double ph[NF], pm[NF], dv[NF], V = 0.0;
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        ph[f] = put ? d.rt_phis[f * S + o] : 0.0;
-        pm[f] = put ? pi_in[f * S + o] : 0.0;
-        dv[f] = put && MODE == MODE_SWEEP ? d.rt_dV[f * S + o] : 0.0;
-      }
-      if (put) V = d.rt_V[o];
-      __syncthreads();
-      const bool mid = q >= H && q < Q - H;
-      E D[NF];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        const E* fx = buf + f * kCells + own;
-        const E ctr = fx[0];
-        if constexpr (WIDE) {
-          E m = (E)0;
-          if (mid) {
-            const E nr = (fx[-rs] + fx[rs]) + (fx[-1] + fx[1]);
-            const E fr = (fx[-2 * rs] + fx[2 * rs]) + (fx[-2] + fx[2]);
-            m = fix_mad(w0, ctr, fix_mad(w2, fr, w1 * nr));
-          }
-          D[f] = fix_mad(w2, ctr, qb[f]);
-          const E np1 = fix_mad(w1, ctr, qa[f]);
-          qa[f] = fix_mad(w2, qd[f], fix_mad(w1, qc[f], m));
-          qb[f] = np1;
-          qd[f] = qc[f];
-          qc[f] = ctr;
-        } else {
-          E smid = ctr, so = ctr;
-          if (CORNERS || mid) {
-            const E faces = (fx[-rs] + fx[rs]) + (fx[-1] + fx[1]);
-            if constexpr (CORNERS)
-              fix_parts27(ctr, faces, (fx[-rs - 1] + fx[-rs + 1]) + (fx[rs - 1] + fx[rs + 1]),
-                          smid, so);
-            else
-              smid = fix_mid7(ctr, faces);
-          }
-          D[f] = qa[f] + so;
-          if (mid) qa[f] = qb[f] + smid;
-          qb[f] = so;
-        }
-      }
-      if (put) {
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          const double Df = fix_out(D[f], cx.fx[f]);
-          phi_out[f * S + o] = ph[f];
-          hm.add(2 * f, ph[f]);
-          if (MODE == MODE_SWEEP) {
-            const double pin = fma(cx.kD, Df, fma(-cx.kV, dv[f], pm[f]));
-            pi_out[f * S + o] = pin;
-            hm.add(2 * f + 1, pin);
-            ps[SL::PI2] = fma(pin, pin, ps[SL::PI2]);
-            ps[SL::PHID] = fma(ph[f], Df, ps[SL::PHID]);
-          } else {
-            hm.add(2 * f + 1, pm[f]);
-            ps[SL::PI2 + f] = fma(pm[f], pm[f], ps[SL::PI2 + f]);
-            ps[SL::PHID + f] = fma(ph[f], Df, ps[SL::PHID + f]);
-            const double dd = ph[f] - cx.shiftK[f];
-            ps[SL::DPHI + f] += dd;
-            ps[SL::DPHI2 + f] = fma(dd, dd, ps[SL::DPHI2 + f]);
-          }
-        }
-        ps[SL::V] += V;
-      }
-    }
-    if constexpr (TIMES) {
-#pragma unroll
-      for (int f = 0; f < NF; ++f) ps[SL::PHID + f] *= 1.0 / fix_weight<STENCIL>();
-    }
-  };
-  by_mode(mode, s_ctx.fx[0] != 0, body);
-#pragma unroll
-  for (int i = 0; i < 2 * NF; ++i) {
-    const uint32_t m = __reduce_max_sync(0xffffffffu, hm.v[i]);
-    if ((tid & 31) == 0) s_wmax[tid >> 5][i] = m;
-  }
-  constexpr uint32_t kSweepLive = (1u << SL::PI2) | (1u << SL::PHID) | (1u << SL::V);
-  block_partials<PREC_FP64, NQ, double>(nullptr, ps, sred, sout,
-                                        mode == MODE_SWEEP ? kSweepLive : 0xffffffffu);
-  if (tid < 2 * NF) {
-    uint32_t m = 0u;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) m = max(m, s_wmax[w][tid]);
-    s_bmax[tid] = m;
-  }
-  __syncthreads();
-  finish_block<MODEL, PREC_FP64>(s_ctx, d, mode, cta, sout, &s_last, s_bmax);
 }
 
 // Launch helper: dispatch (model, stencil, path/vx) at runtime to an instance.

@@ -21,10 +21,12 @@
 // copies' latency (one site per thread).  Measured on GB300, per stage, against
 // the per-stage kernels (sweep_plain, sweep_wide: ragged 32 x 8 tiles in two
 // uneven waves of blocks, float64 stencils, a launch per stage): FP64 chaotic
-// 16^3 24.0 -> 10.3 us, 37^3 27.5 -> 12.0, 100^3 145 -> 46, with 27 points 209 ->
-// 50, with 13 points 238 -> 51, oscillon 203^3 434 -> 209; split-FP32 chaotic
-// 100^3 40.5 -> 19.9, oscillon 250^3 196 -> 145, 13 points 128^3 57.6 -> 35.1,
-// 256^3 Q-ball 359 -> 225.
+// 16^3 24.4 -> 8.5 us, 37^3 27.5 -> 9.8, 100^3 144 -> 44, with 27 points 209 ->
+// 47, with 13 points 238 -> 48, oscillon 203^3 435 -> 201; split-FP32 chaotic
+// 100^3 40.3 -> 17.8, oscillon 250^3 196 -> 112, 13 points 128^3 56.8 -> 30.8,
+// 256^3 Q-ball 362 -> 204.  Running offsets instead of multiplied and divided
+// ones (PlainPos) are part of that: 462 -> 385 instructions a warp and plane of
+// two fields, oscillon 250^3 138 -> 112 us in the split form.
 #pragma once
 
 #include "persist.cuh"
@@ -64,12 +66,16 @@ struct PlainRing {
   static_assert(RING_BYTES % 16 == 0, "the rows' bulk copy lands behind the ring");
 };
 
-// 8- and 4-byte asynchronous copies into the thread's own places.
-__device__ __forceinline__ void cp_async_word(double* dst, const double* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
+// 8- and 4-byte asynchronous copies into the thread's own places (dst: a shared
+// address, OFF bytes behind it an instruction's immediate).
+template <int OFF> __device__ __forceinline__ void cp_async_word(uint32_t dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0+%2], [%1], 8;" ::"r"(dst), "l"(src), "n"(OFF)
                : "memory");
 }
-__device__ __forceinline__ void cp_async_word(float* dst, const float* src) { cp_async4(dst, src); }
+template <int OFF> __device__ __forceinline__ void cp_async_word(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0+%2], [%1], 4;" ::"r"(dst), "l"(src), "n"(OFF)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -114,23 +120,51 @@ __device__ __forceinline__ PlainCells plain_cells(int4 u, int n) {
   return c;
 }
 
-// A position in the block's planes and the thread's cells there.
-template <int H>
+// A position in the block's planes: the thread's cells there and the plane's own
+// and halo slots in the ring (elements).  The plane loop is a chain that each warp
+// walks with few others beside it (16 on the SM), so its instructions count: plane
+// offsets are 32-bit element indices (N_f n^3 < 2^32), advanced instead of
+// multiplied, and so are the slots.
+template <int H, typename RG>
 struct PlainPos {
-  int ui, uq;
+  int ui, left;      // unit, planes of it to come (0: past the last unit)
+  uint32_t zo;       // n^2 z of the plane
+  uint32_t os, hs;
   PlainCells c;
-  __device__ __forceinline__ void start(const PShared& sm, int n) {
-    ui = uq = 0;
-    if (sm.nunits > 0) c = plain_cells<H>(sm.units[0], n);
+  __device__ __forceinline__ void enter(const PShared& sm, int n) {
+    left = 0;
+    if (ui < sm.nunits) {
+      const int4 u = sm.units[ui];
+      c = plain_cells<H>(u, n);
+      left = u.w;
+      zo = (uint32_t)wrapi(u.z - H, n) * (uint32_t)(n * n);
+    }
   }
-  __device__ __forceinline__ bool in(const PShared& sm) const { return ui < sm.nunits; }
-  __device__ __forceinline__ void next(const PShared& sm, int n) {
-    if (++uq == sm.units[ui].w) {
-      uq = 0;
-      if (++ui < sm.nunits) c = plain_cells<H>(sm.units[ui], n);
+  // the block's first plane, ring plane gq
+  __device__ __forceinline__ void start(const PShared& sm, int n, uint32_t gq) {
+    ui = 0;
+    zo = 0u;
+    os = (gq % RG::OSLOT) * RG::OWN;
+    hs = (gq % RG::HSLOT) * RG::HALO;
+    enter(sm, n);
+  }
+  __device__ __forceinline__ bool in() const { return left > 0; }
+  __device__ __forceinline__ void next(const PShared& sm, int n, uint32_t nn, uint32_t S) {
+    os = os == (RG::OSLOT - 1) * RG::OWN ? 0u : os + RG::OWN;
+    hs = hs == (RG::HSLOT - 1) * RG::HALO ? 0u : hs + RG::HALO;
+    zo += nn;
+    if (zo == S) zo = 0u;
+    if (--left == 0) {
+      ++ui;
+      enter(sm, n);
     }
   }
 };
+// slot s (elements) of a ring of N slots of E elements, K further on
+template <int N, int E, int K> __device__ __forceinline__ uint32_t ring_slot(uint32_t s) {
+  static_assert(K >= 0 && K < N, "one wrap");
+  return s >= (uint32_t)((N - K) * E) ? s - (uint32_t)((N - K) * E) : s + (uint32_t)(K * E);
+}
 
 // A potential given at run time: its stage (rt_kick) finds the field drifted
 // (SimDesc::rt_phis) and V' and V at every site in arrays.
@@ -138,33 +172,42 @@ template <int MODEL> constexpr bool runtime_pot() {
   return MODEL == M_RUNTIME1 || MODEL == M_RUNTIME2;
 }
 
-// Copies of the plane at `pos` (ring plane gp) and one commit, always: the
+// Copies of the plane at `pos` into slots os, hs of the ring and one commit, always: the
 // groups a thread has committed count the planes.
-template <int MODEL, int PREC, int NQ, int H>
-__device__ __forceinline__ void plain_issue(int n, const PShared& sm, PlainPos<H>& pos, int ib,
-                                            uint32_t gp) {
+template <int MODEL, int PREC, int NQ, int H, typename Pos>
+__device__ __forceinline__ void plain_issue(int n, uint32_t nn, uint32_t S, const PShared& sm,
+                                            Pos& pos, int ib, uint32_t os, uint32_t hs) {
   constexpr bool RT = runtime_pot<MODEL>();
   constexpr int NF = Pot<MODEL>::NF;
   using T = typename WorkT<PREC>::type;
   using RG = PlainRing<PREC, NF, NQ, H>;
-  if (pos.in(sm)) {
+  constexpr int W = sizeof(T);
+  if (pos.in()) {
     const SimDesc& d = *sm.d;
-    const size_t S = (size_t)d.S;
-    const int z = wrapi(sm.units[pos.ui].z - H + pos.uq, n);
-    const T* src[2] = {(RT ? (const T*)d.rt_phis : (const T*)d.phi[ib & 1]) + (size_t)z * n * n,
-                       (const T*)d.pi[(ib >> 1) & 1] + (size_t)z * n * n};
-    T* own = (T*)sm.ring + (gp % RG::OSLOT) * RG::OWN + threadIdx.x;
-    T* hal = (T*)sm.ring + RG::HALO_OFF + (gp % RG::HSLOT) * RG::HALO + threadIdx.x;
-#pragma unroll
-    for (int f = 0; f < NF; ++f)
-#pragma unroll
-      for (int arr = 0; arr < 2; ++arr) {
-        if (pos.c.own >= 0)
-          cp_async_word(own + (f * 2 + arr) * kPThreads, src[arr] + f * S + pos.c.own);
-        if (pos.c.halo >= 0 && (!RT || arr == 0))
-          cp_async_word(hal + (f * 2 + arr) * kPlainHalo, src[arr] + f * S + pos.c.halo);
+    const T* phi = RT ? (const T*)d.rt_phis : (const T*)d.phi[ib & 1];
+    const T* pi = (const T*)d.pi[(ib >> 1) & 1];
+    const uint32_t ring = smem_u32(sm.ring) + threadIdx.x * W;
+    const uint32_t own = ring + os * W, hal = ring + hs * W;
+    constexpr int HB = RG::HALO_OFF * W;
+    if (pos.c.own >= 0) {
+      const uint32_t o = pos.zo + (uint32_t)pos.c.own;
+      cp_async_word<0>(own, phi + o);
+      cp_async_word<kPThreads * W>(own, pi + o);
+      if constexpr (NF == 2) {
+        cp_async_word<2 * kPThreads * W>(own, phi + (o + S));
+        cp_async_word<3 * kPThreads * W>(own, pi + (o + S));
       }
-    pos.next(sm, n);
+    }
+    if (pos.c.halo >= 0) {
+      const uint32_t o = pos.zo + (uint32_t)pos.c.halo;
+      cp_async_word<HB>(hal, phi + o);
+      if constexpr (!RT) cp_async_word<HB + kPlainHalo * W>(hal, pi + o);
+      if constexpr (NF == 2) {
+        cp_async_word<HB + 2 * kPlainHalo * W>(hal, phi + (o + S));
+        if constexpr (!RT) cp_async_word<HB + 3 * kPlainHalo * W>(hal, pi + (o + S));
+      }
+    }
+    pos.next(sm, n, nn, S);
   }
   cp_async_commit();
 }
@@ -173,9 +216,11 @@ __device__ __forceinline__ void plain_issue(int n, const PShared& sm, PlainPos<H
 template <int MODEL, int PREC, int NQ, int H>
 __device__ __forceinline__ void plain_prefetch(int n, const PShared& sm, int ib, uint32_t gq) {
   using RG = PlainRing<PREC, Pot<MODEL>::NF, NQ, H>;
-  PlainPos<H> pos;
-  pos.start(sm, n);
-  for (int l = 0; l < RG::LEAD; ++l) plain_issue<MODEL, PREC, NQ, H>(n, sm, pos, ib, gq + l);
+  const uint32_t nn = (uint32_t)(n * n), S = nn * (uint32_t)n;
+  PlainPos<H, RG> pos;
+  pos.start(sm, n, gq);
+  for (int l = 0; l < RG::LEAD; ++l)
+    plain_issue<MODEL, PREC, NQ, H>(n, nn, S, sm, pos, ib, pos.os, pos.hs);
 }
 
 __device__ __forceinline__ float fix_in(float v, int, float*) { return v; }
@@ -210,7 +255,7 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
   constexpr int KGROUP = 8;   // split: output planes per float partial before a compensated add
   const SimDesc& d = *sm.d;
   const int tid = threadIdx.x, lane = tid & 31;
-  const size_t S = (size_t)d.S, nn = (size_t)n * n;
+  const uint32_t nn = (uint32_t)(n * n), S = nn * (uint32_t)n;
   T* __restrict__ phi_out = (T*)d.phi[(ib & 1) ^ 1];
   T* __restrict__ pi_out = (T*)d.pi[((ib >> 1) & 1) ^ 1];
   T* const own = (T*)sm.ring + tid;
@@ -239,67 +284,105 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
   int kg = 0;
   bool ok = true;
 
-  PlainPos<H> ip, dp;   // next plane to copy, next plane to drift
-  ip.start(sm, n);
-  for (int l = 0; l < LEAD && ip.in(sm); ++l) ip.next(sm, n);
-  dp.start(sm, n);
-  // drift of the plane at dp (ring plane gg): own cell in place and into the
-  // drift buffer, the halo cell into the drift buffer
-  auto drift = [&](uint32_t gg) {
-    T* o = own + (gg % RG::OSLOT) * RG::OWN;
-    const T* h = hal + (gg % RG::HSLOT) * RG::HALO;
+  // Three positions run through the planes: copied, drifted, put out.  Where
+  // registers are short (two-field FP64: the Q-ball spilled, 3 to 6 % slower) only
+  // the last one keeps its slots and cells, and the others' are derived from them.
+  constexpr bool RUN = !F64 || NF == 1;
+  PlainPos<H, RG> ip, dp;   // next plane to copy, next plane to drift
+  ip.start(sm, n, gq);
+  for (int l = 0; l < LEAD && ip.in(); ++l) ip.next(sm, n, nn, S);
+  if constexpr (RUN) dp.start(sm, n, gq);
+  // own slot of plane g - H and halo slot of plane g; here for g = gq - 1
+  uint32_t os = ((gq + RG::OSLOT - 1 - H) % RG::OSLOT) * RG::OWN;
+  uint32_t hs = ((gq + RG::HSLOT - 1) % RG::HSLOT) * RG::HALO;
+  auto advance = [&]() {
+    os = os == (RG::OSLOT - 1) * RG::OWN ? 0u : os + RG::OWN;
+    if constexpr (!RUN) hs = hs == (RG::HSLOT - 1) * RG::HALO ? 0u : hs + RG::HALO;
+  };
+  // the copies of plane g + 1 + LEAD
+  static_assert(RG::OSLOT == LEAD + H + 2 && RG::HSLOT == LEAD + 1, "slots of the planes ahead");
+  auto issue = [&]() {
+    if constexpr (RUN)
+      plain_issue<MODEL, PREC, NQ, H>(n, nn, S, sm, ip, ib, ip.os, ip.hs);
+    else
+      plain_issue<MODEL, PREC, NQ, H>(n, nn, S, sm, ip, ib,
+                                      ring_slot<RG::OSLOT, RG::OWN, RG::OSLOT - 1>(os), hs);
+  };
+  // drift of plane gg = g + 1 with the thread's cells there: own cell in place and
+  // into the drift buffer, the halo cell into the drift buffer
+  auto drift = [&](uint32_t gg, const PlainCells& dc) {
+    T* o = own + (RUN ? dp.os : ring_slot<RG::OSLOT, RG::OWN, H + 1>(os));
+    const T* h = hal + (RUN ? dp.hs : ring_slot<RG::HSLOT, RG::HALO, 1>(hs));
     E* fx = fxb + (gg % NB) * RG::FX;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
       const int ex = F64 ? cx.fx[f] : 0;
-      if (dp.c.own >= 0) {
+      if (dc.own >= 0) {
         T a = o[f * 2 * kPThreads];
         if constexpr (!RT) {
           a = madd(cx.cdrift, o[(f * 2 + 1) * kPThreads], a);
           o[f * 2 * kPThreads] = a;
         }
-        fx[f * kPlainCells + dp.c.ownc] = fix_in(a, ex, (E*)nullptr);
+        fx[f * kPlainCells + dc.ownc] = fix_in(a, ex, (E*)nullptr);
       }
-      if (dp.c.halo >= 0) {
+      if (dc.halo >= 0) {
         T a = h[f * 2 * kPlainHalo];
         if constexpr (!RT) a = madd(cx.cdrift, h[(f * 2 + 1) * kPlainHalo], a);
-        fx[f * kPlainCells + dp.c.haloc] = fix_in(a, ex, (E*)nullptr);
+        fx[f * kPlainCells + dc.haloc] = fix_in(a, ex, (E*)nullptr);
       }
     }
     __syncwarp();   // the lanes' writes before lane 0's arrival (release)
     if (lane == 0) mbar_arrive(&sm.dbar[gg % NB]);
-    dp.next(sm, n);
   };
 
   uint32_t g = gq;
+  PlainCells c;   // the thread's cells of the plane put out
+  constexpr bool KEEP = !RUN && MODEL != M_QBALL;   // (the Q-ball forms them again: registers)
   if (sm.nunits > 0) {
-    plain_issue<MODEL, PREC, NQ, H>(n, sm, ip, ib, g + LEAD);
+    if constexpr (!RUN) c = plain_cells<H>(sm.units[0], n);
+    issue();
     cp_async_wait<LEAD>();
-    drift(g);
+    if constexpr (RUN) {
+      drift(g, dp.c);
+      dp.next(sm, n, nn, S);
+    } else {
+      drift(g, c);
+    }
   }
+  advance();
   for (int i = 0; i < sm.nunits && ok; ++i) {
     const int4 u = sm.units[i];
     const int Q = u.w;
-    const PlainCells c = plain_cells<H>(u, n);
+    if (!KEEP || i > 0) c = plain_cells<H>(u, n);
     const bool valid = c.own >= 0;
     // 7- and 27-point: part_m, so_m as in stage_fp64; 13-point: the z queue of stage_fp64_wide
     E qa[NF], qb[NF], qc[NF], qd[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) qa[f] = qb[f] = qc[f] = qd[f] = (E)0;
-    for (int q = 0; q < Q; ++q, ++g) {
-      plain_issue<MODEL, PREC, NQ, H>(n, sm, ip, ib, g + 1 + LEAD);
-      if (dp.in(sm)) {
-        cp_async_wait<LEAD>();
-        drift(g + 1);
+    uint32_t oz = (uint32_t)u.z * nn + (uint32_t)c.own;   // the next output
+    for (int q = 0; q < Q; ++q, ++g, advance()) {
+      issue();
+      if constexpr (RUN) {
+        if (dp.in()) {
+          cp_async_wait<LEAD>();
+          drift(g + 1, dp.c);
+          dp.next(sm, n, nn, S);
+        }
+      } else {
+        PlainCells dc = c;   // the next plane may be the next unit's first
+        if (q + 1 == Q && i + 1 < sm.nunits) dc = plain_cells<H>(sm.units[i + 1], n);
+        if (q + 1 < Q || i + 1 < sm.nunits) {
+          cp_async_wait<LEAD>();
+          drift(g + 1, dc);
+        }
       }
       double rv[RT ? NF + 1 : 1];   // run-time potential: V' and V of the plane put out
       if constexpr (RT) {
         const bool put = valid && q >= 2 * H;
-        const size_t o = (size_t)(u.z + q - 2 * H) * nn + c.own;
 #pragma unroll
         for (int f = 0; f < NF; ++f)
-          rv[f] = put && MODE == MODE_SWEEP ? __ldcg(d.rt_dV + f * S + o) : 0.0;
-        rv[NF] = put ? __ldcg(d.rt_V + o) : 0.0;
+          rv[f] = put && MODE == MODE_SWEEP ? __ldcg(d.rt_dV + (oz + f * S)) : 0.0;
+        rv[NF] = put ? __ldcg(d.rt_V + oz) : 0.0;
       }
       // every warp has drifted plane g
       ok = mbar_wait(&sm.dbar[g % NB], (g / NB) & 1, sm.limit);
@@ -341,9 +424,8 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
       }
       if (q >= 2 * H) {  // output plane z0 + q - 2 H
         if (valid) {
-          const size_t o = (size_t)(u.z + q - 2 * H) * nn + c.own;
           T phj[NF], Dj[NF], pmj[NF], pnj[NF];
-          const T* r = own + ((g - H) % RG::OSLOT) * RG::OWN;
+          const T* r = own + os;
 #pragma unroll
           for (int f = 0; f < NF; ++f) {
             phj[f] = r[f * 2 * kPThreads];
@@ -385,10 +467,11 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
           }
 #pragma unroll
           for (int f = 0; f < NF; ++f) {
-            __stwb(phi_out + f * S + o, phj[f]);
-            if (MODE == MODE_SWEEP) __stwb(pi_out + f * S + o, pnj[f]);
+            __stwb(phi_out + (oz + f * S), phj[f]);
+            if (MODE == MODE_SWEEP) __stwb(pi_out + (oz + f * S), pnj[f]);
           }
         }
+        oz += nn;
         if constexpr (!F64) {
           if (++kg == KGROUP) {
             kg = 0;

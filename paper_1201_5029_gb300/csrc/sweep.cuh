@@ -1114,7 +1114,9 @@ __device__ __forceinline__ void by_mode(int mode, bool fix, F&& body) {
 // row y0 + w, lane l owns sites x0 + l*VX .. +VX-1.  The drifted plane replaces
 // the plane's phi in its ring slot as the stencil wants it: in fixed point, or in
 // float64 for a stage without a scale (FIX).  Bound by the float64 pipe: serving
-// a batch of twelve requests up to 128^3, 41.3 -> see sweep_tma's note below.
+// a batch of twelve requests up to 128^3 took 41.3 ms with float64 stencils, 32.8
+// in fixed point, 25.9 with its mode as a compile-time constant; alone, a stage of a
+// 128^3 Q-ball 124 us, of a 32^3 oscillon 16.
 // ---------------------------------------------------------------------------
 template <int MODEL, int STENCIL, int VX>
 __global__ void __launch_bounds__(kThreads, 2) sweep_tma(const LaunchTable tab) {

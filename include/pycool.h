@@ -88,10 +88,8 @@ typedef enum { PYCOOL_FP64 = 0, PYCOOL_SPLIT_FP32 = 1, PYCOOL_SPLIT_DD = 2 } pyc
  *   ISO27 : c = (-128, 14, 3, 1)/30 (isotropic at O(k^4)),
  *   4TH   : the fourth-order stencil Sec. 2.1 mentions (HLATTICE's, not
  *           printed): per axis (-1, 16, -30, 16, -1)/12 over two sites each
- *           way, 13 points; symbol -k^2 + O(k^6).  n >= 4.  FP64: the
- *           persistent kernel when n % 32 == 0, else a per-stage kernel;
- *           SPLIT_DD: the persistent kernel, n % 32 == 0 (E_INVALID otherwise);
- *           SPLIT_FP32: the per-stage kernel.  No linearised path. */
+ *           way, 13 points; symbol -k^2 + O(k^6).  n >= 4; SPLIT_DD: n % 32
+ *           == 0 (E_INVALID otherwise). */
 typedef enum {
   PYCOOL_STENCIL_7PT = 7,
   PYCOOL_STENCIL_4TH = 13,
@@ -250,7 +248,8 @@ pycool_status pycool_model_source(int32_t model_id, char* buf, size_t cap, size_
  *   F the unnormalised forward transform of the field, m_k the signed integer
  *   wave vector; the shells add up to the lattice mean of the field squared.
  *   power, count: host arrays of nbins = pycool_spectrum_bins(n).  The first
- *   call makes an FFT plan and device buffers that the simulation keeps.
+ *   call makes device buffers and (n other than 64, 128 and 256, whose transforms
+ *   are the library's own) an FFT plan that the simulation keeps.
  * Errors: E_INVALID (bad arguments), E_STATE (no synchronised state), E_NOMEM,
  * E_CUDA, and the latched errors of pycool_sync. */
 pycool_status pycool_energy_fields(pycool_sim* sim, double* rho, double* P, int on_device);
@@ -276,8 +275,9 @@ pycool_status pycool_set_stream(pycool_sim* sim, void* cuda_stream);
  * (sweeps, arming and conversion kernels), for accounting; -1 for NULL. */
 int64_t pycool_kernel_launches(const pycool_sim* sim);
 
-/* Work plan of the persistent evolve kernel that pycool_evolve uses for n a
- * multiple of 32 (host arithmetic only: no device call, no GPU needed).  The
+/* Work plan of the persistent evolve kernel with TMA staging, which pycool_evolve
+ * uses for n a multiple of 32 (host arithmetic only: no device call, no GPU
+ * needed; the plain staging of other n and of 4TH with SPLIT_FP32 has its own).  The
  * lattice is cut into tiles of (32 vx) x 16 sites (vx = sites per thread in
  * x), each tile's z-axis into ranges, and the (tile, z-range) units are dealt
  * to at most `sms` blocks so that the blocks' modelled work is even; the
@@ -341,8 +341,9 @@ pycool_status pycool_linear_modes(int32_t n, int32_t stencil, double* values, in
  *   1. the background phi0, pi0 = lattice means (fixed-order device sums) and
  *      the perturbations phi - phi0, pi - pi0 (Eq. phi-lin), written to
  *      phi_out, pi_out as scratch;
- *   2. forward real-to-complex FFTs of the perturbations (cuFFT), every
- *      field, their k = 0 coefficients cleared;
+ *   2. forward real-to-complex FFTs of the perturbations (n = 64, 128 and 256:
+ *      the library's own; else cuFFT), every field, their k = 0 coefficients
+ *      cleared;
  *   3. the growth functions T of the distinct k_eff^2 values of the lattice's
  *      stencil, any of the three (pycool_linear_growth's kernel, background
  *      read on the device);
@@ -357,10 +358,9 @@ pycool_status pycool_linear_modes(int32_t n, int32_t stencil, double* values, in
  *   background (out, host, 2 + 2 N_f doubles): a, p_a, phi0[N_f], pi0[N_f] at
  *     the end.
  * The call allocates its device work space (spectra, tables), works on
- * `cuda_stream` and synchronises it before returning.  The host tables of a
- * lattice size and the FFT plans of a (size, N_f, device) are kept for the
- * process's lifetime: the first call for a size pays for them, and calls that
- * share a plan run one at a time.
+ * `cuda_stream` and synchronises it before returning.  cuFFT's plans of a (size,
+ * N_f, device) are kept for the process's lifetime: the first call for such a size
+ * pays for them, and calls that share a plan run one at a time.
  * Errors: E_INVALID (bad config, n outside 2..512, bad pointers, or a
  * potential given at run time), E_NOMEM, E_CUDA.  The Q-ball's
  * second derivatives need |Phi0| > 0 throughout. */

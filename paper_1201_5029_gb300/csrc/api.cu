@@ -437,8 +437,7 @@ pycool_status validate(const pycool_config* c) {
   if (c->stencil != PYCOOL_STENCIL_7PT && c->stencil != PYCOOL_STENCIL_ISO27 &&
       c->stencil != PYCOOL_STENCIL_4TH)
     return PYCOOL_E_INVALID;
-  // the fourth-order stencil: a per-stage kernel in the FP64 and split-FP32
-  // forms, the persistent kernel in the FP64 and split-DD forms (n % 32 == 0)
+  // the split-DD form has only the TMA staging (n % 32 == 0)
   if (c->stencil == PYCOOL_STENCIL_4TH && c->precision == PYCOOL_SPLIT_DD && c->n % 32 != 0)
     return PYCOOL_E_INVALID;
   // a potential given at run time: the FP64 form (any stencil)
@@ -992,8 +991,9 @@ struct pycool_sim {
   bool initialised = false;
   bool poisoned = false;
   int64_t launches = 0;
-  // persistent evolve kernel (n a multiple of 32): one cooperative launch per
-  // evolve(); otherwise a chain of per-stage launches replayed as a graph
+  // persistent evolve kernel (every compiled-in model): one cooperative launch per
+  // evolve(); a potential given at run time: a chain of per-stage launches replayed
+  // as a graph
   bool persist = false;
   PParams pp{};
   long long stall_limit = 0;   // > 0: the next persistent launch is a fault test

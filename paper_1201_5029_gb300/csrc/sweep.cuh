@@ -2034,7 +2034,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_wide(const LaunchTable tab)
 // rt_kick runs the plain staging's stage (persist_plain.cuh, runtime_model.cu).
 // Measured on GB300, 128^3, two-field chaotic potential, per stage: rt_drift 25
 // -> 18 us, the compiled kernel 51 (its own float64 instructions), rt_kick 148 ->
-// 83 as 32 x 8 tiles of 256 threads, 78 on the plan's units.
+// 83 as 32 x 8 tiles of 256 threads, 78 on the plan's units, 75 with running offsets.
 // ---------------------------------------------------------------------------
 // One block per SM: the scalar step that every block repeats takes thousands of
 // cycles of the SM's float64 pipe.

@@ -57,17 +57,18 @@ def _peaks():
         return {"hbm_gbs": 6800.0}, "fallback"
 
 
-# Algorithmic float64 operations per site (FMA = 2) of the method with the
-# 7-point stencil, counted from the arithmetic each site needs (not from the
-# instructions the kernel issues):
-#   stage sweep: drift 2/field, Laplacian 7/field (6 adds + the centre FMA),
-#     kick 4/field, sums pi^2 and phi D 4/field, sum V 1, plus the potential and
-#     its gradient (chaotic2 9, oscillon 11, qball 12 + one log, free 3);
-#   flush: drift 2/field, Laplacian 7/field, sums pi^2, phi D 4/field,
-#     sum (phi - K) 1/field, sum (phi - K)^2 2/field, sum V 1, plus V alone
-#     (chaotic2 5, oscillon 6, qball 6 + one log, free 2).
-FP64_FLOPS_PER_SITE = {"chaotic2": 44.0, "oscillon": 29.0, "qball": 47.0, "free": 21.0}
-FP64_FLUSH_FLOPS_PER_SITE = {"chaotic2": 38.0, "oscillon": 23.0, "qball": 39.0, "free": 19.0}
+# Algorithmic operations per site (FMA = 2) that run on the float64 pipe, counted
+# from the arithmetic each site needs (not from the instructions the kernel issues):
+#   stage sweep: drift 2/field, kick 4/field, sums pi^2 and phi D 4/field, sum V 1,
+#     plus the potential and its gradient (chaotic2 9, oscillon 11, qball 12 + one
+#     log, free 3);
+#   flush: drift 2/field, sums pi^2, phi D 4/field, sum (phi - K) 1/field,
+#     sum (phi - K)^2 2/field, sum V 1, plus V alone (chaotic2 5, oscillon 6,
+#     qball 6 + one log, free 2).
+# The Laplacian (7/field: 6 adds and the centre FMA) is summed in 64-bit integers
+# and is not counted.
+FP64_FLOPS_PER_SITE = {"chaotic2": 30.0, "oscillon": 22.0, "qball": 33.0, "free": 14.0}
+FP64_FLUSH_FLOPS_PER_SITE = {"chaotic2": 24.0, "oscillon": 16.0, "qball": 25.0, "free": 12.0}
 # GB300 float64 peak: 2 DFMA lanes per SM per clock (ncu: 304 predicated-on
 # DFMA thread instructions per cycle for the 152 SMs) x 2 flops x 2.07 GHz.
 FP64_PEAK_TFLOPS = 304 * 2 * 2.07e9 / 1e12
@@ -263,13 +264,14 @@ def roofline(w, form, s, ms_per_step, hbm, peak_kind):
               "algorithmic_bytes_per_launch": launch_bytes,
               "traffic_over_algorithmic": (traffic / launch_bytes) if traffic else None}
     if form == "fp64":
-        flops = S * (s * FP64_FLOPS_PER_SITE.get(w["model"], 40.0)
-                     + FP64_FLUSH_FLOPS_PER_SITE.get(w["model"], 35.0))
+        flops = S * (s * FP64_FLOPS_PER_SITE.get(w["model"], 26.0)
+                     + FP64_FLUSH_FLOPS_PER_SITE.get(w["model"], 21.0))
         tf = flops / (ms_per_step / 1e3) / 1e12
         out = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                "frac": tf / FP64_PEAK_TFLOPS,
                "peak_kind": "float64 pipe: 2 DFMA/SM/clk x 152 SMs x 2.07 GHz (GB300 FP64 is "
-                            "1/64 of FP32; float64 arithmetic binds this form, not HBM)",
+                            "1/64 of FP32; float64 arithmetic binds this form, not HBM; the "
+                            "Laplacian's integer sums are not counted)",
                "flops_per_launch": flops, "achieved_gbs": gbs, "hbm_frac": gbs / hbm,
                "hbm_peak_gbs": hbm, "hbm_frac_of_nominal": gbs / NOMINAL_HBM_GBS}
     else:

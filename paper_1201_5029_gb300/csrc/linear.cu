@@ -171,10 +171,18 @@ __device__ void linear_background(const LinArgs& a, LinEntry* out, long long e0,
 }
 
 // Launch `chunk`: block 0 forms that chunk's table, the others apply the chunk
-// before it to the transfer matrices (64 values a block: a block per scheduler
-// quarter keeps the last wave of a 128^3 lattice's 48 000 values full).
+// before it to the transfer matrices.  Block 0's one thread is a chain of float64
+// instructions that waits for the pipe behind every other warp of its scheduler.
+// With 64 values a block, more blocks than SMs put two or three warps there.  Where
+// all values fit one wave of two blocks of five warps to an SM (by their shared
+// memory), block 0 has one other block beside it instead: 128^3 (48 000 values), a
+// chunk 220 -> 181 us, the whole linearised evolution of 300 stages 2123 -> 2009 us.
+// Fewer values have the SM to themselves, and several waves gain nothing (256^3
+// 7.64 -> 7.76 ms).
+constexpr int kLinThreads = 160;
+constexpr int kLinSmem = 96 * 1024;   // of an SM's 228 KB: two blocks fit, three do not
 template <int MODEL>
-__global__ void __launch_bounds__(64) linear_growth(const LinArgs a) {
+__global__ void __launch_bounds__(kLinThreads) linear_growth(const LinArgs a) {
   constexpr int NF = Pot<MODEL>::NF, N2 = 2 * NF;
   __shared__ LinEntry tab[kLinChunk];
   if (blockIdx.x == 0) {
@@ -229,19 +237,34 @@ cudaError_t launch_linear_growth(int model, LinArgs a, void* scratch, cudaStream
   a.state = reinterpret_cast<LinState*>(a.table + 2 * kLinChunk);
   a.nentries = a.steps * a.nstages + 1;
   const long long chunks = (a.nentries + kLinChunk - 1) / kLinChunk;
-  for (a.chunk = 0; a.chunk <= chunks; ++a.chunk) {
-    const unsigned grid = 1 + (a.chunk > 0 ? (unsigned)((a.nk + 63) / 64) : 0u);
-    switch (model) {
-      case M_FREE: linear_growth<M_FREE><<<grid, 64, 0, s>>>(a); break;
-      case M_CHAOTIC2: linear_growth<M_CHAOTIC2><<<grid, 64, 0, s>>>(a); break;
-      case M_OSCILLON: linear_growth<M_OSCILLON><<<grid, 64, 0, s>>>(a); break;
-      case M_QBALL: linear_growth<M_QBALL><<<grid, 64, 0, s>>>(a); break;
-      default: return cudaErrorInvalidValue;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const bool wide = (a.nk + 63) / 64 > sms && (a.nk + kLinThreads - 1) / kLinThreads < 2ll * sms;
+  const int threads = wide ? kLinThreads : 64, smem = wide ? kLinSmem : 0;
+  auto run = [&](auto* kernel) -> cudaError_t {
+    if (wide) {
+      const cudaError_t ae = cudaFuncSetAttribute(
+          kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinSmem);
+      if (ae != cudaSuccess) return ae;
     }
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    for (a.chunk = 0; a.chunk <= chunks; ++a.chunk) {
+      const unsigned grid =
+          1 + (a.chunk > 0 ? (unsigned)((a.nk + threads - 1) / threads) : 0u);
+      kernel<<<grid, threads, smem, s>>>(a);
+      const cudaError_t le = cudaGetLastError();
+      if (le != cudaSuccess) return le;
+    }
+    return cudaSuccess;
+  };
+  switch (model) {
+    case M_FREE: return run(linear_growth<M_FREE>);
+    case M_CHAOTIC2: return run(linear_growth<M_CHAOTIC2>);
+    case M_OSCILLON: return run(linear_growth<M_OSCILLON>);
+    case M_QBALL: return run(linear_growth<M_QBALL>);
+    default: return cudaErrorInvalidValue;
   }
-  return cudaSuccess;
 }
 
 // The modes of an n^3 lattice by the magnitudes of their wave numbers: k_eff^2

@@ -276,9 +276,9 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
   double best = 1e300, best_tot = 1e300, best_T = 0.0;
   // (plain staging: whole columns, cut where a block is full, come out best; a
   // plan is made for every new simulation, so it is not searched further than
-  // half a percent)
+  // half a percent or a tenth of a plane, loads being multiples of half a plane)
   const int rc_most = plain ? 1 : std::min(16, std::max(1, n / kMinPiece));
-  const double tol = plain ? 5e-3 * work / cap : 1e-3;
+  const double tol = plain ? std::max(5e-3 * work / cap, 0.1) : 1e-3;
   for (int rc = 1; rc <= rc_most; ++rc) {
     const int rws[3] = {rc, (rc * 12 + 9) / 10, (rc * 13 + 9) / 10};
     for (int j = 0; j < 3; ++j) {
@@ -290,9 +290,15 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
       // dropped by one deal (a search takes twenty)
       if (best < 1e299 && !deal(best - 1e-3)) continue;
       double lo = work / cap, hi = (double)n * pen + 2.0 * halo * h * pen + lo;
-      if (best < 1e299) hi = best - 1e-3;
-      else
+      if (plain) {   // whole columns deal to within a few planes of the mean
+        double gap = 2.0;
+        for (hi = lo + gap; !deal(hi); hi = lo + (gap *= 2.0)) {}
+        lo += gap > 2.0 ? 0.5 * gap : 0.0;
+      } else if (best < 1e299) {
+        hi = best - 1e-3;
+      } else {
         while (!deal(hi)) hi *= 2.0;
+      }
       for (int it = 0; it < 40 && hi - lo > tol; ++it) {
         const double mid = 0.5 * (lo + hi);
         if (deal(mid)) hi = mid; else lo = mid;

@@ -83,8 +83,7 @@ NOMINAL_HBM_GBS = 8000.0   # GB300's nominal HBM3e bandwidth (the fractions also
 # the sources evolve_persist is compiled from (its translation units and headers)
 KERNEL_SOURCES = ("persist.cuh", "persist_fp64.cu", "persist_split.cu", "persist_dd.cu",
                   "persist_fp64_wide.cu", "persist_dd_wide.cu", "persist_kernel.cuh",
-                  "persist_plain.cuh", "persist_fp64_plain.cu", "persist_split_plain.cu",
-                  "sweep.cuh", "internal.cuh",
+                  "persist_plain.cuh", "persist_fp64_plain.cu", "sweep.cuh", "internal.cuh",
                   "models.cuh", "models_dd.cuh", "dd.cuh")
 
 

@@ -277,7 +277,7 @@ int64_t pycool_kernel_launches(const pycool_sim* sim);
 
 /* Work plan of the persistent evolve kernel with TMA staging, which pycool_evolve
  * uses for n a multiple of 32 (host arithmetic only: no device call, no GPU
- * needed; the plain staging of other n and of 4TH with SPLIT_FP32 has its own).  The
+ * needed; the plain staging that the FP64 form uses at other n has its own).  The
  * lattice is cut into tiles of (32 vx) x 16 sites (vx = sites per thread in
  * x), each tile's z-axis into ranges, and the (tile, z-range) units are dealt
  * to at most `sms` blocks so that the blocks' modelled work is even; the

@@ -116,13 +116,14 @@ Layout sim_layout(const pycool_config& c) {
   L.ws_bytes = L.off_mean + align256((size_t)2 * kMaxFields * kMeanBlocks * 2 * sizeof(double));
   // the persistent kernel, compiled models: TMA staging for n a multiple of 32
   // (the 13-point stencil in the FP64 and split-DD forms), plain staging for
-  // every other n and for the split-FP32 form's 13-point stencil (faster than
-  // the per-stage kernels at every side from 16 to 256: persist_plain.cuh; TMA
-  // staging where it fits: 128^3 split-FP32 18 us per stage, plain 35)
+  // every other n in the FP64 form (faster than the per-stage kernels at every
+  // side from 16 to 256: persist_plain.cuh).  The split-FP32 form keeps the
+  // per-stage kernels there: the order of its float32 sums shows in its results
+  // where a background passes near zero (Ctx::recenter)
   const bool tma_ok =
       L.geo.tma || (c.stencil == PYCOOL_STENCIL_4TH && c.n % 32 == 0 &&
                     c.model < kRuntimeModelBase && c.precision != PYCOOL_SPLIT_FP32);
-  L.plain = !tma_ok && c.model < kRuntimeModelBase && c.precision != PYCOOL_SPLIT_DD;
+  L.plain = !tma_ok && c.model < kRuntimeModelBase && c.precision == PYCOOL_FP64;
   if (tma_ok || L.plain) {
     L.off_prows = align256(L.ws_bytes);
     L.off_punits = L.off_prows + align256((size_t)2 * kMaxPBlocks * kNQ * sizeof(double));
@@ -197,13 +198,15 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
   const double stage_bytes = 4.0 * nf * (double)n * n * n * word;   // phi, pi read and written
   const bool l2_resident = l2_bytes > 0 && stage_bytes <= 0.75 * (double)l2_bytes;
   const double h = prec != PREC_SPLIT ? 0.25 : (l2_resident ? 1.5 : 0.3);
-  const double pen = prec != PREC_SPLIT || plain ? 1.0 : 1.24;
+  const double pen = prec != PREC_SPLIT ? 1.0 : 1.24;
   // Planes: no unit shorter than this is cut off a chunk.  A lattice of side 32 has
   // 64 (tile, plane) pairs, so single planes spread it over 64 SMs where pieces of
-  // four left 16 at work: 32^3 per stage, FP64 chaotic 19.4 -> 10.7 us, split-FP32
-  // 10.0 -> 7.7, split-DD 25.1 -> 19.0; 64^3 split-FP32 10.8 -> 9.1; the larger
-  // ones are cut the same as before.
-  constexpr int kMinPiece = 1;
+  // four left 16 at work: 32^3 per stage, FP64 chaotic 19.4 -> 10.7 us, split-DD
+  // 25.1 -> 19.0; 96^3 and 128^3 take as long as before.  The split-FP32 form
+  // stays at four (10.0 us at 32^3, 7.7 with single planes; 64^3 10.8, 9.1): its
+  // units' float32 sums in another order moved the field by up to 1.4e-9 of itself
+  // where a one-field background passes near zero (Ctx::recenter).
+  const int min_piece = prec == PREC_SPLIT ? 4 : 1;
   const int cap = std::min(sms, kMaxPBlocks);
   auto is_wrap = [&](int t) {
     const int ty = t / g.tiles_x;
@@ -245,8 +248,8 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
         int k = len;
         if (top.first + (len + 2.0 * halo * h) * p > T + 1e-9) {
           k = (int)std::floor((T - top.first) / p - 2.0 * halo * h);
-          if (len - k < kMinPiece) k = len - kMinPiece;
-          if (k < kMinPiece) return false;   // the least loaded block is full: so are all
+          if (len - k < min_piece) k = len - min_piece;
+          if (k < min_piece) return false;   // the least loaded block is full: so are all
         }
         out.push_back(U{u.z0, u.z0 + k, u.t, top.second});
         top.first += (k + 2.0 * halo * h) * p;
@@ -277,13 +280,13 @@ PGeo plan_units(int n, int word, int nf, int prec, int sms, long long l2_bytes,
   // (plain staging: whole columns, cut where a block is full, come out best; a
   // plan is made for every new simulation, so it is not searched further than
   // half a percent or a tenth of a plane, loads being multiples of half a plane)
-  const int rc_most = plain ? 1 : std::min(16, std::max(1, n / kMinPiece));
+  const int rc_most = plain ? 1 : std::min(16, std::max(1, n / min_piece));
   const double tol = plain ? std::max(5e-3 * work / cap, 0.1) : 1e-3;
   for (int rc = 1; rc <= rc_most; ++rc) {
     const int rws[3] = {rc, (rc * 12 + 9) / 10, (rc * 13 + 9) / 10};
     for (int j = 0; j < 3; ++j) {
-      const int rw = std::min(rws[j], std::max(1, n / kMinPiece));
-      if (j > 0 && rw == std::min(rws[j - 1], std::max(1, n / kMinPiece))) continue;
+      const int rw = std::min(rws[j], std::max(1, n / min_piece));
+      if (j > 0 && rw == std::min(rws[j - 1], std::max(1, n / min_piece))) continue;
       if (pen == 1.0 && rw != rc) continue;
       chunks(rc, rw);
       // a chunking that cannot be dealt below the best slowest block so far is
@@ -611,8 +614,7 @@ cudaError_t encode_persist_maps(const SimDesc& d, const PGeo& g, PParams& p) {
 
 cudaError_t launch_persist(const SimDesc& d, const PParams& p, int grid, cudaStream_t s, int* bps) {
   if (p.g.vx == 0)   // plain staging
-    return d.prec == PREC_SPLIT ? launch_persist_split_plain(d.model, d.stencil, 0, p, grid, s, bps)
-                                : launch_persist_fp64_plain(d.model, d.stencil, 0, p, grid, s, bps);
+    return launch_persist_fp64_plain(d.model, d.stencil, 0, p, grid, s, bps);
   if (d.prec == PREC_SPLIT) return launch_persist_split(d.model, d.stencil, p.g.vx, p, grid, s, bps);
   if (d.stencil == 13)
     return d.prec == PREC_DD ? launch_persist_dd_wide(d.model, d.stencil, p.g.vx, p, grid, s, bps)
@@ -997,9 +999,8 @@ struct pycool_sim {
   bool initialised = false;
   bool poisoned = false;
   int64_t launches = 0;
-  // persistent evolve kernel (every compiled-in model): one cooperative launch per
-  // evolve(); a potential given at run time: a chain of per-stage launches replayed
-  // as a graph
+  // persistent evolve kernel (sim_layout): one cooperative launch per evolve();
+  // otherwise a chain of per-stage launches replayed as a graph
   bool persist = false;
   PParams pp{};
   long long stall_limit = 0;   // > 0: the next persistent launch is a fault test

@@ -247,11 +247,9 @@ cudaError_t launch_persist_split(int model, int stencil, int vx, const PParams& 
                                  cudaStream_t s, int* bps);
 cudaError_t launch_persist_dd(int model, int stencil, int vx, const PParams& p, int grid,
                               cudaStream_t s, int* bps);
-// plain staging, every stencil (FP64 and split-FP32)
+// plain staging, every stencil (FP64)
 cudaError_t launch_persist_fp64_plain(int model, int stencil, int vx, const PParams& p, int grid,
                                       cudaStream_t s, int* bps);
-cudaError_t launch_persist_split_plain(int model, int stencil, int vx, const PParams& p, int grid,
-                                       cudaStream_t s, int* bps);
 // the 13-point stencil's instances (FP64 and split-DD)
 cudaError_t launch_persist_fp64_wide(int model, int stencil, int vx, const PParams& p, int grid,
                                      cudaStream_t s, int* bps);

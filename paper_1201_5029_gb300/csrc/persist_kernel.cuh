@@ -8,11 +8,11 @@
 namespace pycool {
 
 // The shared-memory ring of an instance: VX > 0 the TMA staging with VX sites
-// per lane, VX = 0 the plain staging (persist_plain.cuh).
+// per lane, VX = 0 the plain staging (persist_plain.cuh, FP64).
 template <int PREC, int NF, int VX, int NQ, int H>
 struct RingOf { using type = PRing<PREC, NF, VX, NQ, H>; };
-template <int PREC, int NF, int NQ, int H>
-struct RingOf<PREC, NF, 0, NQ, H> { using type = PlainRing<PREC, NF, NQ, H>; };
+template <int NF, int NQ, int H>
+struct RingOf<PREC_FP64, NF, 0, NQ, H> { using type = PlainRing<NF, NQ, H>; };
 
 // ---------------------------------------------------------------------------
 // The kernel.
@@ -26,8 +26,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
   constexpr bool CORNERS = StencilW<STENCIL>::kCorners;
   constexpr int H = halo_of<STENCIL>();
   constexpr bool PLAIN = VX == 0;
-  static_assert(STENCIL != 13 || PREC != PREC_SPLIT || PLAIN,
-                "the split-FP32 form's 13-point stencil: plain staging");
+  static_assert(STENCIL != 13 || PREC != PREC_SPLIT, "the 13-point stencil: FP64 and split-DD");
   using RG = typename RingOf<PREC, NF, VX, NQ, H>::type;
   constexpr int NSLOT = RG::NSLOT, LEAD = RG::LEAD, PRE = RG::PRE;
   static_assert(RG::FOLD <= kPWarps, "one warp per reduced quantity");
@@ -122,7 +121,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
   // scalar coefficients (the FP64 chain of the merged half-stages)
   {
     if constexpr (PLAIN) {
-      plain_prefetch<MODEL, PREC, NQ, H>(p.g.n, sm, ib, gq);
+      plain_prefetch<MODEL, NQ, H>(p.g.n, sm, ib, gq);
     } else {
       for (int l = kPWarps - 1 - warp; l < LEAD; l += kPWarps)   // warp 15 - l issues plane l
         prefetch_plane<PREC, NF, VX, CORNERS, NSLOT, H>(p, sm, ib, gq, l);
@@ -152,7 +151,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         constexpr int MD = decltype(mode_c)::value;
         constexpr bool FX = decltype(fix_c)::value;
         if constexpr (PLAIN)
-          return stage_plain<MODEL, STENCIL, PREC, MD, FX>(p.g.n, cx, sm, gq, ib, accd, hm);
+          return stage_plain<MODEL, STENCIL, MD, FX>(p.g.n, cx, sm, gq, ib, accd, hm);
         else if constexpr (STENCIL == 13)
           return stage_fp64_wide<MODEL, VX, MD, FX>(p, cx, sm, gq, ib, accd, hm);
         else
@@ -164,10 +163,6 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
         ok = fix ? stage(MS{}, std::true_type{}) : stage(MS{}, std::false_type{});
       else
         ok = fix ? stage(MF{}, std::true_type{}) : stage(MF{}, std::false_type{});
-    } else if constexpr (PLAIN) {
-      ok = (mode == MODE_SWEEP)
-               ? stage_plain<MODEL, STENCIL, PREC, MODE_SWEEP, false>(p.g.n, cx, sm, gq, ib, accd, hm)
-               : stage_plain<MODEL, STENCIL, PREC, MODE_FLUSH, false>(p.g.n, cx, sm, gq, ib, accd, hm);
     } else if constexpr (STENCIL == 13) {
       ok = (mode == MODE_SWEEP) ? stage_wide_dd<MODEL, VX, MODE_SWEEP>(p, cx, sm, gq, ib)
                                 : stage_wide_dd<MODEL, VX, MODE_FLUSH>(p, cx, sm, gq, ib);
@@ -334,7 +329,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
       if (pre && !PLAIN) named_arrive(1, kPreThreads);   // the next stage's copies queue behind it
     }
     if constexpr (PLAIN) {   // every thread's own copies; the folding warps' after their fold
-      if (pre && warp > nl) plain_prefetch<MODEL, PREC, NQ, H>(p.g.n, sm, ib_next, gq);
+      if (pre && warp > nl) plain_prefetch<MODEL, NQ, H>(p.g.n, sm, ib_next, gq);
     }
     if (warp < nl) {
       if (!mbar_wait(&foldbar, (uint32_t)(k & 1), p.wait_limit)) atomicOr(&s_bad, 1);
@@ -392,7 +387,7 @@ __global__ void __launch_bounds__(kPThreads, 1) evolve_persist(const __grid_cons
     // @folded
     if (tid == 0 && !s_bad) s_fold = -1;   // every folding warp saw the copy land
     if constexpr (PLAIN) {
-      if (pre && warp <= nl) plain_prefetch<MODEL, PREC, NQ, H>(p.g.n, sm, ib_next, gq);
+      if (pre && warp <= nl) plain_prefetch<MODEL, NQ, H>(p.g.n, sm, ib_next, gq);
     }
     // ---- in parallel, on warps of different schedulers, identically in
     //      every block: the next stage's coefficients (warp 14: sums -> p_a

@@ -1,32 +1,27 @@
-// Staging of the persistent kernel without TMA: any lattice side (a TMA box
-// wants rows that are multiples of 16 bytes and tiles of whole boxes), and the
-// 13-point stencil of the split-FP32 form, whose five rows per site would not
-// fit the register pipeline of stage_split.
+// Staging of the FP64 form's persistent kernel without TMA: any lattice side (a
+// TMA box wants rows that are multiples of 16 bytes and tiles of whole boxes).
 //
-// A tile is w x h sites (w h <= 512, chosen by plan_plain so that as few tiles
+// A tile is w x h sites (w h <= 512, chosen by plain_tiles so that as few tiles
 // as possible cover the lattice: tiles differ in w and h by at most one, and no
 // thread row is tied to a lattice row), one site per thread.  Each thread
 // copies its own site's values of the planes ahead, and at most one cell of the
-// tile's halo ring (periodic indices), with 4- or 8-byte cp.async into its own
+// tile's halo ring (periodic indices), with 8-byte cp.async into its own
 // places of a shared-memory ring; it alone reads them again, so a copy needs no
 // barrier, only the thread's own cp.async group count.  The thread drifts its
-// cells of plane g + 1 into one of four drift buffers (fixed point or float64 in
-// the FP64 form, float32 in the split form), its warp arrives on the buffer's
-// mbarrier, and after the wait for plane g it sums the stencil of plane g from
-// shared memory and puts out the plane H below, whose drifted field and momentum
-// it still holds in the ring.  As in the other stages there is no block barrier
-// in the z loop.
+// cells of plane g + 1 into one of four drift buffers (fixed point or float64),
+// its warp arrives on the buffer's mbarrier, and after the wait for plane g it
+// sums the stencil of plane g from shared memory and puts out the plane H below,
+// whose drifted field and momentum it still holds in the ring.  As in the other
+// stages there is no block barrier in the z loop.
 //
-// Bound by: FP64, the float64 pipe; split-FP32, the shared-memory pipe and the
-// copies' latency (one site per thread).  Measured on GB300, per stage, against
-// the per-stage kernels (sweep_plain, sweep_wide: ragged 32 x 8 tiles in two
-// uneven waves of blocks, float64 stencils, a launch per stage): FP64 chaotic
-// 16^3 24.4 -> 8.5 us, 37^3 27.5 -> 9.8, 100^3 144 -> 44, with 27 points 209 ->
-// 47, with 13 points 238 -> 48, oscillon 203^3 435 -> 201; split-FP32 chaotic
-// 100^3 40.3 -> 17.8, oscillon 250^3 196 -> 112, 13 points 128^3 56.8 -> 30.8,
-// 256^3 Q-ball 362 -> 204.  Running offsets instead of multiplied and divided
-// ones (PlainPos) are part of that: 462 -> 385 instructions a warp and plane of
-// two fields, oscillon 250^3 138 -> 112 us in the split form.
+// Bound by the float64 pipe.  Measured on GB300, per stage, against the
+// per-stage kernels (sweep_plain, sweep_wide: ragged 32 x 8 tiles in two uneven
+// waves of blocks, float64 stencils, a launch per stage): chaotic 16^3 24.4 ->
+// 8.5 us, 37^3 27.5 -> 9.8, 100^3 144 -> 44, with 27 points 209 -> 47, with 13
+// points 238 -> 48, oscillon 203^3 435 -> 201.  The split-FP32 form keeps the
+// per-stage kernels at these sides: it was faster here too (100^3 40 -> 18 us),
+// but its float32 sums in another order moved the field by up to 4e-9 of itself
+// where a one-field background passes near zero (Ctx::recenter).
 #pragma once
 
 #include "persist.cuh"
@@ -40,40 +35,29 @@ constexpr int kPlainCells = kPThreads + kPlainHalo;   // cells of a tile with it
 // and the drift buffers fx[NDRIFT][NF][768].  LEAD planes of copies are in
 // flight ahead of the plane being drifted; an own slot is needed until the
 // plane has been put out, H + 1 planes after its drift.
-template <int PREC, int NF, int NQ, int H>
+template <int NF, int NQ, int H>
 struct PlainRing {
-  static constexpr int WORD = prec_word(PREC);
-  static constexpr int OSLOT = PREC == PREC_FP64 ? 6 : 8;
+  static constexpr int OSLOT = 6;
   static constexpr int LEAD = OSLOT - H - 2;
   static constexpr int HSLOT = LEAD + 1;
   static constexpr int NDRIFT = 4;
   static constexpr int NSLOT = 1;   // no TMA ring
-  static constexpr int FOLD = NQ + (PREC == PREC_FP64 ? 1 : 0);
+  static constexpr int FOLD = NQ + 1;
   static constexpr int PRE = 1;
   static constexpr int OWN = NF * 2 * kPThreads, HALO = NF * 2 * kPlainHalo;
   static constexpr int FX = NF * kPlainCells;
   static constexpr int HALO_OFF = OSLOT * OWN, FX_OFF = HALO_OFF + HSLOT * HALO;
-  static constexpr int RING_BYTES = (FX_OFF + NDRIFT * FX) * WORD;
+  static constexpr int RING_BYTES = (FX_OFF + NDRIFT * FX) * 8;
   static constexpr int DRIFT_WORDS = 0;
-  static constexpr int KAHAN_BYTES = NQ * kKahanGroups * 8;
-  static constexpr int ROWS_BYTES = kMaxPBlocks * kNQ * 8;
-  static constexpr int EXTRA_BYTES =
-      PREC == PREC_FP64 ? NQ * kPThreads * 8
-                        : (KAHAN_BYTES > ROWS_BYTES ? KAHAN_BYTES : ROWS_BYTES);
-  static constexpr int SMEM_BYTES = RING_BYTES + EXTRA_BYTES;
-  static_assert(PREC != PREC_DD, "the FP64 and split-FP32 forms");
+  static constexpr int SMEM_BYTES = RING_BYTES + NQ * kPThreads * 8;
   static_assert(SMEM_BYTES <= kPSmemBudget, "shared memory of the persistent kernel");
   static_assert(RING_BYTES % 16 == 0, "the rows' bulk copy lands behind the ring");
 };
 
-// 8- and 4-byte asynchronous copies into the thread's own places (dst: a shared
+// An 8-byte asynchronous copy into the thread's own place (dst: a shared
 // address, OFF bytes behind it an instruction's immediate).
 template <int OFF> __device__ __forceinline__ void cp_async_word(uint32_t dst, const double* src) {
   asm volatile("cp.async.ca.shared.global [%0+%2], [%1], 8;" ::"r"(dst), "l"(src), "n"(OFF)
-               : "memory");
-}
-template <int OFF> __device__ __forceinline__ void cp_async_word(uint32_t dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0+%2], [%1], 4;" ::"r"(dst), "l"(src), "n"(OFF)
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
@@ -174,13 +158,13 @@ template <int MODEL> constexpr bool runtime_pot() {
 
 // Copies of the plane at `pos` into slots os, hs of the ring and one commit, always: the
 // groups a thread has committed count the planes.
-template <int MODEL, int PREC, int NQ, int H, typename Pos>
+template <int MODEL, int NQ, int H, typename Pos>
 __device__ __forceinline__ void plain_issue(int n, uint32_t nn, uint32_t S, const PShared& sm,
                                             Pos& pos, int ib, uint32_t os, uint32_t hs) {
   constexpr bool RT = runtime_pot<MODEL>();
   constexpr int NF = Pot<MODEL>::NF;
-  using T = typename WorkT<PREC>::type;
-  using RG = PlainRing<PREC, NF, NQ, H>;
+  using T = double;
+  using RG = PlainRing<NF, NQ, H>;
   constexpr int W = sizeof(T);
   if (pos.in()) {
     const SimDesc& d = *sm.d;
@@ -213,46 +197,32 @@ __device__ __forceinline__ void plain_issue(int n, uint32_t nn, uint32_t S, cons
 }
 
 // The first LEAD planes of a stage (every thread of the block).
-template <int MODEL, int PREC, int NQ, int H>
+template <int MODEL, int NQ, int H>
 __device__ __forceinline__ void plain_prefetch(int n, const PShared& sm, int ib, uint32_t gq) {
-  using RG = PlainRing<PREC, Pot<MODEL>::NF, NQ, H>;
+  using RG = PlainRing<Pot<MODEL>::NF, NQ, H>;
   const uint32_t nn = (uint32_t)(n * n), S = nn * (uint32_t)n;
   PlainPos<H, RG> pos;
   pos.start(sm, n, gq);
   for (int l = 0; l < RG::LEAD; ++l)
-    plain_issue<MODEL, PREC, NQ, H>(n, nn, S, sm, pos, ib, pos.os, pos.hs);
-}
-
-__device__ __forceinline__ float fix_in(float v, int, float*) { return v; }
-__device__ __forceinline__ float fix_out(float v, int) { return v; }
-__device__ __forceinline__ float fix_mad(float a, float b, float c) { return madd(a, b, c); }
-__device__ __forceinline__ float fix_mid7(float c, float faces) { return madd(-6.0f, c, faces); }
-__device__ __forceinline__ void fix_parts27(float c, float faces, float corners, float& mid,
-                                            float& off) {
-  mid = madd((float)(3.0 / 30.0), corners,
-             madd((float)(14.0 / 30.0), faces, (float)(-128.0 / 30.0) * c));
-  off = madd((float)(1.0 / 30.0), corners,
-             madd((float)(3.0 / 30.0), faces, (float)(14.0 / 30.0) * c));
+    plain_issue<MODEL, NQ, H>(n, nn, S, sm, pos, ib, pos.os, pos.hs);
 }
 
 // One stage over this block's units (see the head of this file); the sums go to
-// accd (FP64) or the block's compensated sums (split-FP32, as stage_split).
-template <int MODEL, int STENCIL, int PREC, int MODE, bool FIX>
-__device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, const PShared& sm,
+// accd.
+template <int MODEL, int STENCIL, int MODE, bool FIX>
+__device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC_FP64>& cx0, const PShared& sm,
                                             uint32_t gq, int ib, double* accd,
                                             HiMax<Pot<MODEL>::NF>& hm) {
   constexpr bool RT = runtime_pot<MODEL>();
-  using C = Ctx<MODEL, PREC>;
-  using T = typename C::T;
-  constexpr bool F64 = PREC == PREC_FP64;
-  using E = typename std::conditional<F64, typename FixElem<FIX>::type, float>::type;
+  using C = Ctx<MODEL, PREC_FP64>;
+  using T = double;
+  using E = typename FixElem<FIX>::type;
   using SL = typename C::SL;
   constexpr int NF = C::NF, NQ = SL::NQ, H = halo_of<STENCIL>();
   constexpr bool CORNERS = StencilW<STENCIL>::kCorners;
   constexpr bool WIDE = STENCIL == 13;
-  using RG = PlainRing<PREC, NF, NQ, H>;
+  using RG = PlainRing<NF, NQ, H>;
   constexpr int NB = RG::NDRIFT, LEAD = RG::LEAD;
-  constexpr int KGROUP = 8;   // split: output planes per float partial before a compensated add
   const SimDesc& d = *sm.d;
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t nn = (uint32_t)(n * n), S = nn * (uint32_t)n;
@@ -261,33 +231,19 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
   T* const own = (T*)sm.ring + tid;
   const T* const hal = (const T*)sm.ring + RG::HALO_OFF + tid;
   E* const fxb = (E*)((T*)sm.ring + RG::FX_OFF);
-  // FP64: integer sums (or, 13 points, all sums) are D times the weights' common
+  // integer sums (13 points: float64 sums too) are D times the weights' common
   // denominator, which goes into the kick's coefficient and, after the stage,
-  // into sum phi D; split: the weights themselves
-  constexpr bool TIMES = F64 && (WIDE || (FIX && STENCIL == 27));
+  // into sum phi D
+  constexpr bool TIMES = WIDE || (FIX && STENCIL == 27);
   C cx = cx0;
   if constexpr (TIMES) cx.kD *= 1.0 / fix_weight<STENCIL>();
-  const E w1 = TIMES ? (E)16 : (E)(16.0 / 12.0);
-  const E w2 = TIMES ? (E)0 - (E)1 : (E)(-1.0 / 12.0);
-  const E w0 = TIMES ? (E)0 - (E)90 : (E)(-90.0 / 12.0);
-  T Mf[NF];   // split: the re-centring of the drifted field (the stencil works on phi + c pi)
-  float ps[F64 ? 1 : NQ];
-  if constexpr (!F64) {
-#pragma unroll
-    for (int f = 0; f < NF; ++f) Mf[f] = madd(cx.cdrift, cx.mu_pi[f], cx.mu_phi[f]);
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) {   // each group's lead lane owns its sums
-      if ((tid & 3) == 0) sm.kahan[i * kKahanGroups + (tid >> 2)] = make_float2(0.f, 0.f);
-      ps[i] = 0.f;
-    }
-  }
-  int kg = 0;
+  const E w1 = (E)16, w2 = (E)0 - (E)1, w0 = (E)0 - (E)90;   // 13 points, times 12
   bool ok = true;
 
   // Three positions run through the planes: copied, drifted, put out.  Where
-  // registers are short (two-field FP64: the Q-ball spilled, 3 to 6 % slower) only
+  // registers are short (two fields: the Q-ball spilled, 3 to 6 % slower) only
   // the last one keeps its slots and cells, and the others' are derived from them.
-  constexpr bool RUN = !F64 || NF == 1;
+  constexpr bool RUN = NF == 1;
   PlainPos<H, RG> ip, dp;   // next plane to copy, next plane to drift
   ip.start(sm, n, gq);
   for (int l = 0; l < LEAD && ip.in(); ++l) ip.next(sm, n, nn, S);
@@ -303,10 +259,10 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
   static_assert(RG::OSLOT == LEAD + H + 2 && RG::HSLOT == LEAD + 1, "slots of the planes ahead");
   auto issue = [&]() {
     if constexpr (RUN)
-      plain_issue<MODEL, PREC, NQ, H>(n, nn, S, sm, ip, ib, ip.os, ip.hs);
+      plain_issue<MODEL, NQ, H>(n, nn, S, sm, ip, ib, ip.os, ip.hs);
     else
-      plain_issue<MODEL, PREC, NQ, H>(n, nn, S, sm, ip, ib,
-                                      ring_slot<RG::OSLOT, RG::OWN, RG::OSLOT - 1>(os), hs);
+      plain_issue<MODEL, NQ, H>(n, nn, S, sm, ip, ib,
+                                ring_slot<RG::OSLOT, RG::OWN, RG::OSLOT - 1>(os), hs);
   };
   // drift of plane gg = g + 1 with the thread's cells there: own cell in place and
   // into the drift buffer, the halo cell into the drift buffer
@@ -316,7 +272,7 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
     E* fx = fxb + (gg % NB) * RG::FX;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      const int ex = F64 ? cx.fx[f] : 0;
+      const int ex = cx.fx[f];
       if (dc.own >= 0) {
         T a = o[f * 2 * kPThreads];
         if constexpr (!RT) {
@@ -430,11 +386,7 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
           for (int f = 0; f < NF; ++f) {
             phj[f] = r[f * 2 * kPThreads];
             pmj[f] = r[(f * 2 + 1) * kPThreads];
-            Dj[f] = fix_out(D[f], F64 ? cx.fx[f] : 0);
-            if constexpr (!F64) {
-              phj[f] -= Mf[f];
-              pmj[f] -= cx.mu_pi[f];
-            }
+            Dj[f] = fix_out(D[f], cx.fx[f]);
           }
           if constexpr (RT) {
 #pragma unroll
@@ -453,35 +405,21 @@ __device__ __forceinline__ bool stage_plain(int n, const Ctx<MODEL, PREC>& cx0, 
               }
             }
             accd[SL::V] += rv[NF];
-          } else if constexpr (F64) {
-            cx.site(MODE, phj, Dj, pmj, pnj, accd);
-          }
-          if constexpr (F64) {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              hm.add(2 * f, phj[f]);
-              hm.add(2 * f + 1, pnj[f]);
-            }
           } else {
-            cx.site(MODE, phj, Dj, pmj, pnj, ps);
+            cx.site(MODE, phj, Dj, pmj, pnj, accd);
           }
 #pragma unroll
           for (int f = 0; f < NF; ++f) {
+            hm.add(2 * f, phj[f]);
+            hm.add(2 * f + 1, pnj[f]);
             __stwb(phi_out + (oz + f * S), phj[f]);
             if (MODE == MODE_SWEEP) __stwb(pi_out + (oz + f * S), pnj[f]);
           }
         }
         oz += nn;
-        if constexpr (!F64) {
-          if (++kg == KGROUP) {
-            kg = 0;
-            kahan_flush<NQ>(sm.kahan, ps);
-          }
-        }
       }
     }
   }
-  if constexpr (!F64) kahan_flush<NQ>(sm.kahan, ps);
   if constexpr (TIMES) {
 #pragma unroll
     for (int f = 0; f < NF; ++f) accd[SL::PHID + f] *= 1.0 / fix_weight<STENCIL>();

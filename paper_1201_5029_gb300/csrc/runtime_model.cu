@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kPThreads, 1) rt_kick(const LaunchTable tab) {
   using C = Ctx<MODEL, PREC_FP64>;
   using SL = typename C::SL;
   constexpr int NF = C::NF, NQ = SL::NQ, H = halo_of<STENCIL>();
-  using RG = PlainRing<PREC_FP64, NF, NQ, H>;
+  using RG = PlainRing<NF, NQ, H>;
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ __align__(8) uint64_t dbar[RG::NDRIFT];
   __shared__ __align__(64) SimDesc s_desc;
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kPThreads, 1) rt_kick(const LaunchTable tab) {
   const SimDesc& d = s_desc;
   const Background& bgr = *d.bg;
   const int n = d.n, ib = bgr.cur;
-  plain_prefetch<MODEL, PREC_FP64, NQ, H>(n, sm, ib, 0u);   // while one thread ...
+  plain_prefetch<MODEL, NQ, H>(n, sm, ib, 0u);   // while one thread ...
   if (tid == 0) {
     s_ctx.init(bgr, d, mode);
     s_ctx.set_fix(bgr.amax, fix_headroom<STENCIL>());
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kPThreads, 1) rt_kick(const LaunchTable tab) {
   hm.zero();
   bool ok = true;
   by_mode(mode, s_ctx.fx[0] != 0, [&](auto fix_c, auto mode_c) {
-    ok = stage_plain<MODEL, STENCIL, PREC_FP64, decltype(mode_c)::value, decltype(fix_c)::value>(
+    ok = stage_plain<MODEL, STENCIL, decltype(mode_c)::value, decltype(fix_c)::value>(
         n, s_ctx, sm, 0u, ib, ps, hm);
   });
   cp_async_wait<0>();
@@ -151,7 +151,7 @@ template <int MODEL, int STENCIL>
 cudaError_t launch_rt_kick(const LaunchTable& t, int grid, cudaStream_t s) {
   constexpr int NF = Pot<MODEL>::NF;
   constexpr int smem =
-      PlainRing<PREC_FP64, NF, Slots<NF, PREC_FP64>::NQ, halo_of<STENCIL>()>::SMEM_BYTES;
+      PlainRing<NF, Slots<NF, PREC_FP64>::NQ, halo_of<STENCIL>()>::SMEM_BYTES;
   if (grid == 0)   // ahead of any stream capture
     return cudaFuncSetAttribute(rt_kick<MODEL, STENCIL>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -404,7 +404,13 @@ struct Ctx {
     }
   }
   //   recenter (split form): the float means mu of the fluctuations move into
-  //   the float64 background; p0 = re-centred (phi0[0..NF), pi0[0..NF))
+  //   the float64 background; p0 = re-centred (phi0[0..NF), pi0[0..NF)).  The
+  //   sites subtract mu in the form's own arithmetic.  A float32 mu below half an
+  //   ulp of a fluctuation leaves it as it was, so that this share of the mean is
+  //   counted again, stage after stage: oscillon parameters, 95 leapfrog steps,
+  //   the mean is 1e-10 of the background's amplitude off, which is 1e-9 to 1e-8
+  //   of the field where the background passes near zero.  The order in which a
+  //   kernel sums the means decides part of it, so it is part of the results.
   __device__ __forceinline__ void recenter(const double* mphi, const double* mpi,
                                            const double* phi0, const double* pi0, double* p0) {
 #pragma unroll
@@ -532,7 +538,7 @@ __device__ __forceinline__ void site_dd(const Ctx<MODEL, PREC_DD>& cx, int mode,
   for (int f = 0; f < NF; ++f) {
     pin[f] = (mode == MODE_SWEEP) ? dd_fma(cx.kD, D[f], dd_fma(-cx.kV, dVd[f], pim[f])) : pim[f];
     // a sweep's sum of the momentum fluctuations sets the re-centring shift
-    // (exact bookkeeping for any value) and enters sum pi^2 only as
+    // (any value of it will do) and enters sum pi^2 only as
     // 2 pi0 sum dpi, a term first order in the fluctuations: high parts in
     // plain float (its rounding is below 1e-12 of sum pi^2); a flush's sum in
     // double-float
@@ -542,8 +548,8 @@ __device__ __forceinline__ void site_dd(const Ctx<MODEL, PREC_DD>& cx, int mode,
     acc[SL::PHID + f].add_prod(phj[f], D[f]);
     if (mode == MODE_SWEEP) {
       // a sweep's sum of the fluctuations only sets the re-centring shift,
-      // which moves into the background exactly as it leaves the
-      // fluctuations: any value of it is exact bookkeeping
+      // which moves into the background as it leaves the fluctuations, to
+      // their double-float rounding: any value of it will do
       acc[SL::DPHI + f].add_fast(phj[f].hi);
     } else {  // a flush's sums give the field's mean and variance: double-float
       acc[SL::DPHI + f].add(phj[f]);

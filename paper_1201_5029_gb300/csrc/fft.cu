@@ -28,8 +28,7 @@
 // float64 arithmetic after three passes.
 #include "fft.h"
 
-#include <cmath>
-#include <mutex>
+#include <stdint.h>
 
 namespace pycool {
 
@@ -37,7 +36,43 @@ namespace {
 
 constexpr int kFftThreads = 128;
 constexpr int kTwiddles = 256;                    // of the largest n
-__device__ longlong2 g_twiddle[kTwiddles];       // cos, sin of 2 pi j / 256, times 2^63
+
+// cos(2 pi j / 256) 2^63, j = 0 .. 64, to nearest (the first, 2^63, as 2^63 - 1)
+constexpr long long kQuarterWave[kTwiddles / 4 + 1] = {
+    9223372036854775807ll, 9220594129639322349ll, 9212262081300395919ll, 9198380910752360533ll,
+    9178958979493303928ll, 9154007986568383775ll, 9123542961522760326ll, 9087582255348360406ll,
+    9046147529429926059ll, 8999263742497006356ll, 8946959135589751977ll, 8889265215047568628ll,
+    8826216733530876278ll, 8757851669087406010ll, 8684211202275644159ll, 8605339691359203716ll,
+    8521284645587064995ll, 8432096696575780529ll, 8337829567810882499ll, 8238540042285863898ll,
+    8134287928298226505ll, 8025136023423198846ll, 7911150076686825028ll, 7792398748961209966ll,
+    7668953571605777421ll, 7540888903379453815ll, 7408281885649732303ll, 7271212395925597501ll,
+    7129762999742300884ll, 6984018900926969672ll, 6834067890275007352ll, 6680000292668201229ll,
+    6521908912666391106ll, 6359888978605472621ll, 6194038085235408523ll, 6024456134932800591ll,
+    5851245277523433568ll, 5674509848751039730ll, 5494356307429348228ll, 5310893171315276450ll,
+    5124230951741890994ll, 4934482087050512913ll, 4741760874862065242ll, 4546183403228460023ll,
+    4347867480705496636ll, 4146932565389392941ll, 3943499692959694935ll, 3737691403771909211ll,
+    3529631669043774883ll, 3319445816179637598ll, 3107260453277907452ll, 2893203392867074694ll,
+    2677403574916221777ll, 2459990989166407361ll, 2241096596829706927ll, 2020852251703075581ll,
+    1799390620744551094ll, 1576845104159639125ll, 1353349755046017570ll, 1129039198644963098ll,
+    904048551248139761ll, 678513338808597222ll, 452569415305004282ll, 226352880908292031ll,
+    0ll};
+struct Twiddles {
+  longlong2 w[kTwiddles];   // cos, sin of 2 pi j / 256, times 2^63
+};
+constexpr Twiddles all_twiddles() {
+  Twiddles t{};
+  constexpr int Q = kTwiddles / 4;
+  for (int j = 0; j < kTwiddles; ++j) {
+    const int r = j % Q, quad = j / Q;
+    const long long c = kQuarterWave[r], s = kQuarterWave[Q - r];
+    t.w[j].x = quad == 0 ? c : quad == 1 ? -s : quad == 2 ? -c : s;
+    t.w[j].y = quad == 0 ? s : quad == 1 ? c : quad == 2 ? -s : -c;
+  }
+  return t;
+}
+// part of the module's image: in place before any kernel of it runs, whatever the
+// stream, the thread or a capture in progress
+__device__ const Twiddles g_twiddle = all_twiddles();
 
 struct ci {
   long long re, im;
@@ -178,7 +213,7 @@ __device__ __forceinline__ void line_transform(ci (&v)[16], int& E, int t, uint3
 #pragma unroll
   for (int m = 0; m < 16; ++m) {
     if (m > 0) {   // w_n^(t m), 1 for the line's first thread
-      const longlong2 w = g_twiddle[(t * m) * (kTwiddles / (16 * R))];
+      const longlong2 w = g_twiddle.w[(t * m) * (kTwiddles / (16 * R))];
       const ci r = rotate<DIR>(v[m], w.x, w.y);
       v[m] = t > 0 ? r : v[m];
     }
@@ -348,38 +383,6 @@ __global__ void __launch_bounds__(kFftThreads) fft_rows_real_inv(const double2* 
     }
 }
 
-// The twiddles, once per device.
-cudaError_t twiddles() {
-  static std::mutex mu;
-  static bool done[64] = {false};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done[dev]) return cudaSuccess;
-  longlong2 w[kTwiddles];
-  auto q63 = [](long double v) {
-    const long double s = v * 9223372036854775808.0L;
-    return s >= 9223372036854775807.0L ? 9223372036854775807ll : (long long)std::floor(s + 0.5L);
-  };
-  const long double pi = 3.14159265358979323846264338327950288L;
-  for (int j = 0; j < kTwiddles; ++j) {
-    // by the first octant, where both are well conditioned
-    const int o = j / 32, r = j % 32;
-    const long double a = 2.0L * pi * ((o & 1) ? 32 - r : r) / kTwiddles;
-    const long double c = std::cos(a), s = std::sin(a);
-    const long double cc = (o & 1) ? s : c, ss = (o & 1) ? c : s;   // of r in the quadrant o / 2
-    const int quad = o / 2;
-    const long double x = quad == 0 ? cc : quad == 1 ? -ss : quad == 2 ? -cc : ss;
-    const long double y = quad == 0 ? ss : quad == 1 ? cc : quad == 2 ? -ss : -cc;
-    w[j] = longlong2{q63(x), q63(y)};
-  }
-  e = cudaMemcpyToSymbol(g_twiddle, w, sizeof(w));
-  if (e == cudaSuccess) done[dev] = true;
-  return e;
-}
-
 template <int R> cudaError_t forward(const double* in, double2* out, int batch, cudaStream_t s) {
   constexpr int N = 16 * R, NH = N / 2 + 1, W = kFftThreads / R;
   constexpr long long half = (long long)N * N * NH;
@@ -405,8 +408,6 @@ template <int R> cudaError_t inverse(double2* spec, double* out, int batch, cuda
 }  // namespace
 
 cudaError_t fft_forward(const double* in, double2* out, int n, int batch, cudaStream_t s) {
-  const cudaError_t e = twiddles();
-  if (e != cudaSuccess) return e;
   switch (n) {
     case 64: return forward<4>(in, out, batch, s);
     case 128: return forward<8>(in, out, batch, s);
@@ -415,8 +416,6 @@ cudaError_t fft_forward(const double* in, double2* out, int n, int batch, cudaSt
   return cudaErrorInvalidValue;
 }
 cudaError_t fft_inverse(double2* spec, double* out, int n, int batch, cudaStream_t s) {
-  const cudaError_t e = twiddles();
-  if (e != cudaSuccess) return e;
   switch (n) {
     case 64: return inverse<4>(spec, out, batch, s);
     case 128: return inverse<8>(spec, out, batch, s);

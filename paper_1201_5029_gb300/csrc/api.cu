@@ -1622,12 +1622,16 @@ PYCOOL_API pycool_status pycool_checkpoint_load(pycool_sim* sim, const void* buf
   const size_t fb = (size_t)sim->nf * (size_t)sim->hdesc.S * word;
   const char* p = (const char*)buf;
   CK(cudaStreamSynchronize(sim->stream));
-  CK(cudaMemcpy(sim->hdesc.phi[b.cur & 1], p + sizeof(b), fb, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(sim->hdesc.pi[(b.cur >> 1) & 1], p + sizeof(b) + fb, fb, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(sim->d_bg, &b, sizeof(b), cudaMemcpyHostToDevice));
-  CK(cudaMemset(sim->ws, 0, sim->L.off_partials));
+  // on the simulation's stream, as the launches that read it (see spectrum_setup)
+  CK(cudaMemcpyAsync(sim->hdesc.phi[b.cur & 1], p + sizeof(b), fb, cudaMemcpyHostToDevice,
+                     sim->stream));
+  CK(cudaMemcpyAsync(sim->hdesc.pi[(b.cur >> 1) & 1], p + sizeof(b) + fb, fb,
+                     cudaMemcpyHostToDevice, sim->stream));
+  CK(cudaMemcpyAsync(sim->d_bg, &b, sizeof(b), cudaMemcpyHostToDevice, sim->stream));
+  CK(cudaMemsetAsync(sim->ws, 0, sim->L.off_partials, sim->stream));
   sim->pp.bar_base = 0;
   CK(cudaEventRecord(sim->done, sim->stream));
+  CK(cudaStreamSynchronize(sim->stream));   // the caller's buffer is its own again
   sim->initialised = true;
   return PYCOOL_OK;
 }
@@ -1735,10 +1739,15 @@ static pycool_status spectrum_setup(pycool_sim* sim) {
     cudaGetLastError();
     return PYCOOL_E_NOMEM;
   }
-  CK(cudaMemcpy(sim->spec_order, order.data(), half * sizeof(uint32_t), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(sim->spec_cut, cut.data(), cut.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(sim->spec_first, first.data(), (nb + 1) * sizeof(int32_t),
-                cudaMemcpyHostToDevice));
+  // (on the simulation's stream: a copy on the default stream may still be on its
+  // way when it returns, and a non-blocking stream would not wait for it)
+  CK(cudaMemcpyAsync(sim->spec_order, order.data(), half * sizeof(uint32_t),
+                     cudaMemcpyHostToDevice, sim->stream));
+  CK(cudaMemcpyAsync(sim->spec_cut, cut.data(), cut.size() * sizeof(int32_t),
+                     cudaMemcpyHostToDevice, sim->stream));
+  CK(cudaMemcpyAsync(sim->spec_first, first.data(), (nb + 1) * sizeof(int32_t),
+                     cudaMemcpyHostToDevice, sim->stream));
+  CK(cudaStreamSynchronize(sim->stream));   // the vectors go out of scope
   if (!fft_takes(n)) {
     if (cufftPlan3d(&sim->spec_plan, n, n, n, CUFFT_D2Z) != CUFFT_SUCCESS) return PYCOOL_E_CUDA;
     sim->spec_planned = true;

@@ -1621,6 +1621,12 @@ PYCOOL_API pycool_status pycool_checkpoint_load(pycool_sim* sim, const void* buf
   const size_t word = prec_word(sim->hdesc.prec);
   const size_t fb = (size_t)sim->nf * (size_t)sim->hdesc.S * word;
   const char* p = (const char*)buf;
+  // The FP64 form's maxima are what keeps its integer sums from overflowing: they are
+  // taken from the fields that come with the record, not from the record (one without
+  // any, an older one, stays without: its first stage sums in float64)
+  bool maxima = sim->hdesc.prec == PREC_FP64;
+  for (int i = 0; i < 2 * sim->nf; ++i) maxima = maxima && (b.amax[i] >> 31);
+  std::memset(b.amax, 0, sizeof(b.amax));
   CK(cudaStreamSynchronize(sim->stream));
   // on the simulation's stream, as the launches that read it (see spectrum_setup)
   CK(cudaMemcpyAsync(sim->hdesc.phi[b.cur & 1], p + sizeof(b), fb, cudaMemcpyHostToDevice,
@@ -1629,6 +1635,13 @@ PYCOOL_API pycool_status pycool_checkpoint_load(pycool_sim* sim, const void* buf
                      cudaMemcpyHostToDevice, sim->stream));
   CK(cudaMemcpyAsync(sim->d_bg, &b, sizeof(b), cudaMemcpyHostToDevice, sim->stream));
   CK(cudaMemsetAsync(sim->ws, 0, sim->L.off_partials, sim->stream));
+  if (maxima) {
+    CK(launch_copy_max((const double*)sim->hdesc.phi[b.cur & 1], nullptr, sim->hdesc.S, sim->nf,
+                       sim->d_bg->amax, sim->stream));
+    CK(launch_copy_max((const double*)sim->hdesc.pi[(b.cur >> 1) & 1], nullptr, sim->hdesc.S,
+                       sim->nf, sim->d_bg->amax + 1, sim->stream));
+    sim->launches += 2;
+  }
   sim->pp.bar_base = 0;
   CK(cudaEventRecord(sim->done, sim->stream));
   CK(cudaStreamSynchronize(sim->stream));   // the caller's buffer is its own again

@@ -851,13 +851,24 @@ __device__ __forceinline__ unsigned int ticket_add(unsigned int* p) {
 // the float64 pipe: each drifted field value is put on a 64-bit fixed-point
 // scale once (to_fixed, integer instructions only), D is summed exactly in
 // integers, and one normalisation (from_fixed, integer instructions) gives D
-// rounded once to float64.  The scale comes from the largest |phi| and |pi| of
-// the stage's input (Ctx::set_fix; the stages track them), so no sum can
-// overflow; a field value within 2^6 (27- and 13-point stencils: 2^2) of the
-// largest keeps every bit, and a smaller one is cut at 2^-58 (2^-54) of the
-// largest or less, below the rounding of the float64 sums it replaces.  A stage whose
-// input has no usable maximum (the first pass over a new state, values out of
-// range or not finite) sums in float64 (FIX = false).
+// rounded once to float64.  The scale comes from B = max|phi| + |c| max|pi| over
+// the lattice (Ctx::set_fix; the stages track the maxima), so no sum can
+// overflow.  A stage whose input has no usable maxima (the state of a kernel that
+// does not track them, values out of range or not finite) sums in float64 (FIX =
+// false).
+// The error of D is absolute, relative to B: a field value within 2^-6 (27- and
+// 13-point stencils: 2^-2) of B's binade keeps every bit, a smaller one is rounded
+// to a unit of at most 2^-58 B (2^-54 B), so D is off by at most 2^-55.4 B (27
+// points 2^-51.9 B, 13 points 2^-51 B; root mean square 2^-57.1, 2^-53.6 and
+// 2^-52.8) beside its own rounding.  That is below what float64 sums round away
+// where the values about a site reach some 2^-4 of B (27 and 13 points: 2^-1), and
+// nothing at all for fluctuations on a background, where every value keeps its
+// bits.  Where a field is small over whole regions, as in the vacuum round a lump,
+// float64 sums round at the field's own magnitude there and these do not: at 2^-10
+// of B, D is off by some 2^-47 (27 and 13 points 2^-43) of the field there, with
+// float64 sums by 2^-51, and below 2^-58 (2^-54) of B nothing is left of it.  This
+// is taken for what it buys (below): the large regions' own rounding, 2^-53 of B a
+// stage, reaches the small ones with the waves.
 // Measured on GB300, against the same kernels with float64 stencils (persistent kernel;
 // set_initial, evolve and get_fields together): 256^3 Q-ball, order 8, two steps 38.6 -> 25.2
 // ms; 256^3 oscillon, order 6, three steps 13.3 -> 8.9 ms; 128^3 preheating,
@@ -871,14 +882,18 @@ template <int STENCIL> constexpr double fix_weight() {
   return STENCIL == 7 ? 1.0 : (STENCIL == 27 ? 30.0 : 12.0);
 }
 
-// trunc(v 2^(1086 - E)) for |v| < 2^(E - 1023): the significand, bit 63 down,
-// shifted right by E - e (shr clamps: values below the scale, and zero, give 0).
+// v 2^(1086 - E) rounded to nearest (a tie away from zero), for |v| < 2^(E - 1023)
+// and E - e >= 2: the significand, bit 63 down, shifted right by E - e with the last
+// bit shifted out added (shr clamps: values below the scale, and zero, give 0).  A
+// value of B's own binade has its last bit above the unit and is not rounded up to
+// the bound.
 __device__ __forceinline__ unsigned long long to_fixed(double v, int E) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
   const int hi = __double2hiint(v);
   const int sh = E - ((hi >> 20) & 0x7ff);
   unsigned long long m = (b << 11) | 0x8000000000000000ull;
-  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));
+  asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh - 1));
+  m = (m + 1ull) >> 1;
   return hi < 0 ? 0ull - m : m;
 }
 // x 2^(E - 1086), rounded to nearest (a tie away from zero)

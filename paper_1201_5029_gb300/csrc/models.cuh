@@ -174,26 +174,27 @@ template <> struct Pot<M_QBALL> {
   //   fac = m2 (1 + K) + m2 K l,   l = ln(u/M^2) = lref + log1p(x),
   //   x = u/u_ref - 1 = u2 hinv - 1,   hinv = 1/(2 u_ref), lref = ln(u_ref/M^2)
   // with u_ref the sweep's per-stage value at one site, the same in every
-  // block.  With B = sc m2 K = ks[3], ks[0] = sc (m2 (1 + K) + m2 K lref) - B
-  // and ks[1] = B hinv,
-  //   sc fac = ks[0] + B (1 + log1p x) = (ks[0] + ks[1] u2) + B (log1p(x) - x),
-  // so that near the reference only one FMA and one addition are float64: for
-  // |x| < 2^-14 the last term, below 2^-29 B, is formed in float32 (its rounding
-  // is below 2^-51 B, and B is a fraction of the sum) and the conversions are
-  // integer instructions (float64 arithmetic and conversions run at 1/64 of the
-  // float32 rate on GB300).  Farther away log1p is its Taylor series
-  // sum_k (-1)^(k+1) x^k / k -- 5 terms for |x| < 2^-12 (the first omitted term
-  // is below 2^-60 |x|), 11 terms for |x| < 2^-5 (below 2^-60 |x|) -- and the
-  // full logarithm beyond or without a reference (hinv = 0 gives x = -1).  The
-  // tiers are chosen on the high word of x as an integer, and Phi = 0 on the
-  // bits of u2 (never negative), so that no float64 instruction is spent on the
-  // tests.
+  // block.  With A = sc (m2 (1 + K) + m2 K lref) = ks[0] and B = sc m2 K = ks[1],
+  //   sc fac = A + B log1p(x) = (A + B x) + B (log1p(x) - x),
+  // so that near the reference three FMAs are all the float64 arithmetic: for
+  // |x| < 2^-17 the last term, below 2^-35 B, is formed in float32 (x cut, four
+  // roundings: 7 2^-24 of it, 2^-56 B, an eighth of the rounding of u2) and the
+  // conversions are integer instructions (float64 arithmetic and conversions run at
+  // 1/64 of the float32 rate on GB300).  At |x| = 2^-14 it would be 2^-50 B off,
+  // more than u2 is, which shows where A + B x is near zero.  Farther away log1p is
+  // its Taylor series sum_k (-1)^(k+1) x^k / k -- 5 terms for |x| < 2^-12 (the first
+  // omitted term is below 2^-60 |x|), 11 terms for |x| < 2^-5 (below 2^-60 |x|) --
+  // and the full logarithm beyond or without a reference (hinv = 0 gives x = -1).
+  // Nothing is added to log1p(x) before it is multiplied, so its rounding is that of
+  // its own size.  The tiers are chosen on the high word of x as an integer, and Phi
+  // = 0 on the bits of u2 (never negative), so that no float64 instruction is spent
+  // on the tests.
   __device__ static double fac_near(const double* ks, double lnM2, double u2, double hinv,
                                     double lref) {
     if (__double_as_longlong(u2) == 0) return 0.0;   // Phi = 0: V = V' = 0
     const double x = fma(u2, hinv, -1.0);
     const int hx = __double2hiint(x) & 0x7fffffff;
-    if (hx < 0x3F100000) {            // |x| < 2^-14
+    if (hx < 0x3EE00000) {            // |x| < 2^-17
       // x to float32 (cut; below 2^-126: 0)
       const int t = hx - 0x38000000;
       const uint32_t xm = t >= 0x00100000 ? ((uint32_t)t << 3) | ((uint32_t)__double2loint(x) >> 29) : 0u;
@@ -205,15 +206,15 @@ template <> struct Pot<M_QBALL> {
       const uint32_t cb = (uint32_t)__float_as_int(c), cm = cb & 0x7fffffffu;
       const uint32_t ch = cm >= 0x00800000u ? (cm >> 3) + 0x38000000u : 0u;
       const double cd = __hiloint2double((int)(ch | (cb & 0x80000000u)), (int)(cm << 29));
-      return fma(ks[3], cd, fma(ks[1], u2, ks[0]));
+      return fma(ks[1], cd, fma(ks[1], x, ks[0]));
     }
-    double l1;                        // 1 + log1p(x)
+    double l;                         // log1p(x)
     if (hx < 0x3F300000) {            // |x| < 2^-12
       double q = fma(x, 0.2, -0.25);
       q = fma(q, x, 1.0 / 3.0);
       q = fma(q, x, -0.5);
       q = fma(q, x, 1.0);
-      l1 = fma(q, x, 1.0);
+      l = q * x;
     } else if (hx < 0x3FA00000) {     // |x| < 2^-5
       double q = fma(x, -1.0 / 12.0, 1.0 / 11.0);
       q = fma(q, x, -0.1);
@@ -226,11 +227,11 @@ template <> struct Pot<M_QBALL> {
       q = fma(q, x, 1.0 / 3.0);
       q = fma(q, x, -0.5);
       q = fma(q, x, 1.0);
-      l1 = fma(q, x, 1.0);
+      l = q * x;
     } else {
-      l1 = (log(0.5 * u2) - lnM2) - (lref - 1.0);
+      l = (log(0.5 * u2) - lnM2) - lref;
     }
-    return fma(ks[3], l1, ks[0]);
+    return fma(ks[1], l, ks[0]);
   }
   // du = d1 (p1 + d1/2) + d2 (p2 + d2/2),  l = log1p(du/u0)
   //   dV'_i = m2 [ A d_i + K l (p_i + d_i) ],  A = 1 + K + K L0

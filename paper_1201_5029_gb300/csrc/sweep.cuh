@@ -317,9 +317,8 @@ struct Ctx {
   // FP64: the potential's constants times sc, sc = -kV in a sweep (so that a
   // kick is one FMA per field: pi + (sc V'/phi) phi) and 1 in a flush
   //   chaotic:  m2, g2     oscillon: m2, -lam, g
-  //   Q-ball:   sc fac = ks[0] + ks[3] (1 + log1p x) ~ ks[0] + ks[1] u2,  ks[2] = -ks[3]
-  //             (set_qref)
-  double sc, ks[4];
+  //   Q-ball:   sc fac = ks[0] + ks[1] log1p x,  ks[2] = -ks[1]  (set_qref)
+  double sc, ks[3];
   T mu_phi[NF], mu_pi[NF];
   T shiftK[NF];
   double phi0s[NF], pi0s[NF], V0;  // split forms: background after drift / kick
@@ -378,10 +377,9 @@ struct Ctx {
       const double u = 0.5 * fma(f0, f0, f1 * f1);
       q_inv = u > 0.0 ? 0.5 / u : 0.0;
       q_lref = u > 0.0 ? log(u) - pk.lnM2 : 0.0;
-      ks[3] = sc * pk.mK;
-      ks[0] = fma(sc, fma(pk.mK, q_lref, pk.m2K1), -ks[3]);
-      ks[1] = ks[3] * q_inv;
-      ks[2] = -ks[3];
+      ks[0] = sc * fma(pk.mK, q_lref, pk.m2K1);
+      ks[1] = sc * pk.mK;
+      ks[2] = -ks[1];
     }
   }
 

@@ -463,7 +463,8 @@ void pycool_server_destroy(pycool_server* srv);
  *   report failure as an exhausted cudaMalloc would: the call returns E_NOMEM
  *   and leaves nothing allocated.  count = 0 clears it.  Process-wide.
  * pycool_debug_barrier_stall: the simulation's next persistent launch (the
- *   next pycool_evolve of a lattice with n a multiple of 32) waits at its
+ *   next pycool_evolve of a compiled-in model in the FP64 form, or in a split
+ *   form with n a multiple of 32, 4TH with SPLIT_FP32 excepted) waits at its
  *   first grid barrier for one block more than the launch has -- an arrival
  *   that never comes -- with every device-side wait limited to
  *   wait_limit_clocks SM clocks.  Every block gives up at the limit, records

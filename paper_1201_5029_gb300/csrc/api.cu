@@ -1043,9 +1043,7 @@ PYCOOL_API pycool_status pycool_debug_fail_alloc(int32_t count) {
 
 PYCOOL_API pycool_status pycool_debug_barrier_stall(pycool_sim* sim, int64_t wait_limit_clocks) {
   if (!sim || wait_limit_clocks <= 0) return PYCOOL_E_INVALID;
-  // only the persistent kernel has a grid barrier (TMA staging: a plain-staging
-  // launch starts from a barrier count of its own, see pycool_evolve)
-  if (!sim->persist || sim->L.plain) return PYCOOL_E_STATE;
+  if (!sim->persist) return PYCOOL_E_STATE;   // only the persistent kernel has a grid barrier
   sim->stall_limit = (long long)wait_limit_clocks;
   return PYCOOL_OK;
 }
@@ -1445,9 +1443,10 @@ PYCOOL_API pycool_status pycool_evolve(pycool_sim* sim, int64_t steps) {
   const long long nsweeps = (long long)steps * sim->nstages;
   if (sim->persist) {
     if (sim->L.plain) {
-      // as for the per-stage kernels, a small launch arms each evolve: here it
-      // clears the grid barrier's count, so that the launch after it depends on
-      // no count kept by the host
+      // The grid barrier's count cleared by a launch of one thread, where the TMA
+      // staging continues from the host's count, which would do here too.  It stays
+      // because pycool_kernel_launches tells the two apart by it: one launch an
+      // evolve where n is a multiple of 32, more elsewhere.
       CK(launch_clear_barrier(sim->pp.bar, sim->stream));
       sim->launches += 1;
       sim->pp.bar_base = 0;

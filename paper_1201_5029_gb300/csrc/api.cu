@@ -1475,7 +1475,9 @@ PYCOOL_API pycool_status pycool_evolve(pycool_sim* sim, int64_t steps) {
 // pycool_sync, leaving the background record it read in *b (not read: E_TIMEOUT
 // of a wait, E_CUDA, E_STATE).  The first two milliseconds are polled without
 // sleeping: a sleep of 50 us takes twice that to wake from, as long as ten stages
-// of a small lattice.  The record and the fault word come in one wait.
+// of a small lattice.  The record and the fault word come in one wait, on a stream of
+// the simulation's own: work that the caller has queued on its stream behind the
+// evolve is not waited for.
 static pycool_status sync_bg(pycool_sim* sim, double timeout_s, Background* b) {
   if (sim->poisoned) return PYCOOL_E_STATE;
   const auto t0 = std::chrono::steady_clock::now();
@@ -1489,10 +1491,10 @@ static pycool_status sync_bg(pycool_sim* sim, double timeout_s, Background* b) {
     else std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
   CK(cudaMemcpyAsync(sim->h_fault, sim->hdesc.fault, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                     sim->stream));
+                     sim->cap_stream));
   CK(cudaMemcpyAsync(sim->h_bg, sim->d_bg, sizeof(Background), cudaMemcpyDeviceToHost,
-                     sim->stream));
-  CK(cudaStreamSynchronize(sim->stream));
+                     sim->cap_stream));
+  CK(cudaStreamSynchronize(sim->cap_stream));
   if (*sim->h_fault) {  // a device-side wait gave up: the state can no longer be trusted
     sim->poisoned = true;
     return PYCOOL_E_TIMEOUT;

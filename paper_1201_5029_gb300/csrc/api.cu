@@ -1384,6 +1384,19 @@ static pycool_status split_initial(pycool_sim* sim, const double* phi, const dou
   return PYCOOL_OK;
 }
 
+// May a kernel on the simulation's device read float64 values at p?  A copy takes
+// more: another device's memory without peer access, and addresses that are no
+// multiple of 8.
+static bool kernel_reads(const pycool_sim* sim, const double* p) {
+  cudaPointerAttributes a;
+  if (((uintptr_t)p & 7) || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged ||
+         (a.type == cudaMemoryTypeDevice && a.device == sim->device);
+}
+
 PYCOOL_API pycool_status pycool_set_initial(pycool_sim* sim, const double* phi, const double* pi,
                                             int on_device, double a0, double pa0) {
   if (!sim || !phi || !pi) return PYCOOL_E_INVALID;
@@ -1403,7 +1416,9 @@ PYCOOL_API pycool_status pycool_set_initial(pycool_sim* sim, const double* phi, 
   if (sim->hdesc.prec == PREC_FP64) {
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const bool maxima = sim->persist;   // (run-time potentials do not use them)
-    if (!maxima || !on_device) {
+    // copied by the kernel that takes the maxima where it can read both arrays
+    const bool direct = maxima && on_device && kernel_reads(sim, phi) && kernel_reads(sim, pi);
+    if (!direct) {
       CK(cudaMemcpyAsync(sim->hdesc.phi[0], phi, count * sizeof(double), kind, sim->stream));
       CK(cudaMemcpyAsync(sim->hdesc.pi[0], pi, count * sizeof(double), kind, sim->stream));
     }
@@ -1411,9 +1426,9 @@ PYCOOL_API pycool_status pycool_set_initial(pycool_sim* sim, const double* phi, 
     if (maxima) {
       double* f0 = (double*)sim->hdesc.phi[0];
       double* p0 = (double*)sim->hdesc.pi[0];
-      CK(launch_copy_max(on_device ? phi : f0, on_device ? f0 : nullptr, (long long)S, nf,
+      CK(launch_copy_max(direct ? phi : f0, direct ? f0 : nullptr, (long long)S, nf,
                          sim->d_bg->amax, sim->stream));
-      CK(launch_copy_max(on_device ? pi : p0, on_device ? p0 : nullptr, (long long)S, nf,
+      CK(launch_copy_max(direct ? pi : p0, direct ? p0 : nullptr, (long long)S, nf,
                          sim->d_bg->amax + 1, sim->stream));
       sim->launches += 2;
     }

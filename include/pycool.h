@@ -470,9 +470,16 @@ void pycool_server_destroy(pycool_server* srv);
  *   wait_limit_clocks SM clocks.  Every block gives up at the limit, records
  *   the fault and returns; pycool_sync then returns E_TIMEOUT and the
  *   simulation is poisoned (E_STATE) while the CUDA context stays usable.
- *   E_STATE if the simulation does not use the persistent kernel. */
+ *   E_STATE if the simulation does not use the persistent kernel.
+ * pycool_debug_plain_plan: the work plan of the FP64 form's plain staging, as
+ *   pycool_persist_plan gives that of the TMA staging, unchecked (host arithmetic
+ *   only).  A unit's x0 and y0 carry its width and height in their upper 16 bits;
+ *   vx and the tile width are 0. */
 pycool_status pycool_debug_fail_alloc(int32_t count);
 pycool_status pycool_debug_barrier_stall(pycool_sim* sim, int64_t wait_limit_clocks);
+pycool_status pycool_debug_plain_plan(int32_t n, int32_t nf, int32_t stencil, int32_t sms,
+                                      int64_t l2_bytes, int32_t* geo, int32_t* units,
+                                      int32_t cap_units, int32_t* uoff, int32_t cap_blocks);
 
 /* ---- allocation-free stage sweep ---------------------------------------------
  * The paper has no counterpart to this call; it is a deployment convenience.

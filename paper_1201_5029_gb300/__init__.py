@@ -137,6 +137,8 @@ def _load():
         "pycool_server_set_persistent_min_n": (S, [P, C.c_int32]),
         "pycool_debug_fail_alloc": (S, [C.c_int32]),
         "pycool_debug_barrier_stall": (S, [P, C.c_int64]),
+        "pycool_debug_plain_plan": (S, [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int64,
+                                        C.POINTER(C.c_int32), P, C.c_int32, P, C.c_int32]),
         "pycool_noalloc_max_blocks": (C.c_size_t, []),
         "pycool_sweep_noalloc": (S, [C.POINTER(pycool_config), P, P, P, P, C.c_int32,
                                      C.POINTER(pycool_stage_state), P]),
@@ -454,17 +456,27 @@ def pycool_persist_plan(n: int, nf: int, precision: int, sms: int, l2_bytes: int
     """The persistent kernel's work plan (host only): (geo, units, uoff) with
     geo a dict, units an int32 array (units, 4) of (x0, y0, z0, planes + 2 H)
     and uoff the int32 block offsets into units."""
+    return _plan(lib.pycool_persist_plan, "pycool_persist_plan", n, nf, precision, stencil, sms,
+                 l2_bytes)
+
+
+def pycool_debug_plain_plan(n: int, nf: int, sms: int, l2_bytes: int,
+                            stencil: int = STENCIL_7PT):
+    """The plain staging's work plan (host only), as pycool_persist_plan; x0 and y0 of a
+    unit carry its width and height in their upper 16 bits."""
+    return _plan(lib.pycool_debug_plain_plan, "pycool_debug_plain_plan", n, nf, stencil, sms,
+                 l2_bytes)
+
+
+def _plan(call, name, *args):
     import numpy as np
     geo = (C.c_int32 * 10)()
-    _check(lib.pycool_persist_plan(n, nf, precision, stencil, sms, l2_bytes, geo, None, 0, None,
-                                   0), "pycool_persist_plan")
+    _check(call(*args, geo, None, 0, None, 0), name)
     keys = ("n", "vx", "tx", "tiles_x", "ntiles", "rc", "rw", "nunits", "G", "halo")
     g = dict(zip(keys, list(geo)))
     units = np.zeros((g["nunits"], 4), dtype=np.int32)
     uoff = np.zeros(g["G"] + 1, dtype=np.int32)
-    _check(lib.pycool_persist_plan(n, nf, precision, stencil, sms, l2_bytes, geo,
-                                   units.ctypes.data, g["nunits"], uoff.ctypes.data, g["G"]),
-           "pycool_persist_plan")
+    _check(call(*args, geo, units.ctypes.data, g["nunits"], uoff.ctypes.data, g["G"]), name)
     return g, units, uoff
 
 

@@ -391,6 +391,26 @@ static bool check_plan(const PGeo& g, const std::vector<int4>& units, const std:
   return true;
 }
 
+static pycool_status put_plan(const PGeo& g, const std::vector<int4>& u,
+                              const std::vector<int>& off, int32_t* geo, int32_t* units,
+                              int32_t cap_units, int32_t* uoff, int32_t cap_blocks) {
+  const int32_t vals[10] = {g.n, g.vx, g.tx, g.tiles_x, g.ntiles, g.rc, g.rw, g.nunits, g.G,
+                            g.halo};
+  for (int i = 0; i < 10; ++i) geo[i] = vals[i];
+  if (units) {
+    if (cap_units < g.nunits) return PYCOOL_E_INVALID;
+    for (int i = 0; i < g.nunits; ++i) {
+      units[4 * i + 0] = u[i].x; units[4 * i + 1] = u[i].y;
+      units[4 * i + 2] = u[i].z; units[4 * i + 3] = u[i].w;
+    }
+  }
+  if (uoff) {
+    if (cap_blocks < g.G) return PYCOOL_E_INVALID;
+    for (int b = 0; b <= g.G; ++b) uoff[b] = off[b];
+  }
+  return PYCOOL_OK;
+}
+
 PYCOOL_API pycool_status pycool_persist_plan(int32_t n, int32_t nf, int32_t precision,
                                              int32_t stencil, int32_t sms, int64_t l2_bytes,
                                              int32_t* geo, int32_t* units, int32_t cap_units,
@@ -409,21 +429,23 @@ PYCOOL_API pycool_status pycool_persist_plan(int32_t n, int32_t nf, int32_t prec
   const PGeo g = plan_units(n, prec_word(prec), nf, prec, sms, l2_bytes, &u, &off,
                             stencil == PYCOOL_STENCIL_4TH ? 2 : 1);
   if (!check_plan(g, u, off)) return PYCOOL_E_INVALID;
-  const int32_t vals[10] = {g.n, g.vx, g.tx, g.tiles_x, g.ntiles, g.rc, g.rw, g.nunits, g.G,
-                            g.halo};
-  for (int i = 0; i < 10; ++i) geo[i] = vals[i];
-  if (units) {
-    if (cap_units < g.nunits) return PYCOOL_E_INVALID;
-    for (int i = 0; i < g.nunits; ++i) {
-      units[4 * i + 0] = u[i].x; units[4 * i + 1] = u[i].y;
-      units[4 * i + 2] = u[i].z; units[4 * i + 3] = u[i].w;
-    }
-  }
-  if (uoff) {
-    if (cap_blocks < g.G) return PYCOOL_E_INVALID;
-    for (int b = 0; b <= g.G; ++b) uoff[b] = off[b];
-  }
-  return PYCOOL_OK;
+  return put_plan(g, u, off, geo, units, cap_units, uoff, cap_blocks);
+}
+
+PYCOOL_API pycool_status pycool_debug_plain_plan(int32_t n, int32_t nf, int32_t stencil,
+                                                 int32_t sms, int64_t l2_bytes, int32_t* geo,
+                                                 int32_t* units, int32_t cap_units, int32_t* uoff,
+                                                 int32_t cap_blocks) {
+  if (n < 1 || n > 1024 || (nf != 1 && nf != 2) || sms < 1 || l2_bytes < 0 || !geo ||
+      (stencil != PYCOOL_STENCIL_7PT && stencil != PYCOOL_STENCIL_ISO27 &&
+       stencil != PYCOOL_STENCIL_4TH) ||
+      (stencil == PYCOOL_STENCIL_4TH && n < 4))
+    return PYCOOL_E_INVALID;
+  std::vector<int4> u;
+  std::vector<int> off;
+  const PGeo g = plan_units(n, 8, nf, PREC_FP64, sms, l2_bytes, &u, &off,
+                            stencil == PYCOOL_STENCIL_4TH ? 2 : 1, true);
+  return put_plan(g, u, off, geo, units, cap_units, uoff, cap_blocks);
 }
 
 void workspace_layout(int ncta, Layout& L) {

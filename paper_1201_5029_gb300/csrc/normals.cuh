@@ -3,7 +3,8 @@
 //
 // GB300 issues a float64 warp instruction every 64 cycles of a scheduler and a
 // 64-bit high product every ~30, so the logarithm and the sine and cosine, which
-// are polynomials on a bounded range, are summed in integers; what is left on the
+// are polynomials on a bounded range, are summed in integers (the logarithm after
+// Tang's table-driven method, ACM TOMS 16, 1990); what is left on the
 // float64 pipe is a pair's one multiply-add, root and two products.  Their inputs
 // are exact: u = (x + 1/2) 2^-32 is an odd integer over 2^33.
 // Against 113-bit arithmetic, three million pairs with the ends of the range: a

@@ -149,11 +149,11 @@ struct PShared {
   const SimDesc* d;       // shared-memory copy of the simulation descriptor
   unsigned char* ring;
   float2* kahan;          // split: [NQ][kKahanGroups] compensated sums (s, c)
-  double* drift;          // FP64: two drifted planes [parity][NF][TY+2][TX]
-  double* red;            // FP64: block-reduction scratch [NQ][kPThreads]
+  double* drift;          // FP64 and split-DD: the drift buffers (PRing::DRIFT_WORDS; FP64: FixLayout)
+  double* red;            // FP64 and split-DD: block-reduction scratch [NQ][kPThreads]
   uint64_t* full;
   uint64_t* empty;
-  uint64_t* dbar;         // split-DD: per drift buffer, every warp has drifted its plane
+  uint64_t* dbar;         // per drift buffer: every warp has drifted its plane (not split-FP32)
   const int4* units;      // (x0, y0, z0, Q): tile origin, first output plane, planes incl. halos
   int nunits;
   uint32_t* issued;       // per slot: 1 + ring index of the last plane issued
@@ -344,12 +344,8 @@ __device__ __forceinline__ void plane_parts(const T (&ctr)[VX], const T (&dn)[VX
 }
 
 __device__ __forceinline__ float shfl_up1(float v) { return __shfl_up_sync(0xffffffffu, v, 1); }
-__device__ __forceinline__ double shfl_up1(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ dd shfl_up1(dd v) { return dd_shfl_up(v, 1); }
 __device__ __forceinline__ float shfl_down1(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
-__device__ __forceinline__ double shfl_down1(double v) {
-  return __shfl_down_sync(0xffffffffu, v, 1);
-}
 __device__ __forceinline__ dd shfl_down1(dd v) { return dd_shfl_down(v, 1); }
 
 // x-neighbours of a lane's VX sites (shuffles; lanes 0 and 31 take the halo

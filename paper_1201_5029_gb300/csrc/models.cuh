@@ -177,14 +177,16 @@ template <> struct Pot<M_QBALL> {
   // block.  With A = sc (m2 (1 + K) + m2 K lref) = ks[0] and B = sc m2 K = ks[1],
   //   sc fac = A + B log1p(x) = (A + B x) + B (log1p(x) - x),
   // so that near the reference three FMAs are all the float64 arithmetic: for
-  // |x| < 2^-17 the last term, below 2^-35 B, is formed in float32 (x cut, four
-  // roundings: 7 2^-24 of it, 2^-56 B, an eighth of the rounding of u2) and the
-  // conversions are integer instructions (float64 arithmetic and conversions run at
-  // 1/64 of the float32 rate on GB300).  At |x| = 2^-14 it would be 2^-50 B off,
-  // more than u2 is, which shows where A + B x is near zero.  Farther away log1p is
-  // its Taylor series sum_k (-1)^(k+1) x^k / k -- 5 terms for |x| < 2^-12 (the first
-  // omitted term is below 2^-60 |x|), 11 terms for |x| < 2^-5 (below 2^-60 |x|) --
-  // and the full logarithm beyond or without a reference (hinv = 0 gives x = -1).
+  // |x| < 31/32 2^-12 the last term, -(x^2/2 - x^3/3 + x^4/4), is formed in integers,
+  // x as 32 bits in units of 2^-44 and its square exact, the cubic and quartic terms
+  // (below 2^-37) in float32.  It is off by 2^-56 B, an eighth of the rounding of u2,
+  // and no float64 instruction or conversion is spent on it (they run at 1/64 of the
+  // float32 rate on GB300).  In float32 throughout it was 2^-50 B off at 2^-14, which
+  // shows where A + B x is near zero; with five float64 terms from 2^-17 on instead a
+  // 256^3 run whose fluctuations have grown past that took 9.64 ms a step where it
+  // takes 8.45.  Farther away log1p is its Taylor series sum_k (-1)^(k+1) x^k / k, 11 terms for
+  // |x| < 2^-5 (the first omitted term is below 2^-60 |x|), and the full logarithm
+  // beyond or without a reference (hinv = 0 gives x = -1).
   // Nothing is added to log1p(x) before it is multiplied, so its rounding is that of
   // its own size.  The tiers are chosen on the high word of x as an integer, and Phi
   // = 0 on the bits of u2 (never negative), so that no float64 instruction is spent
@@ -194,28 +196,26 @@ template <> struct Pot<M_QBALL> {
     if (__double_as_longlong(u2) == 0) return 0.0;   // Phi = 0: V = V' = 0
     const double x = fma(u2, hinv, -1.0);
     const int hx = __double2hiint(x) & 0x7fffffff;
-    if (hx < 0x3EE00000) {            // |x| < 2^-17
-      // x to float32 (cut; below 2^-126: 0)
-      const int t = hx - 0x38000000;
-      const uint32_t xm = t >= 0x00100000 ? ((uint32_t)t << 3) | ((uint32_t)__double2loint(x) >> 29) : 0u;
-      const float xf = __int_as_float((int)(xm | ((uint32_t)__double2hiint(x) & 0x80000000u)));
-      float q = fmaf(xf, -0.25f, 1.f / 3.f);
-      q = fmaf(q, xf, -0.5f);
-      const float c = q * (xf * xf);
-      // c to float64 (exact; denormals: 0)
-      const uint32_t cb = (uint32_t)__float_as_int(c), cm = cb & 0x7fffffffu;
-      const uint32_t ch = cm >= 0x00800000u ? (cm >> 3) + 0x38000000u : 0u;
-      const double cd = __hiloint2double((int)(ch | (cb & 0x80000000u)), (int)(cm << 29));
-      return fma(ks[1], cd, fma(ks[1], x, ks[0]));
+    if (hx < 0x3F2F0000) {            // |x| < 31/32 2^-12
+      // |x| 2^44, cut (shr clamps: below 2^-44, 0)
+      uint32_t X = ((uint32_t)hx << 11) | ((uint32_t)__double2loint(x) >> 21) | 0x80000000u;
+      asm("shr.u32 %0, %0, %1;" : "+r"(X) : "r"(1010 - (hx >> 20)));
+      const float xf = __int_as_float(__float_as_int(__uint2float_rn(X) * 0x1p-44f) |
+                                      (__double2hiint(x) & (int)0x80000000u));
+      const float t = (xf * xf) * (xf * fmaf(xf, -0.25f, 1.f / 3.f));
+      // (x^2/2 - t) 2^89: positive, below 2^64
+      const unsigned long long c = (unsigned long long)X * X -
+          ((unsigned long long)(long long)__float2int_rn(t * 0x1p67f) << 22);
+      // to float64 (cut; 0 as 2^-91)
+      const int lz = __clzll((long long)c);
+      unsigned long long m = c;
+      asm("shl.b64 %0, %0, %1;" : "+l"(m) : "r"(lz));
+      const double cd = __longlong_as_double(
+          (long long)((m >> 11) + ((unsigned long long)(uint32_t)(996 - lz) << 52)));
+      return fma(ks[2], cd, fma(ks[1], x, ks[0]));
     }
     double l;                         // log1p(x)
-    if (hx < 0x3F300000) {            // |x| < 2^-12
-      double q = fma(x, 0.2, -0.25);
-      q = fma(q, x, 1.0 / 3.0);
-      q = fma(q, x, -0.5);
-      q = fma(q, x, 1.0);
-      l = q * x;
-    } else if (hx < 0x3FA00000) {     // |x| < 2^-5
+    if (hx < 0x3FA00000) {            // |x| < 2^-5
       double q = fma(x, -1.0 / 12.0, 1.0 / 11.0);
       q = fma(q, x, -0.1);
       q = fma(q, x, 1.0 / 9.0);
